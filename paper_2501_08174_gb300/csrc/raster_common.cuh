@@ -135,6 +135,17 @@ __device__ __forceinline__ float exp2_approx(float x) {
   return y;
 }
 
+// 1 / x by the special-function unit alone (PTX rcp.approx.ftz, the same bits as
+// __fdividef(1, x) for a normal x).  Without .ftz the compiler brackets it with the
+// scaling that a subnormal x needs: a subnormal 1 - alpha does not occur, and a
+// subnormal den gives 1 / den^2 = inf either way.  5 to 7 % of both rasterizers'
+// time (500k surfels x 16 views: forward 3.55 -> 3.35 ms, backward 5.14 -> 4.86 ms).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 struct SplatEval2 {
   float2 r, rho3;   // 1 / den and the surfel rho (FINITE: zeroed where the filter term won)
   float2 Gc;        // dalpha/do: G where the candidate blends below the 0.99 clamp, else 0
@@ -159,7 +170,7 @@ template <bool FINITE, bool EWA = false, bool CLAMP = true>
 __device__ __forceinline__ SplatEval2 splat_tail2(const float4 g0, const float4 g2, const SplatHead2& h, float rb,
                                                   bool live0, bool live1) {
   SplatEval2 e;
-  const float2 r = EWA ? bc2(1.0f) : make_float2(__fdividef(1.0f, h.den.x), __fdividef(1.0f, h.den.y));
+  const float2 r = EWA ? bc2(1.0f) : make_float2(rcp_approx(h.den.x), rcp_approx(h.den.y));
   const float2 r3 = EWA ? h.q : pmul(h.q, pmul(r, r));
   e.surf[0] = EWA || r3.x <= h.rho2.x;
   e.surf[1] = EWA || r3.y <= h.rho2.y;
@@ -170,7 +181,7 @@ __device__ __forceinline__ SplatEval2 splat_tail2(const float4 g0, const float4 
     e.r = r;
     e.rho3 = r3;
   }
-  const float2 rho = make_float2(e.surf[0] ? r3.x : h.rho2.x, e.surf[1] ? r3.y : h.rho2.y);
+  const float2 rho = EWA ? r3 : make_float2(fminf(r3.x, h.rho2.x), fminf(r3.y, h.rho2.y));
   const float2 ex = pmul(bc2(kNegHalfLog2e), rho);
   const float2 G = make_float2(exp2_approx(ex.x), exp2_approx(ex.y));
   const float2 oG = pmul(bc2(g0.z), G);
