@@ -7,10 +7,8 @@
 // stored between the passes.  Per-Gaussian gradients are summed over the
 // thread's pixels, reduced over the warp, gathered per batch in the warp's
 // shared memory and added to global memory with one vector atomic per 4
-// values, entry and warp.  The warp reduction of the 15 sums of a colour and
-// opacity loss goes through shared memory (each lane writes its sums, then
-// 30 lanes each add 16 of them and pair up with one shuffle); the 20 sums
-// with depth and normal cotangents use a halving transpose of shuffles.
+// values, entry and warp.  The warp reduction goes through shared memory (see
+// warp_totals).
 //
 // Terms that are linear in per-entry or per-column constants are summed before
 // they are multiplied: a thread sums the pixel terms of its column and scales
@@ -46,41 +44,6 @@ __device__ unsigned long long g_diag[8];
 constexpr int kBW = OCGS_BWD_BLOCK_WARPS;
 static_assert(OCGS_BWD_WARPS % kBW == 0 && OCGS_BWD_WARPS_GEO % kBW == 0, "resident warps per CTA");
 
-// One halving step of a warp transpose-reduction: lanes with bit OFF clear keep
-// the first ceil(C/2) of their C values, the others keep the rest, and each
-// adds the partner's copy of what it keeps.  After the steps for OFF = 16..1
-// every lane holds the warp total of one slot: C + C/2 + ... shuffles in all
-// instead of 5 C for independent butterflies.
-template <int C, int OFF>
-__device__ __forceinline__ void halve(float* v, int lane, int& base, int& real) {
-  constexpr int KEEP = (C + 1) / 2;
-  const bool upper = (lane & OFF) != 0;
-#pragma unroll
-  for (int i = 0; i < KEEP; ++i) {
-    const float lo = v[i];
-    const float hi = (KEEP + i < C) ? v[KEEP + i] : 0.f;
-    const float got = __shfl_xor_sync(kFull, upper ? lo : hi, OFF);
-    v[i] = (upper ? hi : lo) + got;
-  }
-  if (upper) {
-    base += KEEP;
-    real -= KEEP;
-  } else if (real > KEEP) {
-    real = KEEP;
-  }
-}
-
-// Warp sum of the 20 sums; returns the one this lane holds (or -1).
-__device__ __forceinline__ int warp_reduce20(float* v, int lane) {
-  int base = 0, real = 20;
-  halve<20, 16>(v, lane, base, real);
-  halve<10, 8>(v, lane, base, real);
-  halve<5, 4>(v, lane, base, real);
-  halve<3, 2>(v, lane, base, real);
-  halve<2, 1>(v, lane, base, real);
-  return real >= 1 ? base : -1;
-}
-
 // Two sums beside the gradient slots, kept in the row's padding until the
 // flush: the totals of the u and v terms, 2 dL/drho (u, v) / den^2, from
 // which the flush forms the centre gradient's share through (u, v, den).
@@ -92,13 +55,46 @@ static_assert(kSumV < kGradStride && kGradSlots <= kSumU, "sums in the row paddi
 constexpr int kRedSums = kGradSlotsRGB + 2;
 __device__ __forceinline__ int red_target(int q) { return q < kGradSlotsRGB ? q : kSumU + (q - kGradSlotsRGB); }
 
-// Row of one lane in the reduction buffer of the 15-sum path: 15 float2 (the
-// two pixel lanes of the packed sums, not yet added).  15 is odd, so the
-// 16-lane phases of the 64-bit stores (lane L writes row L) and of the 64-bit
-// loads (lane L reads sum L & 15 of rows 16 (L >> 4) + i) hit distinct banks.
-constexpr int kRedRow = kRedSums;
-// sum 15 of the last row is read (and ignored) by lanes 15 and 31
-constexpr int kRedSize = 32 * kRedRow + 1;
+// Reduction buffer of a warp: for each of S sums two rows (the values of lanes
+// 0-15 and of lanes 16-31), each 16 floats at a stride of 20.  The upper rows
+// start 16 banks after the lower ones (modulo 32), so a store of one sum by all
+// lanes hits every bank once, and the 16-byte loads, eight consecutive rows per
+// phase, are free of conflicts.
+//
+// What bounds it: shared-memory wavefronts.  The 15 sums of the two pixel lanes
+// stored as pairs and read back with 16 64-bit loads took 62 wavefronts per entry
+// (about 3 ms of a 5.1 ms launch at one wavefront per cycle and SM on 500k
+// surfels x 16 views); added first and read back with four 16-byte loads they
+// take 31, and the launch 4.34 ms against 4.68.  The 20 sums of the depth and
+// normal form took a transpose of 41 shuffles before (64.3 -> 63.3 ms on 1M
+// surfels x 64 views).
+constexpr int kRedStride = 20;
+constexpr int red_upper(int s) { return s * kRedStride + (48 - s * kRedStride % 32) % 32; }
+// one row more than the sums have: the lanes without a sum read past the upper rows
+constexpr int red_floats(int s) { return red_upper(s) + (s + 1) * kRedStride; }
+
+// Stores the S per-lane sums v(q) and returns, in lane L and in lane L ^ 16, the
+// warp total of sum L & 15 (lane 15: undefined for S = 15).  Ends before the
+// reads of other lanes are ordered: the caller synchronises before the next call.
+template <int S, class F>
+__device__ __forceinline__ float warp_totals(float* red, int lane, F v) {
+  float* wr = red + (lane >> 4) * red_upper(S) + (lane & 15);
+#pragma unroll
+  for (int q = 0; q < S; ++q) wr[q * kRedStride] = v(q);
+  __syncwarp();
+  const float4* rd = reinterpret_cast<const float4*>(red + (lane >> 4) * red_upper(S) + (lane & 15) * kRedStride);
+  float4 t = rd[0];
+#pragma unroll
+  for (int i = 1; i < 4; ++i) {
+    const float4 b = rd[i];
+    const float2 lo = padd(make_float2(t.x, t.y), make_float2(b.x, b.y));
+    const float2 hi = padd(make_float2(t.z, t.w), make_float2(b.z, b.w));
+    t = make_float4(lo.x, lo.y, hi.x, hi.y);
+  }
+  const float2 u = padd(make_float2(t.x, t.y), make_float2(t.z, t.w));
+  const float tot = __fadd_rn(u.x, u.y);
+  return __fadd_rn(tot, __shfl_xor_sync(kFull, tot, 16));
+}
 
 // Slots accumulated with the opposite sign (flipped when the lanes are summed).
 __device__ __forceinline__ bool negated_slot(int q) { return q == kGe0 || q == kGe1 || q == kGe2; }
@@ -112,14 +108,13 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
   constexpr int WPT = TW * TH / PPT / 32;  // warps per tile: each owns a band of full tile rows
   constexpr int ROWS = BATCH > 32 ? BATCH / 32 : 1;  // gradient rows of a batch each lane flushes
   using B = Batch<BATCH>;
-  __shared__ float4 s_g0[kBW][BATCH], s_g1[kBW][BATCH], s_g2[kBW][BATCH],
-      s_a0[kBW][BATCH];
-  __shared__ float2 s_a1[kBW][BATCH];
+  __shared__ float4 s_g0[kBW][BATCH], s_g1[kBW][BATCH], s_g2[kBW][BATCH], s_a0[kBW][BATCH];
+  // (n_y, n_z, blend bound, list position); the colour and opacity form, which needs neither
+  // normals nor depths, keeps the last two in the depth fields of g0 and g2
+  __shared__ float4 s_b[kBW][GEO ? BATCH : 1];
   __shared__ uint32_t s_idx[kBW][BATCH];
-  __shared__ int s_q[kBW][BATCH];  // list position of each kept entry
   __shared__ __align__(16) float s_grad[kBW][BATCH * kGradStride];  // per-batch gradient sums of each entry
-  __shared__ float s_rb[kBW][BATCH];
-  __shared__ __align__(16) float2 s_red[kBW][GEO ? 1 : kRedSize];
+  __shared__ __align__(16) float s_red[kBW][red_floats(GEO ? kGradStride : kRedSums)];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
@@ -130,10 +125,9 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
       for (int q = 0; q < kGradStride; ++q) row[q] = 0.f;
     }
   }
-  // the sum this lane adds up in the 15-sum reduction, its sign and its place in the row
-  const int red_slot = lane & 15;
-  const float red_sign = negated_slot(red_slot) ? -1.f : 1.f;
-  const int red_dst = red_target(red_slot);
+  // the sign of the sum this lane holds after the reduction, and (15-sum form) its place in the row
+  const float red_sign = negated_slot(lane & 15) ? -1.f : 1.f;
+  const int red_dst = red_target(lane & 15);
   const uint32_t n_units = a.n_tiles * (uint32_t)WPT;
   for (uint32_t it = 0;; ++it) {
     // work unit: one warp's band of one tile; the warps run independently
@@ -205,6 +199,14 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
     // entries at or beyond the warp's largest last index are idle for every lane
     const int warp_last = (int)__reduce_max_sync(kFull, thread_last);
     const float4 band = warp_band<TW, TH, PPT>(cam, local, (int)(unit % WPT));
+    auto list_at = [&](int q) { return (uint32_t)q < len1 ? a.vals[start + q] : a.vals2[start2 + ((uint32_t)q - len1)]; };
+    const float2 pyb = make_float2((float)py0 + 0.5f, (float)py0 + 1.5f);
+    // the next batch's list entries are requested while the current one is processed
+    uint32_t nidx = 0;
+    if (B::kRounds == 1) {
+      const int q = max(0, warp_last - BATCH) + lane;
+      if (lane < B::kLanes && q < warp_last) nidx = list_at(q);
+    }
     for (int bend = warp_last; bend > 0; bend -= BATCH) {
       const int bstart = max(0, bend - BATCH);
       __syncwarp();  // the previous batch is consumed and flushed
@@ -217,76 +219,86 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
         uint32_t idx = 0;
         float4 a1 = make_float4(0.f, 0.f, 0.f, 0.f);
         if (lane < B::kLanes && q < bend) {
-          idx = (uint32_t)q < len1 ? a.vals[start + q] : a.vals2[start2 + ((uint32_t)q - len1)];
+          idx = B::kRounds == 1 ? nidx : list_at(q);
           a1 = a.rec.a1[idx];
           keep = a1.w >= band.z && a1.z <= band.w;
         }
         const unsigned km = __ballot_sync(kFull, keep);
         if (keep) {
           const int slot = cnt + __popc(km & lt);
-          const float4 g0 = a.rec.g0[idx];
+          float4 g0 = a.rec.g0[idx], g2 = a.rec.g2[idx];
+          const float rb = blend_rho(g0.z);
+          if (GEO) {
+            s_b[wib][slot] = make_float4(a1.x, a1.y, rb, __int_as_float(q));
+          } else {
+            g0.w = rb;
+            g2.w = __int_as_float(q);
+          }
           s_g0[wib][slot] = g0;
           s_g1[wib][slot] = a.rec.g1[idx];
-          s_g2[wib][slot] = a.rec.g2[idx];
+          s_g2[wib][slot] = g2;
           s_a0[wib][slot] = a.rec.a0[idx];
-          s_a1[wib][slot] = make_float2(a1.x, a1.y);
-          s_rb[wib][slot] = blend_rho(g0.z);
           s_idx[wib][slot] = idx;
-          s_q[wib][slot] = q;
         }
         cnt += __popc(km);
       }
+      if (B::kRounds == 1) {
+        const int q = max(0, bstart - BATCH) + lane;
+        if (lane < B::kLanes && q < bstart) nidx = list_at(q);
+      }
       __syncwarp();
       for (int j = cnt - 1; j >= 0; --j) {
-        const int jj = s_q[wib][j];
 #ifdef OCGS_COUNT
         if (lane == 0) OCGS_DIAG(2, 1);
 #endif
         // every entry of the walk lies before warp_last, so some lane has jj < its
         // last index; the support test of all pixels runs as straight-line code
         const float4 g0 = s_g0[wib][j], g1 = s_g1[wib][j], g2 = s_g2[wib][j];
-        const float rb = s_rb[wib][j];
+        const float4 an = GEO ? s_b[wib][j] : make_float4(0.f, 0.f, g0.w, g2.w);
+        const float rb = an.z;
+        const int jj = __float_as_int(an.w);  // list position
         const SplatColumn col = splat_column(g0, g1, g2, pxf);
         SplatHead2 hd[NP];
         bool live[2 * NP];
         bool any = false;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          const float2 py = make_float2((float)(py0 + 2 * p) + 0.5f, (float)(py0 + 2 * p + 1) + 0.5f);
+          const float2 py = padd(pyb, bc2((float)(2 * p)));  // exact: half-integers below 2^15
           hd[p] = splat_head2(g0, g1, g2, col, py);
           live[2 * p] = jj < (int)last[2 * p];
           live[2 * p + 1] = jj < (int)last[2 * p + 1];
-          any = any || may_blend(hd[p], rb, live[2 * p], live[2 * p + 1]);
+          if (!GEO) any = any || may_blend(hd[p], rb, live[2 * p], live[2 * p + 1]);
         }
-        if (!__any_sync(kFull, any)) continue;  // the support misses every pixel of the band
+        // the support misses every pixel of the band (about one entry in seven; the depth and normal
+        // form evaluates those too: the vote's latency costs it more, 56.7 against 57.2 ms on 1M
+        // surfels x 64 views; the colour and opacity form keeps it, 4.34 against 4.37 ms)
+        if (!GEO && !__any_sync(kFull, any)) continue;
 #ifdef OCGS_COUNT
         if (lane == 0) OCGS_DIAG(5, 1);  // entries evaluated in full
 #endif
         const float4 ap = s_a0[wib][j];
-        const float2 an = s_a1[wib][j];
         const float2 no = bc2(-g0.z);  // 2 dalpha/drho = -alpha = -o G
         // this thread's sums (one lane per pixel of a pair): the slots of the
         // record gradient, and the u and v totals in kSumU, kSumV.  The dx-scaled
         // slots (A00, A10, e1, and the filter term of cx) hold their pixel sums
         // until the column offset is applied after the pairs.
+        // The first pair sets each sum, the others add to it.
         float2 acc[kGradStride];
-#pragma unroll
-        for (int q = 0; q < kGradStride; ++q) acc[q] = bc2(0.f);
-        bool contrib = false;
         // no per-pair branch: a candidate that is not blended has alpha = 0 and
         // Gc = 0, which makes its weight and every term of its adjoint exactly 0
         auto pairs = [&](auto clamp) {
           constexpr bool CLAMP = decltype(clamp)::value;
 #pragma unroll
           for (int p = 0; p < NP; ++p) {
+            auto sum_fma = [&](int q, float2 x, float2 y) { acc[q] = p == 0 ? pmul(x, y) : pfma(x, y, acc[q]); };
+            auto sum_add = [&](int q, float2 x) { acc[q] = p == 0 ? x : padd(acc[q], x); };
             const SplatEval2 e = splat_tail2<true, false, CLAMP>(g0, g2, hd[p], rb, live[2 * p], live[2 * p + 1]);
-            contrib = contrib || e.ok[0] || e.ok[1];
 #ifdef OCGS_COUNT
             OCGS_DIAG(6, (e.ok[0] ? 1 : 0) + (e.ok[1] ? 1 : 0));  // (pixel, entry) blends
 #endif
             // undo the entry: T before it, its weight, and dL/dalpha
             const float2 om = pfma(e.alpha, bc2(-1.f), bc2(1.f));  // 1 - alpha
-            const float2 inv = make_float2(__fdividef(1.f, om.x), __fdividef(1.f, om.y));
+            const float2 inv = make_float2(rcp_approx(om.x), rcp_approx(om.y));
             const float2 Ti = pmul(T[p], inv);
             const float2 w = pmul(e.alpha, Ti);
             float2 F = pmul(gC0[p], bc2(ap.x));
@@ -305,18 +317,18 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
             // a skipped candidate has alpha = 0, and the fast reciprocal of 1 - 0 is exactly 1
             // on this GPU (checked at 1, 2 and 0.5), so T passes through it unchanged
             T[p] = Ti;
-            acc[kGr] = pfma(gC0[p], w, acc[kGr]);
-            acc[kGg] = pfma(gC1[p], w, acc[kGg]);
-            acc[kGb] = pfma(gC2[p], w, acc[kGb]);
+            sum_fma(kGr, gC0[p], w);
+            sum_fma(kGg, gC1[p], w);
+            sum_fma(kGb, gC2[p], w);
             if (GEO) {
-              acc[kGnx] = pfma(gN0[p], w, acc[kGnx]);
-              acc[kGny] = pfma(gN1[p], w, acc[kGny]);
-              acc[kGnz] = pfma(gN2[p], w, acc[kGnz]);
+              sum_fma(kGnx, gN0[p], w);
+              sum_fma(kGny, gN1[p], w);
+              sum_fma(kGnz, gN2[p], w);
             }
             // alpha = o G below the clamp: dalpha/do = G, dalpha/drho = -o G / 2
             // (Gc is 0 at the clamp and for skipped candidates); gs2 = 2 dL/drho
             const float2 gop = pmul(ga, e.Gc);
-            acc[kGo] = padd(acc[kGo], gop);
+            sum_add(kGo, gop);
             const float2 gs2 = pmul(gop, no);
             // rho and depth came from the surfel's (u, v) where it won the min, from the
             // screen-space filter elsewhere.  e.r and e.rho3 are 0 where the filter won,
@@ -327,8 +339,8 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
               // d/dz of w (gD z + gQ z^2)
               const float2 gz = pmul(pfma(pmul(bc2(2.f), gQ[p]), e.z, gD[p]), w);
               gzs = make_float2(e.surf[0] ? gz.x : 0.f, e.surf[1] ? gz.y : 0.f);
-              acc[kGzc] = padd(acc[kGzc], pfma(gzs, bc2(-1.f), gz));
-              acc[kGzD] = pfma(gzs, e.r, acc[kGzD]);
+              sum_add(kGzc, pfma(gzs, bc2(-1.f), gz));
+              sum_fma(kGzD, gzs, e.r);
             }
             // 2 grho / den^2, shared by the u, v and den terms (rho3 = q / den^2)
             const float2 t = pmul(gs2, pmul(e.r, e.r));
@@ -338,24 +350,27 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
             // are flipped when the lanes are summed
             const float2 ngden = GEO ? pmul(pfma(gs2, e.rho3, pmul(gzs, e.z)), e.r)
                                      : pmul(t, pmul(hd[p].q, e.r));
-            acc[kSumU] = padd(acc[kSumU], gun);
-            acc[kSumV] = padd(acc[kSumV], gvn);
-            acc[kGA01] = pfma(gun, hd[p].dy, acc[kGA01]);
-            acc[kGA11] = pfma(gvn, hd[p].dy, acc[kGA11]);
-            acc[kGe0] = padd(acc[kGe0], ngden);
-            acc[kGe2] = pfma(ngden, hd[p].dy, acc[kGe2]);
+            sum_add(kSumU, gun);
+            sum_add(kSumV, gvn);
+            sum_fma(kGA01, gun, hd[p].dy);
+            sum_fma(kGA11, gvn, hd[p].dy);
+            sum_add(kGe0, ngden);
+            sum_fma(kGe2, ngden, hd[p].dy);
             // the filter term: d rho2 / d(c) = -4 (x - c) with rho2 = 2 |x - c|^2 (the
             // factor -2 and dx are applied later)
-            acc[kGcx] = padd(acc[kGcx], gf2);
-            acc[kGcy] = pfma(gf2, hd[p].dy, acc[kGcy]);
+            sum_add(kGcx, gf2);
+            sum_fma(kGcy, gf2, hd[p].dy);
           }
         };
-        if (g0.z < kNoClampO) pairs(std::false_type{});
+        // a record that cannot reach the 0.99 clamp takes the clamp-free blend (2 % of the colour
+        // and opacity launch); the depth and normal form is faster without the branch (55.0
+        // against 56.7 ms on 1M surfels x 64 views)
+        if (!GEO && g0.z < kNoClampO) pairs(std::false_type{});
         else pairs(std::true_type{});
-        if (!__any_sync(kFull, contrib)) continue;  // no pixel of the band blends it
+        // nearly every entry that is evaluated blends a pixel, so there is no second vote: the
+        // sums of one that does not are all zero and its flush adds nothing
 #ifdef OCGS_COUNT
         if (lane == 0) OCGS_DIAG(3, 1);
-        OCGS_DIAG(4, contrib ? 1 : 0);
 #endif
         // the column offset of this thread's pixels
         const float2 dx = bc2(col.dx);
@@ -363,33 +378,23 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
         acc[kGA10] = pmul(acc[kSumV], dx);
         acc[kGe1] = pmul(acc[kGe0], dx);
         acc[kGcx] = pmul(acc[kGcx], dx);
+        float* sums = &s_grad[wib][j * kGradStride];
+        auto value = [&](int q) { return __fadd_rn(acc[q].x, acc[q].y); };
         if (GEO) {
-          float gr[kGradStride];
+          const float tot = warp_totals<kGradStride>(s_red[wib], lane, value);
+          // sums 16 to 19: eight lanes each, one 16-byte load per lane
+          const float4 c = *reinterpret_cast<const float4*>(
+              &s_red[wib][((lane >> 2) & 1) * red_upper(kGradStride) + (16 + (lane >> 3)) * kRedStride + 4 * (lane & 3)]);
+          float rest = __fadd_rn(__fadd_rn(c.x, c.y), __fadd_rn(c.z, c.w));
 #pragma unroll
-          for (int q = 0; q < kGradStride; ++q)
-            gr[q] = negated_slot(q) ? -__fadd_rn(acc[q].x, acc[q].y) : __fadd_rn(acc[q].x, acc[q].y);
-          const int slot = warp_reduce20(gr, lane);
-          if (slot >= 0) s_grad[wib][j * kGradStride + slot] = gr[0];  // one lane per slot
+          for (int o = 1; o < 8; o <<= 1) rest = __fadd_rn(rest, __shfl_xor_sync(kFull, rest, o));
+          if (lane < 16) sums[lane] = tot * red_sign;
+          if ((lane & 7) == 0) sums[16 + (lane >> 3)] = rest;
         } else {
-          // through shared memory: lane L's row holds its 15 packed sums; lane L then adds
-          // sum L & 15 over the rows 16 (L >> 4) .. 16 (L >> 4) + 15, both pixel lanes
-          float2* red = s_red[wib];
-#pragma unroll
-          for (int q = 0; q < kRedSums; ++q) red[lane * kRedRow + q] = acc[red_target(q)];
-          __syncwarp();
-          // four independent partial sums keep the dependent chain short
-          const float2* col = red + (lane >> 4) * 16 * kRedRow + red_slot;
-          float2 s4[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) s4[i] = col[i * kRedRow];
-#pragma unroll
-          for (int i = 4; i < 16; ++i) s4[i & 3] = padd(s4[i & 3], col[i * kRedRow]);
-          const float2 sum = padd(padd(s4[0], s4[1]), padd(s4[2], s4[3]));
-          float tot = __fadd_rn(sum.x, sum.y);
-          tot = __fadd_rn(tot, __shfl_xor_sync(kFull, tot, 16));
-          if (lane < kRedSums) s_grad[wib][j * kGradStride + red_dst] = tot * red_sign;
-          __syncwarp();  // the rows are read before the next entry writes them
+          const float tot = warp_totals<kRedSums>(s_red[wib], lane, [&](int q) { return value(red_target(q)); });
+          if (lane < kRedSums) sums[red_dst] = tot * red_sign;
         }
+        __syncwarp();  // the rows are read before the next entry writes them
       }
       // flush the batch: complete the centre gradient, then one vector atomic per
       // 4 slots and entry for the warp
