@@ -10,6 +10,9 @@
 // are sorted per pair instead of tile+depth bits.
 #include "common.cuh"
 
+#include <algorithm>
+#include <type_traits>
+
 namespace ocgs {
 namespace {
 
@@ -122,144 +125,324 @@ cudaError_t scan_exclusive(const T* in, T* out, uint32_t n, T* d_total, char* sc
 }
 
 // ------------------------------------------------------------------ radix sort
-constexpr int kMaxRadix = 256;
+// Stable LSD sort, one kernel per digit (the single-pass scatter with decoupled
+// look-back of Adinets and Merrill, "Onesweep", 2022): a first kernel reads the
+// keys once and counts the digits of every pass; each pass then reads its items
+// once and writes them once.  A block orders its tile by digit in shared memory,
+// publishes its digit counts and adds up those of the tiles before it until one
+// has published its running total.  Tiles are handed out by a counter, so the
+// tiles a block waits for are resident and never wait for a later one; a wait
+// that reaches kSpinLimit polls all the same is given up, and the block counts
+// the digits of all earlier keys itself, so the result never depends on a wait.
+//
+// What bounds it: HBM at full size (16 bytes per item and pass), the launch and
+// the look-back latency below about a million items.
+// 384 threads x 18 items at three blocks per SM (56 registers, 69 KB) was the fastest of
+// 256 to 512 threads x 10 to 24 items: 36 resident warps hide the ranking's shared-memory
+// latency and few tiles keep the look-back short (tile sorts of 500k surfels x 16 views,
+// 28 M pairs: 376 us against 400 to 516 with the others, 584 with a histogram, a scan and
+// a scatter kernel per digit; depth sort of 8 M records: 230 against 390).
+constexpr int kRadixThreads = 384;
+constexpr int kRadixItems = 18;
+constexpr int kRadixBlocks = 3;  // resident per SM
+constexpr int kRadixTile = kRadixThreads * kRadixItems;
+constexpr int kRadixWarps = kRadixThreads / 32;
+#ifndef OCGS_SPIN_LIMIT
+#define OCGS_SPIN_LIMIT (1u << 20)
+#endif
+constexpr uint32_t kSpinLimit = OCGS_SPIN_LIMIT;
+constexpr int kLookBack = 16;  // tiles per round trip of a look-back (4 to 32 measured within 3 %)
 
-// Lanes of the warp whose digit equals this lane's, from one ballot per bit
-// (bits = digit width + 1: the extra bit marks out-of-range items).
-__device__ __forceinline__ unsigned digit_peers(uint32_t d, int bits) {
-  unsigned peers = kFull;
-  for (int b = 0; b < bits; ++b) {
-    const bool set = (d >> b) & 1u;
-    const unsigned bal = __ballot_sync(kFull, set);
-    peers &= set ? bal : ~bal;
-  }
-  return peers;
+// Digits of a sort of n_bits key bits: equal widths of 4 to 8 bits.  (Two digits of 10
+// bits instead of three of 7 took 17.6 against 6.0 ms on 480k tiles: runs of a few items
+// per digit and tile, and four times the look-back words.)
+constexpr int kMinDigit = 4, kMaxDigit = 8;
+struct DigitPlan {
+  int passes, bits;
+};
+DigitPlan digit_plan(int n_bits) {
+  const int passes = (n_bits + kMaxDigit - 1) / kMaxDigit;
+  return DigitPlan{passes, std::max(kMinDigit, (n_bits + passes - 1) / passes)};
 }
 
-__global__ void __launch_bounds__(kBlock) radix_upsweep_kernel(const uint32_t* __restrict__ keys,
-                                                               uint32_t n, int shift, uint32_t mask,
-                                                               uint32_t* __restrict__ counts,
-                                                               uint32_t n_blocks, const uint32_t* __restrict__ d_n) {
-  constexpr int NW = kBlock / 32;
-  __shared__ uint32_t whist[NW][kMaxRadix + 1];
-  if (d_n) n = min(n, *d_n);  // device-side count (capacity launches)
-  const int R = (int)mask + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = lane; i <= R; i += 32) whist[warp][i] = 0;
-  __syncwarp();
-  const uint32_t wbase = blockIdx.x * kChunk + warp * 32 * kItems;
-  uint32_t key[kItems];
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    key[j] = k < n ? keys[k] : 0u;
-  }
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    if (k < n) atomicAdd(&whist[warp][(key[j] >> shift) & mask], 1u);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < R; i += kBlock) {
-    uint32_t t = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) t += whist[w][i];
-    counts[(size_t)i * n_blocks + blockIdx.x] = t;
-  }
-}
-
-// Stable scatter of one pass.  Warp w of the block owns the contiguous slice
-// [w*32*kItems, (w+1)*32*kItems) of the block's chunk and ranks its items in
-// their original order (round j covers the slice's items j*32 .. j*32+31)
-// with a running per-warp count of every digit.  The block then orders its
-// whole chunk by digit in shared memory and writes it out in digit runs, so
-// the global stores are coalesced.
-// vals_in NULL: the values are the items' indices
-__global__ void __launch_bounds__(kBlock) radix_scatter_kernel(const uint32_t* __restrict__ keys_in,
-                                                               const uint32_t* __restrict__ vals_in,
-                                                               uint32_t* __restrict__ keys_out,
-                                                               uint32_t* __restrict__ vals_out,
-                                                               uint32_t n, int shift, uint32_t mask,
-                                                               const uint32_t* __restrict__ offsets,
-                                                               uint32_t n_blocks, const uint32_t* __restrict__ d_n) {
-  constexpr int NW = kBlock / 32;
-  if (d_n) n = min(n, *d_n);  // device-side count (capacity launches)
-  __shared__ uint32_t whist[NW][kMaxRadix + 1];
-  __shared__ uint32_t dstart[kMaxRadix];
-  __shared__ uint32_t gbase[kMaxRadix];
-  __shared__ uint32_t wsum[NW];
-  __shared__ uint32_t sk[kChunk];
-  __shared__ uint32_t sv[kChunk];
-  const int R = (int)mask + 1;
-  const int bits = __popc(mask) + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = lane; i <= R; i += 32) whist[warp][i] = 0;
-  for (int i = threadIdx.x; i < R; i += kBlock) gbase[i] = offsets[(size_t)i * n_blocks + blockIdx.x];
-  __syncwarp();
-  const uint32_t wbase = blockIdx.x * kChunk + warp * 32 * kItems;
-  const unsigned lt = (1u << lane) - 1u;
-  uint32_t key[kItems], val[kItems], rank[kItems];
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    const bool valid = k < n;
-    key[j] = valid ? keys_in[k] : 0u;
-    val[j] = valid ? (vals_in ? vals_in[k] : k) : 0u;  // no values: the item's index
-  }
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    const uint32_t d = k < n ? ((key[j] >> shift) & mask) : (uint32_t)R;
-    const unsigned peers = digit_peers(d, bits);
-    const int leader = __ffs(peers) - 1;
-    uint32_t before = 0;
-    if (lane == leader) before = whist[warp][d];
-    before = __shfl_sync(peers, before, leader);
-    rank[j] = before + __popc(peers & lt);
-    if (lane == leader) whist[warp][d] = before + __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  // per digit: offsets of the warps inside the digit, and the digit's total
-  uint32_t tot = 0;
-  if (threadIdx.x < R) {
-    for (int w = 0; w < NW; ++w) {
-      const uint32_t c = whist[w][threadIdx.x];
-      whist[w][threadIdx.x] = tot;
-      tot += c;
+// Where the keys of a sort come from: an array, or (queue orders) the tiles' pair counts.
+struct ArrayKeys {
+  const uint32_t* keys;
+  __device__ __forceinline__ uint32_t operator()(uint32_t i) const { return keys[i]; }
+};
+struct QueueKeys {
+  const uint2* ranges;
+  const uint2* ranges2;  // optional second segment of each tile's list
+  __device__ __forceinline__ uint32_t operator()(uint32_t i) const {
+    const uint2 r = ranges[i];
+    uint32_t len = r.y - r.x;
+    if (ranges2) {
+      const uint2 q = ranges2[i];
+      len += q.y - q.x;
     }
+    return queue_key(len);
   }
-  // exclusive scan of the digit totals across the block (digit = thread index)
-  uint32_t inc = tot;
+};
+
+// Exclusive scan of kPer values per thread over a block of kRadixThreads; returns
+// this thread's first prefix.  s_w: one word per warp, free to reuse after a barrier.
+template <int PER>
+__device__ __forceinline__ uint32_t block_exclusive(const uint32_t (&v)[PER], uint32_t* s_w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t sum = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, inc, o);
-    if (lane >= o) inc += t;
-  }
-  if (lane == 31) wsum[warp] = inc;
+  for (int k = 0; k < PER; ++k) sum += v[k];
+  const uint32_t inc = warp_inclusive_scan<uint32_t>(sum, lane);
+  if (lane == 31) s_w[warp] = inc;
   __syncthreads();
   uint32_t carry = 0;
-  for (int w = 0; w < warp; ++w) carry += wsum[w];
-  if (threadIdx.x < R) dstart[threadIdx.x] = carry + inc - tot;
-  __syncthreads();
-  const uint32_t n_here = (blockIdx.x * kChunk >= n) ? 0u
-                          : ((n - blockIdx.x * kChunk < (uint32_t)kChunk) ? n - blockIdx.x * kChunk : (uint32_t)kChunk);
 #pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    if (k < n) {
-      const uint32_t d = (key[j] >> shift) & mask;
-      const uint32_t lp = dstart[d] + whist[warp][d] + rank[j];
-      sk[lp] = key[j];
-      sv[lp] = val[j];
+  for (int w = 0; w < kRadixWarps; ++w) carry += w < warp ? s_w[w] : 0u;
+  return carry + inc - sum;
+}
+
+// Counts the digits of every pass (hist [PASSES][1 << BITS], zeroed); the last
+// block to finish turns each pass's counts into first positions.  DROP: keys
+// 0xffffffff are left out of the sort, and *n_valid gets the number of the others.
+template <class Keys, int BITS, int PASSES, bool DROP>
+__global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const Keys keys, uint32_t n,
+                                                                   const uint32_t* __restrict__ d_n, uint32_t* hist,
+                                                                   uint32_t* done, uint32_t* n_valid) {
+  constexpr int R = 1 << BITS, PER = (R + kRadixThreads - 1) / kRadixThreads;
+  __shared__ uint32_t h[PASSES * R];
+  __shared__ uint32_t s_w[kRadixWarps];
+  __shared__ bool s_last;
+  if (d_n) n = min(n, *d_n);  // device-side count (capacity launches)
+  for (int i = threadIdx.x; i < PASSES * R; i += kRadixThreads) h[i] = 0;
+  __syncthreads();
+  auto count = [&](uint32_t k) {
+    if (DROP && k == 0xffffffffu) return;
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) atomicAdd(&h[p * R + ((k >> (p * BITS)) & (R - 1))], 1u);
+  };
+  const uint32_t stride = gridDim.x * kRadixThreads, first = blockIdx.x * kRadixThreads + threadIdx.x;
+  if constexpr (std::is_same<Keys, ArrayKeys>::value) {  // arena buffers: 16-byte aligned
+    for (uint64_t i = first; 4 * i + 3 < n; i += stride) {
+      const uint4 k = reinterpret_cast<const uint4*>(keys.keys)[i];
+      count(k.x);
+      count(k.y);
+      count(k.z);
+      count(k.w);
     }
+    if (first < (n & 3u)) count(keys((n & ~3u) + first));
+  } else {
+    for (uint64_t i = first; i < n; i += stride) count(keys((uint32_t)i));
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < n_here; i += kBlock) {
-    const uint32_t kk = sk[i];
-    const uint32_t d = (kk >> shift) & mask;
-    const uint32_t pos = gbase[d] + (i - dstart[d]);
-    keys_out[pos] = kk;
+  for (int i = threadIdx.x; i < PASSES * R; i += kRadixThreads)
+    if (h[i]) atomicAdd(&hist[i], h[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+#pragma unroll
+  for (int p = 0; p < PASSES; ++p) {
+    uint32_t c[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int d = threadIdx.x * PER + k;
+      c[k] = d < R ? __ldcg(hist + p * R + d) : 0u;
+    }
+    uint32_t e = block_exclusive<PER>(c, s_w);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int d = threadIdx.x * PER + k;
+      if (d < R) hist[p * R + d] = e;
+      e += c[k];
+    }
+    if (DROP && p == 0 && threadIdx.x == kRadixThreads - 1) *n_valid = e;
+    __syncthreads();
+  }
+}
+
+// Look-back word of one (tile, digit): 0 = nothing yet, 1 + c = the tile's count c
+// (at most kRadixTile), kRadixTile + 2 + t = the total t of the tiles up to it.
+__device__ __forceinline__ uint32_t load_word(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void store_word(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Sum of the tiles before `tile` for this thread's digit (words: the digit's column,
+// R apart).  False if the wait was given up.
+template <int R>
+__device__ __forceinline__ bool look_back(const uint32_t* words, uint32_t tile, uint32_t* excl) {
+  uint32_t sum = 0, polls = 0;
+  int64_t t = (int64_t)tile - 1;
+  while (t >= 0) {
+    uint32_t w[kLookBack];
+#pragma unroll
+    for (int k = 0; k < kLookBack; ++k) w[k] = t - k >= 0 ? load_word(words + (t - k) * R) : 0u;
+    int used = 0;
+#pragma unroll
+    for (int k = 0; k < kLookBack; ++k) {
+      if (used != k || w[k] == 0u) continue;
+      if (w[k] > (uint32_t)kRadixTile + 1u) {
+        *excl = sum + (w[k] - (uint32_t)(kRadixTile + 2));
+        return true;
+      }
+      sum += w[k] - 1u;
+      used = k + 1;
+    }
+    t -= used;
+    if (used == 0 && ++polls > kSpinLimit) return false;
+  }
+  *excl = sum;
+  return true;
+}
+
+// One pass.  Warp w of a block owns the contiguous slice [w * 32 * kRadixItems, ...)
+// of its tile.  The warps first count their digits with shared-memory atomics, so
+// that the tile's counts are published before the ranking: the look-back of the
+// tiles behind it then runs while they rank.  Each warp ranks its items in their order
+// (round j: items 32 j .. 32 j + 31) from the lanes of equal digit (one ballot per
+// digit bit) and the running position of the digit in the tile, and places them in
+// digit order in shared memory; the tile is written in digit runs, so the global
+// stores are coalesced.  INDEX: the values are the items' indices (vals_in is not
+// read).  DROP: see radix_hist_kernel.
+template <class Keys, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
+__global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel(
+    const Keys keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
+    uint32_t* __restrict__ vals_out, uint32_t n, const uint32_t* __restrict__ d_n, int shift,
+    const uint32_t* __restrict__ base, uint32_t* words, uint32_t* next_tile) {
+  constexpr int R = 1 << BITS, PER = (R + kRadixThreads - 1) / kRadixThreads;
+  __shared__ uint32_t whist[kRadixWarps][R];
+  __shared__ uint32_t gofs[R];  // global position minus tile position of each digit's run
+  __shared__ uint32_t s_w[kRadixWarps];
+  __shared__ uint32_t sk[kRadixTile], sv[kRadixTile];
+  __shared__ uint32_t s_tile, s_items;
+  __shared__ int s_gave_up;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    s_tile = atomicAdd(next_tile, 1u);
+    s_gave_up = 0;
+  }
+  for (int i = lane; i < R; i += 32) whist[warp][i] = 0;
+  if (d_n) n = min(n, *d_n);
+  __syncthreads();
+  const uint32_t tile = s_tile;
+  const uint64_t first = (uint64_t)tile * kRadixTile;
+  if (first >= n) return;  // capacity launches: no tile after this one waits for it
+  const uint32_t here = (uint32_t)min((uint64_t)kRadixTile, n - first);
+  const uint32_t slice = (uint32_t)warp * 32 * kRadixItems + lane;
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t key[kRadixItems];
+#pragma unroll
+  for (int j = 0; j < kRadixItems; ++j) {
+    const uint32_t k = slice + j * 32;
+    key[j] = k < here ? keys_in((uint32_t)first + k) : 0xffffffffu;
+  }
+  auto valid = [&](int j) { return slice + j * 32 < here && (!DROP || key[j] != 0xffffffffu); };
+#pragma unroll
+  for (int j = 0; j < kRadixItems; ++j)
+    if (valid(j)) atomicAdd(&whist[warp][(key[j] >> shift) & (R - 1)], 1u);
+  uint32_t val[kRadixItems];
+#pragma unroll
+  for (int j = 0; j < kRadixItems; ++j) {
+    const uint32_t k = slice + j * 32;
+    val[j] = INDEX ? (uint32_t)first + k : k < here ? vals_in[first + k] : 0u;
+  }
+  __syncthreads();
+  // per digit: the tile's count, and the tile position of each warp's first item
+  uint32_t cnt[PER], e;
+  {
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int d = threadIdx.x * PER + k;
+      cnt[k] = 0;
+      if (d < R) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int w = 0; w < kRadixWarps; ++w) c += whist[w][d];
+        cnt[k] = c;
+        store_word(words + (size_t)tile * R + d, tile == 0 ? (uint32_t)(kRadixTile + 2) + c : 1u + c);
+      }
+    }
+    e = block_exclusive<PER>(cnt, s_w);
+    uint32_t pos = e;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int d = threadIdx.x * PER + k;
+      if (d < R) {
+#pragma unroll
+        for (int w = 0; w < kRadixWarps; ++w) {
+          const uint32_t x = whist[w][d];
+          whist[w][d] = pos;
+          pos += x;
+        }
+      }
+    }
+    if (threadIdx.x == kRadixThreads - 1) s_items = pos;  // items of the tile
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kRadixItems; ++j) {
+    const uint32_t d = (key[j] >> shift) & (R - 1);
+    unsigned peers = DROP ? __ballot_sync(kFull, valid(j)) : kFull;
+#pragma unroll
+    for (int b = 0; b < BITS; ++b) {
+      const unsigned bal = __ballot_sync(kFull, (d >> b) & 1u);
+      peers &= bal ^ (((d >> b) & 1u) - 1u);
+    }
+    // (an item past the end has the highest digit and comes last: it moves no other)
+    const int before = __popc(peers & lt);
+    const uint32_t run = whist[warp][d];
+    __syncwarp();
+    if (valid(j)) {
+      if (before == 0) whist[warp][d] = run + __popc(peers);
+      sk[run + before] = key[j];
+      sv[run + before] = val[j];
+    }
+    __syncwarp();
+  }
+  uint32_t excl[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int d = threadIdx.x * PER + k;
+    excl[k] = 0;
+    if (d < R && !look_back<R>(words + d, tile, &excl[k])) s_gave_up = 1;
+  }
+  __syncthreads();
+  if (s_gave_up) {  // count the digits of the earlier keys instead of waiting for their tiles
+    uint32_t* h = &whist[0][0];
+    for (int i = threadIdx.x; i < R; i += kRadixThreads) h[i] = 0;
+    __syncthreads();
+    for (uint64_t i = threadIdx.x; i < first; i += kRadixThreads) {
+      const uint32_t k = keys_in((uint32_t)i);
+      if (!DROP || k != 0xffffffffu) atomicAdd(&h[(k >> shift) & (R - 1)], 1u);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int d = threadIdx.x * PER + k;
+      if (d < R) excl[k] = h[d];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int d = threadIdx.x * PER + k;
+    if (d < R) {
+      if (tile) store_word(words + (size_t)tile * R + d, (uint32_t)(kRadixTile + 2) + excl[k] + cnt[k]);
+      gofs[d] = base[d] + excl[k] - e;
+    }
+    e += cnt[k];
+  }
+  __syncthreads();
+  const uint32_t n_out = DROP ? s_items : here;
+  for (uint32_t i = threadIdx.x; i < n_out; i += kRadixThreads) {
+    const uint32_t k = sk[i];
+    const uint32_t pos = gofs[(k >> shift) & (R - 1)] + i;
+    if (KEYS_OUT) keys_out[pos] = k;
     vals_out[pos] = sv[i];
   }
 }
@@ -555,11 +738,65 @@ cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, uint32_t n, ui
   return scan_exclusive<uint32_t>(in, out, n, d_total, static_cast<char*>(scratch), s);
 }
 
+namespace {
+
+// Scratch of one sort, zeroed by one memset: digit positions, counters, look-back words.
+struct RadixScratch {
+  uint32_t *base, *done, *next_tile, *words;
+  size_t tiles, bytes;
+};
+RadixScratch radix_layout(void* scratch, uint32_t n, int passes, int bits) {
+  RadixScratch w;
+  const size_t R = (size_t)1 << bits;
+  w.tiles = ((size_t)n + kRadixTile - 1) / kRadixTile;
+  w.base = static_cast<uint32_t*>(scratch);
+  w.done = w.base + passes * R;
+  w.next_tile = w.done + 1;
+  w.words = w.base + passes * R + 64;
+  w.bytes = sizeof(uint32_t) * (passes * R + 64 + passes * w.tiles * R);
+  return w;
+}
+
+template <class Keys, int BITS, int PASSES, bool DROP>
+cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const RadixScratch& w, uint32_t* n_valid,
+                        cudaStream_t s) {
+  // about 16 keys per thread, at most four blocks per SM
+  const uint32_t blocks = (uint32_t)std::min<size_t>((size_t)152 * 4, ((size_t)n + 16 * kRadixThreads - 1) / (16 * kRadixThreads));
+  radix_hist_kernel<Keys, BITS, PASSES, DROP><<<blocks, kRadixThreads, 0, s>>>(k, n, d_n, w.base, w.done, n_valid);
+  return launched();
+}
+
+template <class Keys, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
+cudaError_t launch_pass(const Keys& k, const uint32_t* vals, uint32_t* keys_out, uint32_t* vals_out, uint32_t n,
+                        const uint32_t* d_n, int p, const RadixScratch& w, cudaStream_t s) {
+  radix_pass_kernel<Keys, BITS, INDEX, DROP, KEYS_OUT><<<(unsigned)w.tiles, kRadixThreads, 0, s>>>(
+      k, vals, keys_out, vals_out, n, d_n, p * BITS, w.base + (size_t)p * (1 << BITS),
+      w.words + (size_t)p * w.tiles * (1 << BITS), w.next_tile + p);
+  return launched();
+}
+
+template <int BITS, int PASSES>
+cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
+                        void* scratch, cudaStream_t s, const uint32_t* d_n, bool index_vals) {
+  const RadixScratch w = radix_layout(scratch, n, PASSES, BITS);
+  cudaError_t e = cudaMemsetAsync(scratch, 0, w.bytes, s);
+  if (e != cudaSuccess) return e;
+  e = launch_hist<ArrayKeys, BITS, PASSES, false>(ArrayKeys{keys}, n, d_n, w, nullptr, s);
+  uint32_t *kin = keys, *vin = vals, *kout = keys_alt, *vout = vals_alt;
+  for (int p = 0; p < PASSES && e == cudaSuccess; ++p) {
+    e = p == 0 && index_vals
+            ? launch_pass<ArrayKeys, BITS, true, false, true>(ArrayKeys{kin}, nullptr, kout, vout, n, d_n, p, w, s)
+            : launch_pass<ArrayKeys, BITS, false, false, true>(ArrayKeys{kin}, vin, kout, vout, n, d_n, p, w, s);
+    std::swap(kin, kout);
+    std::swap(vin, vout);
+  }
+  return e;
+}
+
+}  // namespace
+
 size_t radix_scratch_bytes(uint32_t n) {
-  const uint32_t nb = (n + kChunk - 1) / kChunk;
-  const size_t counts = (size_t)kMaxRadix * nb;
-  const size_t cbytes = (counts * sizeof(uint32_t) + 255) & ~(size_t)255;
-  return cbytes + scan_levels_bytes<uint32_t>((uint32_t)counts) + 256;
+  return radix_layout(nullptr, n, 4, kMaxDigit).bytes;  // the largest of any digit plan
 }
 
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
@@ -567,37 +804,19 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
                              const uint32_t* d_n, bool index_vals) {
   *result_in_alt = false;
   if (n <= 1 || n_bits <= 0) {
-    if (index_vals && n > 0) {  // nothing to sort: the values are the indices
-      launch_iota(vals, n, s);
-      return launched();
-    }
+    if (index_vals && n > 0) return launch_iota(vals, n, s);  // nothing to sort: the values are the indices
     return cudaSuccess;
   }
-  const uint32_t nb = (n + kChunk - 1) / kChunk;
-  const int passes = (n_bits + 7) / 8;
-  const int digit = (n_bits + passes - 1) / passes;  // balanced digit width <= 8
-  uint32_t* counts = static_cast<uint32_t*>(scratch);
-  const size_t cbytes = ((size_t)kMaxRadix * nb * sizeof(uint32_t) + 255) & ~(size_t)255;
-  char* scan_scratch = static_cast<char*>(scratch) + cbytes;
-  uint32_t *kin = keys, *vin = vals, *kout = keys_alt, *vout = vals_alt;
-  for (int p = 0; p < passes; ++p) {
-    const int shift = p * digit;
-    const int width = min(digit, n_bits - shift);
-    const uint32_t mask = (1u << width) - 1u;
-    radix_upsweep_kernel<<<nb, kBlock, 0, s>>>(kin, n, shift, mask, counts, nb, d_n);
-    cudaError_t e = launched();
-    if (e != cudaSuccess) return e;
-    e = scan_exclusive<uint32_t>(counts, counts, (mask + 1) * nb, nullptr, scan_scratch, s);
-    if (e != cudaSuccess) return e;
-    radix_scatter_kernel<<<nb, kBlock, 0, s>>>(kin, p == 0 && index_vals ? nullptr : vin, kout, vout, n, shift,
-                                               mask, counts, nb, d_n);
-    e = launched();
-    if (e != cudaSuccess) return e;
-    uint32_t* t = kin; kin = kout; kout = t;
-    t = vin; vin = vout; vout = t;
-    *result_in_alt = !*result_in_alt;
-  }
-  return cudaSuccess;
+  const DigitPlan pl = digit_plan(n_bits);
+  *result_in_alt = pl.passes % 2 != 0;
+#define OCGS_SORT(B, P) \
+  if (pl.bits == B && pl.passes == P) \
+    return sort_passes<B, P>(keys, vals, keys_alt, vals_alt, n, scratch, s, d_n, index_vals);
+  OCGS_SORT(4, 1) OCGS_SORT(5, 1) OCGS_SORT(6, 1) OCGS_SORT(7, 1) OCGS_SORT(8, 1)
+  OCGS_SORT(5, 2) OCGS_SORT(6, 2) OCGS_SORT(7, 2) OCGS_SORT(8, 2)
+  OCGS_SORT(6, 3) OCGS_SORT(7, 3) OCGS_SORT(8, 3) OCGS_SORT(8, 4)
+#undef OCGS_SORT
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_gather_counts(const uint32_t* order, const int32_t* ntiles, uint64_t* counts,
