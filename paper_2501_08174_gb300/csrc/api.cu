@@ -9,6 +9,7 @@
 #include "ocgs.h"
 #include "common.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -29,9 +30,9 @@ struct ocgs_ctx {
   int cover_rect = 0;  // ocgs_set_coverage
   ocgs_stats stats{};
   std::string err;
+  uint64_t* d_scalar = nullptr;   // device scalars [32]; d_status is the last of them
+  uint64_t* h_scalar = nullptr;   // pinned copy
   int* d_status = nullptr;
-  uint64_t* d_scalar = nullptr;   // [4]
-  uint64_t* h_scalar = nullptr;   // pinned [4]
   int sm_count = 0;
   // built-in stage profiler: event pairs recorded on the stream around each stage
   bool prof = false;
@@ -110,6 +111,40 @@ struct Arena {
     dst.insert(dst.end(), ptrs.begin(), ptrs.end());
     ptrs.clear();
   }
+};
+
+// Several buffers of one arena in one allocation, each 256-byte aligned: a call pays the
+// allocator once per phase instead of once per buffer.  Buffers added with zeroed() lie
+// together at the front and are cleared by one memset.
+class Block {
+ public:
+  template <typename T>
+  void add(T** p, size_t count) { parts_.push_back({reinterpret_cast<void**>(p), bytes_of(count * sizeof(T))}); }
+  template <typename T>
+  void zeroed(T** p, size_t count) { zero_.push_back({reinterpret_cast<void**>(p), bytes_of(count * sizeof(T))}); }
+  cudaError_t alloc(Arena& a, cudaStream_t s) {
+    size_t total = 0, clear = 0;
+    for (const Part& q : zero_) clear += q.bytes;
+    total = clear;
+    for (const Part& q : parts_) total += q.bytes;
+    char* base = nullptr;
+    const cudaError_t e = a.alloc(&base, total);
+    if (e != cudaSuccess) return e;
+    for (const std::vector<Part>* v : {&zero_, &parts_})
+      for (const Part& q : *v) {
+        *q.p = base;
+        base += q.bytes;
+      }
+    return clear ? cudaMemsetAsync(base - total, 0, clear, s) : cudaSuccess;
+  }
+
+ private:
+  struct Part {
+    void** p;
+    size_t bytes;
+  };
+  static size_t bytes_of(size_t n) { return (std::max<size_t>(n, 16) + 255) & ~(size_t)255; }
+  std::vector<Part> zero_, parts_;
 };
 
 // Records a CUDA event pair around one stage when the profiler is on.
@@ -248,10 +283,14 @@ ocgs_status plan_loss(ocgs_ctx* ctx, const ocgs_camera* cams, int n_views, LossP
   return OCGS_OK;
 }
 
-ocgs_status read_status(ocgs_ctx* ctx, int* status) {
-  CK(cudaMemcpyAsync(ctx->h_scalar + 3, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// Device scalars of a forward pass (one copy reads them all back), by index into d_scalar.
+enum { kPairs1 = 0, kPairs2 = 1, kValid = 2, kScalarStatus = 31 };
+
+// Copies the device scalars back and waits for the stream.
+ocgs_status read_scalars(ocgs_ctx* ctx, int* status) {
+  CK(cudaMemcpyAsync(ctx->h_scalar, ctx->d_scalar, 32 * sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  *status = *reinterpret_cast<int*>(ctx->h_scalar + 3);
+  *status = *reinterpret_cast<int*>(ctx->h_scalar + kScalarStatus);
   return OCGS_OK;
 }
 
@@ -271,7 +310,8 @@ void free_state(ocgs_fwd_state* st) {
 }
 
 // The forward pipeline shared by ocgs_render and ocgs_accumulate_contribution:
-// preprocess, depth sort, duplication, tile sort, ranges, rasterization.
+// preprocess, depth sort, duplication, tile sort, ranges, rasterization.  keep_state:
+// the backward's state is kept in st.
 ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_camera* cams, int V,
                          const ocgs_image* out, float* score, ocgs_fwd_state* st, bool keep_state,
                          bool ewa = false) {
@@ -282,41 +322,69 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
     return set_err(ctx, OCGS_ERR_CAPACITY, "n_views * n exceeds 2^32 - 1 records");
   if (pl.tiles >= (int64_t)INT32_MAX) return set_err(ctx, OCGS_ERR_CAPACITY, "too many tiles");
   const uint32_t VN = (uint32_t)(N * V);
+  const uint32_t n_t = (uint32_t)pl.tiles;
   cudaStream_t s = ctx->stream;
   Arena keep(ctx), tmp(ctx);
 
   st->ctx = ctx; st->V = V; st->N = N; st->deg = g->sh_degree; st->P = pl.P;
-  st->n_tiles = (uint32_t)pl.tiles; st->tile_w = tw; st->tile_h = th; st->ppt = ctx->opts.pixels_per_thread;
+  st->n_tiles = n_t; st->tile_w = tw; st->tile_h = th; st->ppt = ctx->opts.pixels_per_thread;
   st->batch = ctx->opts.batch;
   st->persistent = ctx->opts.persistent;
-  CK(keep.alloc(&st->d_cams, V));
-  CK(keep.alloc(&st->d_tile_prefix, V + 1));
-  CK(cudaMemcpyAsync(st->d_cams, pl.cams.data(), sizeof(DevCam) * V, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(st->d_tile_prefix, pl.tile_prefix.data(), sizeof(int) * (V + 1), cudaMemcpyHostToDevice, s));
-  CK(keep.alloc(&st->rec.g0, VN));
-  CK(keep.alloc(&st->rec.g1, VN));
-  CK(keep.alloc(&st->rec.g2, VN));
-  CK(keep.alloc(&st->rec.a0, VN));
-  CK(keep.alloc(&st->rec.a1, VN));
-  CK(keep.alloc(&st->ntiles, VN));
-  CK(keep.alloc(&st->ranges, pl.tiles));
-  CK(keep.alloc(&st->t_final, keep_state ? pl.P : 1));
-  CK(keep.alloc(&st->last, keep_state ? pl.P : 1));
-  float4* bin;
-  uint32_t *dkey, *order, *dkey_alt, *order_alt;
-  uint64_t* counts;
-  CK(tmp.alloc(&bin, 3 * (size_t)VN));
-  CK(tmp.alloc(&dkey, VN));
-  CK(tmp.alloc(&order, VN));
-  CK(tmp.alloc(&dkey_alt, VN));
-  CK(tmp.alloc(&order_alt, VN));
-  CK(tmp.alloc(&counts, VN));
-  char* scratch;
-  const size_t sbytes = std::max(radix_scratch_bytes(VN), scan_scratch_bytes(VN));
-  CK(tmp.alloc(&scratch, sbytes));
-  CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), s));
-  CK(cudaMemsetAsync(st->ranges, 0, sizeof(uint2) * pl.tiles, s));
+  // Two passes need something to continue: images, or the contribution score.  The front of
+  // the depth order is binned and rendered first.  Each tile with a pixel still running at
+  // the end of that prefix is then binned with the records behind the front and continues
+  // from the state the first pass left (T, the sums, the last blended position, the stop
+  // flags): every pixel walks the same list, in the same order, as in one pass.
+  const bool img = out != nullptr;
+  const bool two_pass = (img || score != nullptr) && st->persistent && ctx->opts.front_fraction > 0.f && VN > 0;
+  uint32_t M = VN;  // entries of the depth order binned in the first pass
+  if (two_pass) {
+    const double front = std::ceil((double)ctx->opts.front_fraction * (double)VN);
+    M = (uint32_t)std::min<double>((double)VN, std::max(1.0, front));
+  }
+  const int tbits = bits_for((uint64_t)pl.tiles);
 
+  char* tables;  // the cameras, then the tile prefix
+  const size_t cam_bytes = (sizeof(DevCam) * V + 255) & ~(size_t)255;
+  const size_t table_bytes = cam_bytes + sizeof(int) * (V + 1);
+  float4* bin;
+  uint32_t *dkey, *dkey_alt, *order, *order_alt, *done1;
+  uint64_t* unit_base;
+  char* dscratch;
+  {
+    Block b;
+    b.add(&tables, table_bytes);
+    b.add(&st->rec.g0, VN);
+    b.add(&st->rec.g1, VN);
+    b.add(&st->rec.g2, VN);
+    b.add(&st->rec.a0, VN);
+    b.add(&st->rec.a1, VN);
+    b.add(&st->ntiles, VN);
+    b.zeroed(&st->ranges, n_t);
+    if (keep_state) {
+      b.add(&st->t_final, pl.P);
+      b.add(&st->last, pl.P);
+      if (st->persistent) b.add(&st->tile_order, n_t);
+    }
+    CK(b.alloc(keep, s));
+    Block t;
+    t.add(&bin, 3 * (size_t)VN);
+    t.add(&dkey, VN);
+    t.add(&dkey_alt, VN);
+    t.add(&order, VN);
+    t.add(&order_alt, VN);
+    t.add(&unit_base, unit_base_words(VN));
+    t.zeroed(&done1, 1);
+    t.zeroed(&dscratch, depth_sort_scratch_bytes(VN));
+    CK(t.alloc(tmp, s));
+  }
+  st->d_cams = reinterpret_cast<DevCam*>(tables);
+  st->d_tile_prefix = reinterpret_cast<int*>(tables + cam_bytes);
+  std::vector<char> h_tables(table_bytes);
+  std::memcpy(h_tables.data(), pl.cams.data(), sizeof(DevCam) * V);
+  std::memcpy(h_tables.data() + cam_bytes, pl.tile_prefix.data(), sizeof(int) * (V + 1));
+  CK(cudaMemcpyAsync(tables, h_tables.data(), table_bytes, cudaMemcpyHostToDevice, s));
+  CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), s));
   {
     StageTimer t(ctx, OCGS_STAGE_PREPROCESS);
     if (ewa)
@@ -326,293 +394,174 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
       CK(launch_preprocess(gptrs(g), N, g->sh_degree, st->d_cams, V, tw, th, st->rec, st->ntiles, bin, dkey,
                            ctx->d_status, s));
   }
+  uint32_t* d_valid = reinterpret_cast<uint32_t*>(ctx->d_scalar + kValid);  // records with a non-empty screen box
+  {
+    StageTimer t(ctx, OCGS_STAGE_DEPTH_SORT);
+    CK(depth_sort(dkey, dkey_alt, order, order_alt, VN, d_valid, dscratch, s));
+  }
+  {
+    StageTimer t(ctx, OCGS_STAGE_BINNING);
+    CK(launch_bin_count(order, M, d_valid, bin, st->d_cams, N, tw, th, unit_base, done1,
+                        ctx->d_scalar + kPairs1, s));
+  }
   int status = 0;
-  uint32_t K = 0;
-  // two passes need something to continue: images, or the contribution score
-  const bool two_pass = (out != nullptr || score != nullptr) && st->persistent && ctx->opts.front_fraction > 0.f &&
-                        VN > 0;
-  if (!two_pass) {
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_tile_count(bin, st->d_cams, N, VN, tw, th, st->ntiles, dkey, s));
-    }
-    bool alt = false;
-    {
-      StageTimer t(ctx, OCGS_STAGE_DEPTH_SORT);
-      CK(radix_sort_pairs(dkey, order, dkey_alt, order_alt, VN, 32, scratch, &alt, s, nullptr, true));
-    }
-    uint32_t* sorted = alt ? order_alt : order;
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_gather_counts(sorted, st->ntiles, counts, VN, s));
-      CK(scan_exclusive_u64(counts, counts, VN, ctx->d_scalar, scratch, s));
-    }
-    CK(cudaMemcpyAsync(ctx->h_scalar, ctx->d_scalar, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    ocgs_status rs = read_status(ctx, &status);
-    if (rs != OCGS_OK) return rs;
-    const uint64_t K64 = VN ? ctx->h_scalar[0] : 0;
-    if (K64 > (uint64_t)INT32_MAX)
-      return set_err(ctx, OCGS_ERR_CAPACITY, "more than 2^31-1 (tile, Gaussian) pairs; split the views");
-    K = (uint32_t)K64;
-    st->K = K;
+  ocgs_status rs = read_scalars(ctx, &status);
+  if (rs != OCGS_OK) return rs;
+  const uint64_t K1_64 = ctx->h_scalar[kPairs1];
+  if (K1_64 > (uint64_t)INT32_MAX)
+    return set_err(ctx, OCGS_ERR_CAPACITY, "more than 2^31-1 (tile, Gaussian) pairs; split the views");
+  const uint32_t K1 = (uint32_t)K1_64;
+  const uint32_t n_valid = *reinterpret_cast<const uint32_t*>(ctx->h_scalar + kValid);
+  const bool second = M < n_valid;  // records behind the front remain
+  const uint32_t n_back = second ? n_valid - M : 0u;
 
-    uint32_t *pkey, *pval, *pkey_alt, *pval_alt;
-    CK(tmp.alloc(&pkey, K));
-    CK(keep.alloc(&pval, K));
-    CK(tmp.alloc(&pkey_alt, K));
-    CK(keep.alloc(&pval_alt, K));
-    char* pscratch;
-    CK(tmp.alloc(&pscratch, radix_scratch_bytes(K)));
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_duplicate(sorted, counts, reinterpret_cast<const uint64_t*>(ctx->d_scalar), VN, bin, st->d_cams,
-                          N, tw, th, K, pkey, pval, s));
-    }
-    const int tbits = bits_for((uint64_t)pl.tiles);
-    bool palt = false;
-    {
-      StageTimer t(ctx, OCGS_STAGE_TILE_SORT);
-      CK(radix_sort_pairs(pkey, pval, pkey_alt, pval_alt, K, tbits, pscratch, &palt, s));
-    }
-    uint32_t* skey = palt ? pkey_alt : pkey;
-    st->vals = palt ? pval_alt : pval;
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_tile_ranges(skey, K, st->ranges, s));
-    }
-
-    uint32_t* queue = nullptr;
-    st->tile_order = nullptr;
+  // the first pass: pairs, tile sort, ranges, queue order, rasterization
+  uint32_t *pkey, *pval, *pkey_alt, *pval_alt, *queue = nullptr, *ids = nullptr;
+  uint32_t *open = nullptr, *prefix = nullptr, *open_ids = nullptr, *open_words = nullptr, *done2 = nullptr;
+  uint32_t* n_cand = nullptr;
+  uint8_t* done = nullptr;
+  char *pscratch, *oscratch = nullptr, *qscratch = nullptr, *bscratch = nullptr;
+  // the second pass continues from T (and, with images, the last blended position)
+  float* t_fin = keep_state && img ? st->t_final : nullptr;
+  uint32_t* lst = keep_state && img ? st->last : nullptr;
+  const bool alt1 = radix_result_in_alt(K1, tbits);
+  {
+    Block b;
+    b.add(alt1 ? &pval_alt : &pval, K1);
+    CK(b.alloc(keep, s));
+    Block t;
+    t.add(alt1 ? &pval : &pval_alt, K1);
+    t.add(&pkey, K1);
+    t.add(&pkey_alt, K1);
+    t.zeroed(&pscratch, radix_scratch_bytes(K1, tbits));
     if (st->persistent) {
-      CK(tmp.alloc(&queue, 1));
-      CK(cudaMemsetAsync(queue, 0, sizeof(uint32_t), s));
-      uint32_t *wk, *ids, *wk_alt, *ids_alt;
-      CK(tmp.alloc(&wk, pl.tiles));
-      CK(keep.alloc(&ids, pl.tiles));
-      CK(tmp.alloc(&wk_alt, pl.tiles));
-      CK(keep.alloc(&ids_alt, pl.tiles));
-      char* tscratch;
-      CK(tmp.alloc(&tscratch, radix_scratch_bytes((uint32_t)pl.tiles)));
-      CK(launch_tile_order(st->ranges, (uint32_t)pl.tiles, wk, ids, s));
-      bool talt = false;
-      CK(radix_sort_pairs(wk, ids, wk_alt, ids_alt, (uint32_t)pl.tiles, 8, tscratch, &talt, s));
-      st->tile_order = talt ? ids_alt : ids;
+      t.zeroed(&queue, 2);
+      t.add(&ids, n_t);
+      t.zeroed(&oscratch, tile_order_scratch_bytes(n_t));
+      if (keep_state && two_pass) t.zeroed(&bscratch, tile_order_scratch_bytes(n_t));
     }
+    if (second) {
+      if (!t_fin) t.add(&t_fin, pl.P);
+      t.add(&done, pl.P);
+      t.zeroed(&open, n_t);
+      t.add(&prefix, (size_t)n_t + 1);
+      t.add(&open_ids, n_t);
+      t.zeroed(&open_words, open_scan_words(n_t));
+      t.zeroed(&done2, 1);
+      t.add(&n_cand, unit_capacity(n_back));
+      t.zeroed(&qscratch, tile_order_scratch_bytes(n_t));
+    }
+    CK(t.alloc(tmp, s));
+  }
+  {
+    StageTimer t(ctx, OCGS_STAGE_BINNING);
+    CK(launch_duplicate(order, M, d_valid, unit_base, bin, st->d_cams, N, tw, th, K1, pkey, pval, s));
+  }
+  {
+    StageTimer t(ctx, OCGS_STAGE_TILE_SORT);
+    CK(radix_sort_pairs(pkey, pval, pkey_alt, pval_alt, K1, tbits, pscratch, s));
+  }
+  st->vals = alt1 ? pval_alt : pval;
+  {
+    StageTimer t(ctx, OCGS_STAGE_BINNING);
+    CK(launch_tile_ranges(alt1 ? pkey_alt : pkey, K1, st->ranges, s));
+  }
+  if (st->persistent) {
+    if (keep_state && !two_pass) ids = st->tile_order;  // the backward takes the same order
+    CK(launch_tile_order(st->ranges, nullptr, n_t, ids, oscratch, s));
+  }
+  RasterArgs ra{};
+  ra.ewa = ewa ? 1 : 0;
+  ra.cams = st->d_cams;
+  ra.tile_prefix = st->d_tile_prefix;
+  ra.n_views = V;
+  ra.n_gauss = N;
+  ra.n_tiles = n_t;
+  ra.ranges = st->ranges;
+  ra.vals = st->vals;
+  ra.rec = st->rec;
+  if (img) ra.out = ImgPtrs{out->rgb, out->alpha, out->depth, out->normal, out->depth2};
+  ra.t_final = t_fin;
+  ra.last = lst;
+  ra.score = score;
+  ra.tile_order = ids;
+  ra.queue = queue;
+  ra.persistent_ctas = st->persistent ? ctx->sm_count * (2048 * st->ppt / (tw * th)) : 0;
+  ra.open = open;
+  ra.done = done;
+  {
+    StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
+    CK(launch_raster_forward(ra, tw, th, st->ppt, st->batch, img, s));
+  }
 
-    RasterArgs ra{};
-    ra.ewa = ewa ? 1 : 0;
-    ra.cams = st->d_cams;
-    ra.tile_prefix = st->d_tile_prefix;
-    ra.n_views = V;
-    ra.n_gauss = N;
-    ra.n_tiles = (uint32_t)pl.tiles;
-    ra.ranges = st->ranges;
-    ra.vals = st->vals;
-    ra.rec = st->rec;
-    if (out) ra.out = ImgPtrs{out->rgb, out->alpha, out->depth, out->normal, out->depth2};
-    ra.t_final = keep_state ? st->t_final : nullptr;  // no state kept: nothing to write
-    ra.last = keep_state ? st->last : nullptr;
-    ra.score = score;
-    ra.tile_order = st->tile_order;
-    ra.queue = queue;
-    ra.persistent_ctas = st->persistent ? ctx->sm_count * (2048 * st->ppt / (tw * th)) : 0;
-    {
-      StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
-      CK(launch_raster_forward(ra, tw, th, st->ppt, st->batch, out != nullptr, s));
-    }
-
-  } else {
-    // Two passes.  The front of the depth order is binned and rendered first.
-    // Each tile with a pixel still running at the end of that prefix is then
-    // binned with the records behind the front and continues from the state
-    // the first pass left (T, the sums, the last blended position, the stop
-    // flags): every pixel walks the same list, in the same order, as in one pass.
-    bool alt = false;
-    {
-      StageTimer t(ctx, OCGS_STAGE_DEPTH_SORT);
-      CK(radix_sort_pairs(dkey, order, dkey_alt, order_alt, VN, 32, scratch, &alt, s, nullptr, true));
-    }
-    uint32_t* sorted = alt ? order_alt : order;
-    const uint32_t* skeys = alt ? dkey_alt : dkey;
-    const double front = std::ceil((double)ctx->opts.front_fraction * (double)VN);
-    const uint32_t M = (uint32_t)std::min<double>((double)VN, std::max(1.0, front));
-    uint32_t* d_valid = reinterpret_cast<uint32_t*>(ctx->d_scalar + 4);
+  uint32_t K2 = 0;
+  if (second) {
+    uint32_t *cand = order_alt, *counts = dkey;  // their last use was in the depth sort
     {
       StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_tile_count_sorted(sorted, M, bin, st->d_cams, N, tw, th, st->ntiles, counts, s));
-      CK(scan_exclusive_u64(counts, counts, M, ctx->d_scalar, scratch, s));
-      CK(launch_count_below(skeys, VN, 0xffffffffu, d_valid, s));  // records with a non-empty screen box
+      CK(launch_open_scan(open, n_t, prefix, open_ids, open_words, s));
+      CK(launch_open_count(order + M, n_back, bin, st->d_cams, N, tw, th, prefix, cand, counts, n_cand, unit_base,
+                           done2, ctx->d_scalar + kPairs2, s));
     }
-    CK(cudaMemcpyAsync(ctx->h_scalar, ctx->d_scalar, 5 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    ocgs_status rs = read_status(ctx, &status);
+    int later = 0;
+    rs = read_scalars(ctx, &later);
     if (rs != OCGS_OK) return rs;
-    const uint64_t K1_64 = ctx->h_scalar[0];
-    const uint32_t n_valid = *reinterpret_cast<const uint32_t*>(ctx->h_scalar + 4);
-    if (K1_64 > (uint64_t)INT32_MAX)
+    const uint64_t K2_64 = ctx->h_scalar[kPairs2];
+    if ((uint64_t)K1 + K2_64 > (uint64_t)INT32_MAX)
       return set_err(ctx, OCGS_ERR_CAPACITY, "more than 2^31-1 (tile, Gaussian) pairs; split the views");
-    const uint32_t K1 = (uint32_t)K1_64;
-    const bool second = M < n_valid;  // records behind the front remain
-    const int tbits = bits_for((uint64_t)pl.tiles);
-    const uint32_t n_t = (uint32_t)pl.tiles;
-
-    uint32_t *pkey, *pval, *pkey_alt, *pval_alt;
-    CK(tmp.alloc(&pkey, K1));
-    CK(keep.alloc(&pval, K1));
-    CK(tmp.alloc(&pkey_alt, K1));
-    CK(keep.alloc(&pval_alt, K1));
-    char* pscratch;
-    CK(tmp.alloc(&pscratch, radix_scratch_bytes(K1)));
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_duplicate(sorted, counts, reinterpret_cast<const uint64_t*>(ctx->d_scalar), M, bin, st->d_cams, N,
-                          tw, th, K1, pkey, pval, s));
-    }
-    bool palt = false;
-    {
-      StageTimer t(ctx, OCGS_STAGE_TILE_SORT);
-      CK(radix_sort_pairs(pkey, pval, pkey_alt, pval_alt, K1, tbits, pscratch, &palt, s));
-    }
-    st->vals = palt ? pval_alt : pval;
-    {
-      StageTimer t(ctx, OCGS_STAGE_BINNING);
-      CK(launch_tile_ranges(palt ? pkey_alt : pkey, K1, st->ranges, s));
-    }
-    uint32_t *queue, *wk, *ids, *wk_alt, *ids_alt;
-    CK(tmp.alloc(&queue, 1));
-    CK(tmp.alloc(&wk, n_t));
-    CK(tmp.alloc(&ids, n_t));
-    CK(tmp.alloc(&wk_alt, n_t));
-    CK(tmp.alloc(&ids_alt, n_t));
-    char* tscratch;
-    CK(tmp.alloc(&tscratch, std::max(radix_scratch_bytes(n_t), scan_scratch_bytes(n_t + 1))));
-    CK(cudaMemsetAsync(queue, 0, sizeof(uint32_t), s));
-    CK(launch_tile_order(st->ranges, n_t, wk, ids, s));
-    bool talt = false;
-    CK(radix_sort_pairs(wk, ids, wk_alt, ids_alt, n_t, 8, tscratch, &talt, s));
-    // the first pass leaves each pixel's state for the second: T and the last
-    // blended position (the kept state, or scratch), the stop flags, the open tiles
-    const bool img = out != nullptr;
-    float* t_fin = keep_state && img ? st->t_final : nullptr;
-    uint32_t* lst = keep_state && img ? st->last : nullptr;
-    uint32_t* open = nullptr;
-    uint8_t* done = nullptr;
-    if (second) {
-      if (!t_fin) CK(tmp.alloc(&t_fin, pl.P));
-      if (!lst && img) CK(tmp.alloc(&lst, pl.P));
-      CK(tmp.alloc(&open, n_t));
-      CK(tmp.alloc(&done, pl.P));
-      CK(cudaMemsetAsync(open, 0, sizeof(uint32_t) * n_t, s));
-    }
-    RasterArgs ra{};
-    ra.ewa = ewa ? 1 : 0;
-    ra.cams = st->d_cams;
-    ra.tile_prefix = st->d_tile_prefix;
-    ra.n_views = V;
-    ra.n_gauss = N;
-    ra.n_tiles = n_t;
-    ra.ranges = st->ranges;
-    ra.vals = st->vals;
-    ra.rec = st->rec;
-    if (img) ra.out = ImgPtrs{out->rgb, out->alpha, out->depth, out->normal, out->depth2};
-    ra.t_final = t_fin;
-    ra.last = lst;
-    ra.score = score;
-    ra.tile_order = talt ? ids_alt : ids;
-    ra.queue = queue;
-    ra.persistent_ctas = ctx->sm_count * (2048 * st->ppt / (tw * th));
-    ra.open = open;
-    ra.done = done;
-    {
-      StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
-      CK(launch_raster_forward(ra, tw, th, st->ppt, st->batch, img, s));
-    }
-    uint32_t K2 = 0;
-    uint32_t* P = nullptr;
-    const uint32_t n_back = second ? n_valid - M : 0u;  // records behind the front
-    // candidates of the second pass: the sorted order's first M entries are no longer
-    // needed, nor are the depth keys (flag and position scratch)
-    uint32_t* cand = order == sorted ? order_alt : order;
-    uint32_t* n_cand = reinterpret_cast<uint32_t*>(ctx->d_scalar + 7);
-    if (second) {
-      CK(tmp.alloc(&P, (size_t)n_t + 1));
-      {
-        StageTimer t(ctx, OCGS_STAGE_BINNING);
-        CK(scan_exclusive_u32(open, P, n_t, P + n_t, tscratch, s));
-        // the records behind the front whose screen box meets an open tile, then their exact counts
-        CK(launch_open_candidates(sorted + M, n_back, bin, st->d_cams, N, P, dkey, dkey_alt, cand, n_cand, scratch,
-                                  s));
-        CK(launch_open_count(cand, n_back, n_cand, bin, st->d_cams, N, tw, th, P, counts, s));
-        CK(scan_exclusive_u64(counts, counts, n_back, ctx->d_scalar + 5, scratch, s));
-      }
-      CK(cudaMemcpyAsync(ctx->h_scalar + 5, ctx->d_scalar + 5, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-      CK(cudaStreamSynchronize(s));
-      const uint64_t K2_64 = ctx->h_scalar[5];
-      if ((uint64_t)K1 + K2_64 > (uint64_t)INT32_MAX)
-        return set_err(ctx, OCGS_ERR_CAPACITY, "more than 2^31-1 (tile, Gaussian) pairs; split the views");
-      K2 = (uint32_t)K2_64;
-    }
+    K2 = (uint32_t)K2_64;
     if (K2) {
       uint32_t *qkey, *qval, *qkey_alt, *qval_alt;
-      CK(tmp.alloc(&qkey, K2));
-      CK(keep.alloc(&qval, K2));
-      CK(tmp.alloc(&qkey_alt, K2));
-      CK(keep.alloc(&qval_alt, K2));
-      char* qscratch;
-      CK(tmp.alloc(&qscratch, radix_scratch_bytes(K2)));
-      CK(keep.alloc(&st->ranges2, n_t));
-      CK(cudaMemsetAsync(st->ranges2, 0, sizeof(uint2) * n_t, s));
+      char* pscratch2;
+      const bool alt2 = radix_result_in_alt(K2, tbits);
+      {
+        Block b;
+        b.add(alt2 ? &qval_alt : &qval, K2);
+        b.zeroed(&st->ranges2, n_t);
+        CK(b.alloc(keep, s));
+        Block t;
+        t.add(alt2 ? &qval : &qval_alt, K2);
+        t.add(&qkey, K2);
+        t.add(&qkey_alt, K2);
+        t.zeroed(&pscratch2, radix_scratch_bytes(K2, tbits));
+        CK(t.alloc(tmp, s));
+      }
       {
         StageTimer t(ctx, OCGS_STAGE_BINNING);
-        uint32_t* open_ids;
-        CK(tmp.alloc(&open_ids, n_t));
-        CK(launch_duplicate_open(cand, counts, ctx->d_scalar + 5, n_back, n_cand, bin, st->d_cams, N, tw, th, open,
-                                 P, n_t, open_ids, K2, qkey, qval, s));
+        CK(launch_duplicate_open(cand, n_back, counts, n_cand, unit_base, bin, st->d_cams, N, tw, th, open_ids, prefix,
+                                 K2, qkey, qval, s));
       }
-      bool qalt = false;
       {
         StageTimer t(ctx, OCGS_STAGE_TILE_SORT);
-        CK(radix_sort_pairs(qkey, qval, qkey_alt, qval_alt, K2, tbits, qscratch, &qalt, s));
+        CK(radix_sort_pairs(qkey, qval, qkey_alt, qval_alt, K2, tbits, pscratch2, s));
       }
-      st->vals2 = qalt ? qval_alt : qval;
-      uint32_t* n_again = reinterpret_cast<uint32_t*>(ctx->d_scalar + 6);
+      st->vals2 = alt2 ? qval_alt : qval;
+      RasterArgs rb = ra;
       {
         StageTimer t(ctx, OCGS_STAGE_BINNING);
-        CK(launch_tile_ranges(qalt ? qkey_alt : qkey, K2, st->ranges2, s));
-        CK(cudaMemsetAsync(n_again, 0, sizeof(uint32_t), s));
-        CK(launch_second_queue(st->ranges2, n_t, wk, ids, n_again, s));
-        CK(radix_sort_pairs(wk, ids, wk_alt, ids_alt, n_t, 8, tscratch, &talt, s));
+        CK(launch_tile_ranges(alt2 ? qkey_alt : qkey, K2, st->ranges2, s));
+        // the tiles with a second segment come first; only they are in the queue
+        CK(launch_tile_order(st->ranges2, nullptr, n_t, ids, qscratch, s, &rb.n_queue));
       }
-      RasterArgs rb = ra;
       rb.ranges = st->ranges2;
       rb.vals = st->vals2;
       rb.prior = st->ranges;
-      rb.tile_order = talt ? ids_alt : ids;
-      rb.n_queue = n_again;
+      rb.queue = queue + 1;
       rb.open = nullptr;
-      CK(cudaMemsetAsync(queue, 0, sizeof(uint32_t), s));
       {
         StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
         CK(launch_raster_forward(rb, tw, th, st->ppt, st->batch, img, s));
       }
     }
-    K = K1 + K2;
-    st->K = K;
-    if (keep_state) {
-      // the backward's work order: longest complete lists first
-      uint32_t *bids, *bids_alt;
-      CK(keep.alloc(&bids, n_t));
-      CK(keep.alloc(&bids_alt, n_t));
-      CK(launch_tile_order(st->ranges, n_t, wk, bids, s, st->ranges2));
-      bool balt = false;
-      CK(radix_sort_pairs(wk, bids, wk_alt, bids_alt, n_t, 8, tscratch, &balt, s));
-      st->tile_order = balt ? bids_alt : bids;
-    }
   }
+  if (keep_state && two_pass)  // the backward's work order: longest complete lists first
+    CK(launch_tile_order(st->ranges, st->ranges2, n_t, st->tile_order, bscratch, s));
+  st->K = K1 + K2;
 
   ctx->stats.n_gaussians = N;
   ctx->stats.n_views = V;
   ctx->stats.n_pixels = pl.P;
-  ctx->stats.n_pairs = K;
+  ctx->stats.n_pairs = st->K;
   ctx->stats.n_tiles = pl.tiles;
   ctx->stats.tile_w = tw;
   ctx->stats.tile_h = th;
@@ -632,35 +581,56 @@ struct SweepWs {
   uint2* ranges = nullptr;
   float4* bin = nullptr;
   uint32_t *dkey = nullptr, *order = nullptr, *dkey_alt = nullptr, *order_alt = nullptr;
-  uint64_t *counts = nullptr, *total = nullptr;
-  uint32_t* n32 = nullptr;
-  char *scratch = nullptr, *pscratch = nullptr, *tscratch = nullptr;
-  uint32_t *pkey = nullptr, *pval = nullptr, *pkey_alt = nullptr, *pval_alt = nullptr;
-  uint32_t *queue = nullptr, *wk = nullptr, *ids = nullptr, *wk_alt = nullptr, *ids_alt = nullptr;
-  float* t_final = nullptr;
-  uint32_t* last = nullptr;
+  uint64_t *unit_base = nullptr, *total = nullptr;
+  uint32_t *n_valid = nullptr, *n32 = nullptr;
+  uint32_t *pkey = nullptr, *pval = nullptr, *pkey_alt = nullptr, *pval_alt = nullptr, *ids = nullptr;
+  // cleared at the start of every chunk: [zero, zero + zero_bytes)
+  char* zero = nullptr;
+  size_t zero_bytes = 0;
+  char *dscratch = nullptr, *pscratch = nullptr, *oscratch = nullptr;
+  uint32_t *queue = nullptr, *done = nullptr;
   uint32_t vn_max = 0, cap = 0;
   int64_t tiles_max = 0;
 };
 
-cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_max, uint32_t cap) {
+cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_max, uint32_t cap, cudaStream_t s) {
   w.vn_max = vn_max;
   w.tiles_max = tiles_max;
   w.cap = cap;
-  cudaError_t e = cudaSuccess;
-#define OCGS_A(ptr, n) if (e == cudaSuccess) e = a.alloc(&(ptr), (size_t)(n))
-  OCGS_A(w.rec.g0, vn_max); OCGS_A(w.rec.g1, vn_max); OCGS_A(w.rec.g2, vn_max);
-  OCGS_A(w.rec.a0, vn_max); OCGS_A(w.rec.a1, vn_max);
-  OCGS_A(w.ntiles, vn_max); OCGS_A(w.ranges, tiles_max); OCGS_A(w.bin, 3 * (size_t)vn_max);
-  OCGS_A(w.dkey, vn_max); OCGS_A(w.order, vn_max); OCGS_A(w.dkey_alt, vn_max); OCGS_A(w.order_alt, vn_max);
-  OCGS_A(w.counts, vn_max); OCGS_A(w.total, 1); OCGS_A(w.n32, 1);
-  OCGS_A(w.scratch, std::max(radix_scratch_bytes(vn_max), scan_scratch_bytes(vn_max)));
-  OCGS_A(w.pkey, cap); OCGS_A(w.pval, cap); OCGS_A(w.pkey_alt, cap); OCGS_A(w.pval_alt, cap);
-  OCGS_A(w.pscratch, radix_scratch_bytes(cap));
-  OCGS_A(w.queue, 1); OCGS_A(w.wk, tiles_max); OCGS_A(w.ids, tiles_max); OCGS_A(w.wk_alt, tiles_max);
-  OCGS_A(w.ids_alt, tiles_max); OCGS_A(w.tscratch, radix_scratch_bytes((uint32_t)tiles_max));
-  OCGS_A(w.t_final, 1); OCGS_A(w.last, 1);
-#undef OCGS_A
+  const int tbits = bits_for((uint64_t)tiles_max);
+  Block b;
+  b.zeroed(&w.dscratch, depth_sort_scratch_bytes(vn_max));
+  // a chunk with fewer tiles may sort fewer bits in fewer passes: any plan up to tbits fits
+  size_t psort = 0;
+  for (int k = 0; k <= tbits; ++k) psort = std::max(psort, radix_scratch_bytes(cap, k));
+  b.zeroed(&w.pscratch, psort);
+  b.zeroed(&w.oscratch, tile_order_scratch_bytes((uint32_t)tiles_max));
+  b.zeroed(&w.queue, 1);
+  b.zeroed(&w.done, 1);
+  b.zeroed(&w.ranges, tiles_max);
+  b.add(&w.rec.g0, vn_max);
+  b.add(&w.rec.g1, vn_max);
+  b.add(&w.rec.g2, vn_max);
+  b.add(&w.rec.a0, vn_max);
+  b.add(&w.rec.a1, vn_max);
+  b.add(&w.ntiles, vn_max);
+  b.add(&w.bin, 3 * (size_t)vn_max);
+  b.add(&w.dkey, vn_max);
+  b.add(&w.order, vn_max);
+  b.add(&w.dkey_alt, vn_max);
+  b.add(&w.order_alt, vn_max);
+  b.add(&w.unit_base, unit_base_words(vn_max));
+  b.add(&w.total, 1);
+  b.add(&w.n_valid, 1);
+  b.add(&w.n32, 1);
+  b.add(&w.pkey, cap);
+  b.add(&w.pval, cap);
+  b.add(&w.pkey_alt, cap);
+  b.add(&w.pval_alt, cap);
+  b.add(&w.ids, tiles_max);
+  const cudaError_t e = b.alloc(a, s);
+  w.zero = w.dscratch;
+  w.zero_bytes = (size_t)(reinterpret_cast<char*>(w.rec.g0) - w.dscratch);
   return e;
 }
 
@@ -672,23 +642,18 @@ ocgs_status enqueue_sweep_chunk(ocgs_ctx* ctx, const ocgs_gaussians* g, int V, c
   const int tw = ctx->opts.tile_w, th = ctx->opts.tile_h, ppt = ctx->opts.pixels_per_thread;
   const int64_t N = g->n;
   const uint32_t VN = (uint32_t)(N * V);
-  CK(cudaMemsetAsync(w.ranges, 0, sizeof(uint2) * n_tiles, s));
+  const int tbits = bits_for((uint64_t)n_tiles);
+  CK(cudaMemsetAsync(w.zero, 0, w.zero_bytes, s));
   CK(launch_preprocess(gptrs(g), N, g->sh_degree, d_cams, V, tw, th, w.rec, w.ntiles, w.bin, w.dkey, ctx->d_status,
                        s));
-  CK(launch_tile_count(w.bin, d_cams, N, VN, tw, th, w.ntiles, w.dkey, s));
-  bool alt = false;
-  CK(radix_sort_pairs(w.dkey, w.order, w.dkey_alt, w.order_alt, VN, 32, w.scratch, &alt, s, nullptr, true));
-  uint32_t* sorted = alt ? w.order_alt : w.order;
-  CK(launch_gather_counts(sorted, w.ntiles, w.counts, VN, s));
-  CK(scan_exclusive_u64(w.counts, w.counts, VN, w.total, w.scratch, s));
-  CK(launch_clamp_count(w.total, w.cap, w.n32, ctx->d_status, s));
-  CK(launch_duplicate(sorted, w.counts, w.total, VN, w.bin, d_cams, N, tw, th, w.cap, w.pkey, w.pval, s));
-  bool palt = false;
-  CK(radix_sort_pairs(w.pkey, w.pval, w.pkey_alt, w.pval_alt, w.cap, bits_for((uint64_t)n_tiles), w.pscratch, &palt,
-                      s, w.n32));
-  uint32_t* skey = palt ? w.pkey_alt : w.pkey;
-  uint32_t* svals = palt ? w.pval_alt : w.pval;
-  CK(launch_tile_ranges(skey, w.cap, w.ranges, s, w.n32));
+  CK(depth_sort(w.dkey, w.dkey_alt, w.order, w.order_alt, VN, w.n_valid, w.dscratch, s));
+  CK(launch_bin_count(w.order, VN, w.n_valid, w.bin, d_cams, N, tw, th, w.unit_base, w.done, w.total, s, w.n32,
+                      w.cap, ctx->d_status));
+  CK(launch_duplicate(w.order, VN, w.n_valid, w.unit_base, w.bin, d_cams, N, tw, th, w.cap, w.pkey, w.pval,
+                      s));
+  CK(radix_sort_pairs(w.pkey, w.pval, w.pkey_alt, w.pval_alt, w.cap, tbits, w.pscratch, s, w.n32));
+  const bool alt = radix_result_in_alt(w.cap, tbits);
+  CK(launch_tile_ranges(alt ? w.pkey_alt : w.pkey, w.cap, w.ranges, s, w.n32));
   RasterArgs ra{};
   ra.cams = d_cams;
   ra.tile_prefix = d_prefix;
@@ -696,17 +661,12 @@ ocgs_status enqueue_sweep_chunk(ocgs_ctx* ctx, const ocgs_gaussians* g, int V, c
   ra.n_gauss = N;
   ra.n_tiles = (uint32_t)n_tiles;
   ra.ranges = w.ranges;
-  ra.vals = svals;
+  ra.vals = alt ? w.pval_alt : w.pval;
   ra.rec = w.rec;
-  ra.t_final = w.t_final;
-  ra.last = w.last;
   ra.score = score;
   if (ctx->opts.persistent) {
-    CK(cudaMemsetAsync(w.queue, 0, sizeof(uint32_t), s));
-    CK(launch_tile_order(w.ranges, (uint32_t)n_tiles, w.wk, w.ids, s));
-    bool talt = false;
-    CK(radix_sort_pairs(w.wk, w.ids, w.wk_alt, w.ids_alt, (uint32_t)n_tiles, 8, w.tscratch, &talt, s));
-    ra.tile_order = talt ? w.ids_alt : w.ids;
+    CK(launch_tile_order(w.ranges, nullptr, (uint32_t)n_tiles, w.ids, w.oscratch, s));
+    ra.tile_order = w.ids;
     ra.queue = w.queue;
     ra.persistent_ctas = ctx->sm_count * (2048 * ppt / (tw * th));
   }
@@ -746,12 +706,13 @@ ocgs_status ocgs_create(ocgs_ctx** out, int32_t device, void* stream) {
   if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) { delete ctx; return OCGS_ERR_CUDA; }
   uint64_t thr = UINT64_MAX;
   cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &thr);
-  if (cudaMalloc(&ctx->d_status, 256) != cudaSuccess || cudaMalloc(&ctx->d_scalar, 256) != cudaSuccess ||
+  if (cudaMalloc(&ctx->d_scalar, 256) != cudaSuccess ||
       cudaHostAlloc(&ctx->h_scalar, 256, cudaHostAllocDefault) != cudaSuccess) {
     ocgs_destroy(ctx);
     return OCGS_ERR_OOM;
   }
-  cudaMemset(ctx->d_status, 0, 256);
+  cudaMemset(ctx->d_scalar, 0, 256);
+  ctx->d_status = reinterpret_cast<int*>(ctx->d_scalar + kScalarStatus);
   *out = ctx;
   return OCGS_OK;
 }
@@ -760,7 +721,6 @@ ocgs_status ocgs_destroy(ocgs_ctx* ctx) {
   if (!ctx) return OCGS_ERR_ARG;
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
-  if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->d_scalar) cudaFree(ctx->d_scalar);
   if (ctx->h_scalar) cudaFreeHost(ctx->h_scalar);
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
@@ -814,7 +774,7 @@ ocgs_status ocgs_sync(ocgs_ctx* ctx) {
   if (!ctx) return OCGS_ERR_ARG;
   CK(cudaSetDevice(ctx->device));
   int status = 0;
-  ocgs_status r = read_status(ctx, &status);
+  ocgs_status r = read_scalars(ctx, &status);
   if (r != OCGS_OK) return r;
   CK(cudaGetLastError());
   if (status & kStatusCapacity)
@@ -837,7 +797,7 @@ ocgs_status ocgs_render(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_camer
   CK(cudaSetDevice(ctx->device));
   if (state) *state = nullptr;
   ocgs_fwd_state* st = new ocgs_fwd_state();
-  r = forward_pass(ctx, g, cams, n_views, out, score, st, true);
+  r = forward_pass(ctx, g, cams, n_views, out, score, st, state != nullptr);
   if (r != OCGS_OK && r != OCGS_ERR_NONFINITE) {
     free_state(st);
     delete st;
@@ -1496,7 +1456,7 @@ extern "C" ocgs_status ocgs_contribution_graph_create(ocgs_ctx* ctx, const ocgs_
   gr->ctx = ctx;
   Arena a(ctx);
   SweepWs w;
-  cudaError_t e = alloc_sweep_ws(a, w, (uint32_t)(g->n * std::min(chunk, n_views)), tiles_max, cap);
+  cudaError_t e = alloc_sweep_ws(a, w, (uint32_t)(g->n * std::min(chunk, n_views)), tiles_max, cap, ctx->stream);
   std::vector<DevCam*> dc(plans.size());
   std::vector<int*> dp(plans.size());
   for (size_t c = 0; c < plans.size() && e == cudaSuccess; ++c) {

@@ -235,29 +235,13 @@ __device__ __forceinline__ void span_tiles(float lo, float hi, int tw, int W, in
   *t1 = min((int)ihi / tw, c1);
 }
 
-// 8-bit log-scale code of a tile's pair count, 16 steps per octave: the
-// persistent queues only need the heaviest tiles roughly first, and one 8-bit
-// radix pass orders them (0 for an empty tile, increasing with the count).
-__device__ __forceinline__ uint32_t work_code(uint32_t len) {
-  const uint32_t x = min(len, 32767u) + 1u;
-  const uint32_t e = 31u - (uint32_t)__clz(x);
-  const uint32_t m = e >= 4u ? (x >> (e - 4u)) & 15u : (x << (4u - e)) & 15u;
-  return e * 16u + m;
-}
-
-#ifndef OCGS_QUEUE_DROP
-#define OCGS_QUEUE_DROP 4
-#endif
-// an empty tile (code 0) must stay behind every non-empty one (codes >= 16)
-static_assert(OCGS_QUEUE_DROP >= 0 && OCGS_QUEUE_DROP <= 4, "queue key bits");
-// Radix key of a tile in a persistent queue: heaviest first.  The low
-// OCGS_QUEUE_DROP bits of the code are dropped (4: whole octaves of the pair
-// count), so that the tiles of one weight class keep their id order (view by
-// view, row by row) and neighbouring tiles, which share records, run close
-// together in time.  On 500k surfels x 16 views this halved the backward's
-// DRAM reads (3.53 -> 1.92 GB per launch) against the exact 8-bit code.
-__device__ __forceinline__ uint32_t queue_key(uint32_t len) {
-  return 255u - (work_code(len) & ~((1u << OCGS_QUEUE_DROP) - 1u));
+// Class of a tile in a persistent queue, by octave of its pair count: heaviest first
+// (0), empty tiles last (15).  The tiles of one class keep their id order (view by view,
+// row by row), so that neighbouring tiles, which share records, run close together in
+// time: on 500k surfels x 16 views this halved the backward's DRAM reads (3.53 -> 1.92 GB
+// per launch) against an order by 16 steps per octave.
+__device__ __forceinline__ uint32_t queue_class(uint32_t len) {
+  return 15u - (31u - (uint32_t)__clz(min(len, 32767u) + 1u));
 }
 
 // Tile runs of one row of a record's candidate rectangle: the union of the
@@ -357,16 +341,20 @@ cudaError_t launch_preprocess_backward(const GaussPtrs& g, int64_t n, int sh_deg
                                        const DevCam* cams, int n_views, const float* grad_rec,
                                        const int32_t* ntiles, GaussOut out, cudaStream_t s);
 
-// stable LSD radix sort of (key, value) 32-bit pairs on key bits [0, n_bits)
-// in ping-pong buffers; returns in *result_in_alt whether the sorted data ended
-// in the alternate buffers.  scratch must hold radix_scratch_bytes(n) bytes.
-size_t radix_scratch_bytes(uint32_t n);
-// d_n (optional): device-side item count, read by the kernels and clamped to n
-// (n sizes the launch: a capacity).  index_vals: the values are 0, 1, ..., n - 1 (the
-// first pass generates them instead of reading vals, which need not be initialised)
-cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                             uint32_t n, int n_bits, void* scratch, bool* result_in_alt,
-                             cudaStream_t s, const uint32_t* d_n = nullptr, bool index_vals = false);
+// Stable LSD radix sort of (key, value) 32-bit pairs on key bits [0, n_bits) in ping-pong
+// buffers; the result is in the alternate ones if radix_result_in_alt.  scratch holds
+// radix_scratch_bytes and is zeroed by the caller.  d_n (optional): device-side item count,
+// read by the kernels and clamped to n (n sizes the launch: a capacity).
+size_t radix_scratch_bytes(uint32_t n, int n_bits);
+bool radix_result_in_alt(uint32_t n, int n_bits);
+cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
+                             int n_bits, void* scratch, cudaStream_t s, const uint32_t* d_n = nullptr);
+// The records in depth order: order[0 .. *n_valid) are the indices of the keys other than
+// 0xffffffff, ascending by key, ties by index.  keys and the alternates are overwritten;
+// scratch holds depth_sort_scratch_bytes and is zeroed by the caller.
+size_t depth_sort_scratch_bytes(uint32_t n);
+cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint32_t* order_alt, uint32_t n,
+                       uint32_t* n_valid, void* scratch, cudaStream_t s);
 
 // exclusive scan of n uint64 values (in may equal out); the total is written to *d_total.
 size_t scan_scratch_bytes(uint32_t n);
@@ -375,62 +363,50 @@ cudaError_t scan_exclusive_u64(const uint64_t* in, uint64_t* out, uint32_t n, ui
 cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* d_total,
                                void* scratch, cudaStream_t s);
 
-cudaError_t launch_gather_counts(const uint32_t* order, const int32_t* ntiles, uint64_t* counts,
-                                 uint32_t n, cudaStream_t s);
-cudaError_t launch_iota(uint32_t* v, uint32_t n, cudaStream_t s);
-// exact tile counts: ntiles[r] = tiles of rect[r] the record's support reaches
-// (row_runs); a record with none gets depth key 0xffffffff so that it sorts to
-// the tail
-cudaError_t launch_tile_count(const float4* bin, const DevCam* cams, int64_t n_gauss, uint32_t n_rec, int tile_w,
-                              int tile_h, int32_t* ntiles, uint32_t* depth_key, cudaStream_t s);
-// write the (tile, record) pairs in depth order: offsets [n_rec] are the
-// exclusive scan of the tile counts taken in depth order (order), total their
-// sum (device); pairs at or past n_pairs are dropped
-cudaError_t launch_duplicate(const uint32_t* order, const uint64_t* offsets, const uint64_t* total, uint32_t n_rec,
+// Binning of the depth order (entries order[0 .. min(n, *d_n))) in work units of consecutive
+// entries.  unit_base [unit_base_words(n)]: first pair of each unit, *total = the pairs (row_runs
+// over every record's candidate rows).  With n32, *n32 = min(*total, cap), and kStatusCapacity is
+// raised in *status when the total exceeds cap.  done: one zeroed word.
+size_t unit_base_words(uint32_t n);
+size_t unit_capacity(uint32_t n);  // at least the units of any m <= n entries
+cudaError_t launch_bin_count(const uint32_t* order, uint32_t n, const uint32_t* d_n, const float4* bin,
+                             const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h, uint64_t* unit_base,
+                             uint32_t* done, uint64_t* total, cudaStream_t s, uint32_t* n32 = nullptr,
+                             uint32_t cap = 0, int* status = nullptr);
+// the (tile, record) pairs in depth order from unit_base; pairs at or past n_pairs are dropped
+cudaError_t launch_duplicate(const uint32_t* order, uint32_t n, const uint32_t* d_n, const uint64_t* unit_base,
                              const float4* bin, const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h,
                              uint32_t n_pairs, uint32_t* keys, uint32_t* vals, cudaStream_t s);
 cudaError_t launch_tile_ranges(const uint32_t* keys, uint32_t n_pairs, uint2* ranges, cudaStream_t s,
                                const uint32_t* d_n = nullptr);
-// n32 = min(*total, cap); raises kStatusCapacity when *total > cap
-cudaError_t launch_clamp_count(const uint64_t* total, uint32_t cap, uint32_t* n32, int* status, cudaStream_t s);
-// Work keys of the persistent queue: heaviest tiles first over all views, by octave
-// of the pair count (queue_key; ranges2: an optional second segment of each tile's
-// list, counted with the first), sorted with one 8-bit radix pass.  A strict
-// view-by-view order left SMs idle at the end of each launch, each view's heavy tiles
-// starting late (backward active warps 15.6 -> 14.6 per SM on a 4-view case).
-cudaError_t launch_tile_order(const uint2* ranges, uint32_t n_tiles, uint32_t* work_key, uint32_t* tile_ids,
-                              cudaStream_t s, const uint2* ranges2 = nullptr);
+// Tiles of the persistent queue: heaviest first over all views, by octave of the pair count
+// (queue_class; ranges2: an optional second segment of each tile's list, counted with the
+// first).  A strict view-by-view order left SMs idle at the end of each launch, each view's
+// heavy tiles starting late (backward active warps 15.6 -> 14.6 per SM on a 4-view case).
+// scratch: zeroed, tile_order_scratch_bytes; *n_nonempty: device count of the tiles with pairs
+// (in scratch), which come first.
+size_t tile_order_scratch_bytes(uint32_t n_tiles);
+cudaError_t launch_tile_order(const uint2* ranges, const uint2* ranges2, uint32_t n_tiles, uint32_t* ids,
+                              void* scratch, cudaStream_t s, const uint32_t** n_nonempty = nullptr);
 
-// Two-pass binning (front records first, then the records behind them into the tiles left open):
-// exact tile counts of the first n entries of the depth order (counts[i], and ntiles[order[i]])
-cudaError_t launch_tile_count_sorted(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
-                                     int64_t n_gauss, int tile_w, int tile_h, int32_t* ntiles, uint64_t* counts,
-                                     cudaStream_t s);
-// *out = number of entries of the ascending sorted_keys[n] below key
-cudaError_t launch_count_below(const uint32_t* sorted_keys, uint32_t n, uint32_t key, uint32_t* out,
-                               cudaStream_t s);
-// Second pass over the n entries behind the front (order: their records in depth order).
-// open_prefix [n_tiles + 1] is the exclusive prefix sum of the 0/1 open flags.
-// Candidates (a screen box holding an open tile), compacted in depth order into
-// cand[*n_cand]; flag and pos are [n] scratch, scratch holds scan_scratch_bytes(n).
-cudaError_t launch_open_candidates(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
-                                   int64_t n_gauss, const uint32_t* open_prefix, uint32_t* flag, uint32_t* pos,
-                                   uint32_t* cand, uint32_t* n_cand, void* scratch, cudaStream_t s);
-// counts[c] = open tiles reached by candidate c (0 for c >= *n_cand; counts is [n])
-cudaError_t launch_open_count(const uint32_t* cand, uint32_t n, const uint32_t* n_cand, const float4* bin,
-                              const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h,
-                              const uint32_t* open_prefix, uint64_t* counts, cudaStream_t s);
-// the (open tile, record) pairs of the candidates, in depth order, from the scan of those counts
-// (open_ids: scratch of n_tiles ids, filled with the compacted open tiles first)
-cudaError_t launch_duplicate_open(const uint32_t* cand, const uint64_t* offsets, const uint64_t* total,
-                                  uint32_t n_rec, const uint32_t* n_cand, const float4* bin, const DevCam* cams,
-                                  int64_t n_gauss, int tile_w, int tile_h, const uint32_t* open,
-                                  const uint32_t* open_prefix, uint32_t n_tiles, uint32_t* open_ids, uint32_t n_pairs,
-                                  uint32_t* keys, uint32_t* vals, cudaStream_t s);
-// the second pass's queue: tiles with a non-empty ranges2 first (longest first);
-// n_again (zeroed by the caller) counts them
-cudaError_t launch_second_queue(const uint2* ranges2, uint32_t n_tiles, uint32_t* work_key, uint32_t* ids,
-                                uint32_t* n_again, cudaStream_t s);
+// Two-pass binning (front records first, then the records behind them into the tiles left open).
+// P [n_tiles + 1]: exclusive prefix of the 0/1 open flags; open_ids: the open tiles, ascending;
+// words: open_scan_words zeroed words.
+size_t open_scan_words(uint32_t n_tiles);
+cudaError_t launch_open_scan(const uint32_t* open, uint32_t n_tiles, uint32_t* P, uint32_t* open_ids, uint32_t* words,
+                             cudaStream_t s);
+// Second pass over the n entries behind the front (order: their records in depth order): each
+// unit's candidates (a screen box holding an open tile) with their open tiles, in the unit's own
+// stretch of cand and counts [n]; n_cand [unit_capacity(n)]; unit_base, total and done as above.
+cudaError_t launch_open_count(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
+                              int64_t n_gauss, int tile_w, int tile_h, const uint32_t* P, uint32_t* cand,
+                              uint32_t* counts, uint32_t* n_cand, uint64_t* unit_base, uint32_t* done,
+                              uint64_t* total, cudaStream_t s);
+// the (open tile, record) pairs of the candidates, in depth order
+cudaError_t launch_duplicate_open(const uint32_t* cand, uint32_t n, const uint32_t* counts, const uint32_t* n_cand,
+                                  const uint64_t* unit_base, const float4* bin, const DevCam* cams, int64_t n_gauss,
+                                  int tile_w, int tile_h, const uint32_t* open_ids, const uint32_t* P,
+                                  uint32_t n_pairs, uint32_t* keys, uint32_t* vals, cudaStream_t s);
 
 struct RasterArgs {
   int ewa;  // records are projected 3D Gaussians (preprocess_ewa)

@@ -286,10 +286,9 @@ __global__ void __launch_bounds__(kBlockWarps * 32, (!IMG ? OCGS_SWEEP_WARPS : Q
           a.out.normal[3 * pix + 0] = lane2(n0[p], i);
           a.out.normal[3 * pix + 1] = lane2(n1[p], i);
           a.out.normal[3 * pix + 2] = lane2(n2[p], i);
-          if (a.t_final) {  // the backward's state, when the pass keeps it
-            a.t_final[pix] = Tk;
-            a.last[pix] = last[k];
-          }
+          // the state of the backward, or (T alone) of a second pass, when the pass keeps it
+          if (a.t_final) a.t_final[pix] = Tk;
+          if (a.last) a.last[pix] = last[k];
           if (a.open) a.done[pix] = done[k] ? 1 : 0;
         }
       }

@@ -1,6 +1,6 @@
-// Tile binning: device-wide scans, the stable LSD radix sort of 32-bit keys,
-// duplication of each visible (view, Gaussian) record into its tiles and the
-// per-tile [start, end) ranges.
+// Tile binning: the stable LSD radix sort of 32-bit keys, duplication of each
+// visible (view, Gaussian) record into its tiles and the per-tile [start, end)
+// ranges.
 //
 // Order of the (tile, Gaussian) list (the front-to-back order of Sec. 4.3):
 // records are first sorted by centre depth (stable, so equal depths keep the
@@ -180,11 +180,11 @@ struct QueueKeys {
       const uint2 q = ranges2[i];
       len += q.y - q.x;
     }
-    return queue_key(len);
+    return queue_class(len);
   }
 };
 
-// Exclusive scan of kPer values per thread over a block of kRadixThreads; returns
+// Exclusive scan of PER values per thread over a block of kRadixThreads; returns
 // this thread's first prefix.  s_w: one word per warp, free to reuse after a barrier.
 template <int PER>
 __device__ __forceinline__ uint32_t block_exclusive(const uint32_t (&v)[PER], uint32_t* s_w) {
@@ -448,21 +448,7 @@ __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel
 }
 
 // ------------------------------------------------------------------ binning helpers
-__global__ void gather_counts_kernel(const uint32_t* __restrict__ order, const int32_t* __restrict__ ntiles,
-                                     uint64_t* __restrict__ counts, uint32_t n) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) counts[i] = (uint64_t)ntiles[order[i]];
-}
-
-__global__ void iota_kernel(uint32_t* v, uint32_t n) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = i;
-}
-
 constexpr int kThreads = 256;
-// a record with at most this many candidate rows is a small one: its row runs are
-// kept in shared memory and its tiles written in the warp-flat list
-constexpr int kSmallRows = 16;
 
 __device__ __forceinline__ int row_count(const RowRuns& rr) {
   return max(0, rr.a1 - rr.a0 + 1) + max(0, rr.b1 - rr.b0 + 1);
@@ -476,9 +462,10 @@ struct RowOwner {
   int tile_offset, tiles_x, W, H;
 };
 
-// The candidate tile rows of the warp's 32 records, flattened over the lanes:
-// f(ri, ty) runs once for every row ty of record ri, 32 rows at a time, so
-// records with many rows no longer leave the lanes of small ones idle.
+// The candidate tile rows of the warp's 32 records, flattened over the lanes: f(ri, ty) runs
+// for 32 rows at a time, row ty of record ri, in record order and within a record from top to
+// bottom, so records with many rows do not leave the lanes of small ones idle.  Every lane
+// calls f (it may use warp collectives); ri is -1 for a lane without a row.
 // nrows: the rows of this lane's record (0 for none); s_own[lane] must hold it.
 template <class F>
 __device__ __forceinline__ void for_warp_rows(int nrows, int lane, int* s_incl, const RowOwner* s_own, F f) {
@@ -488,191 +475,227 @@ __device__ __forceinline__ void for_warp_rows(int nrows, int lane, int* s_incl, 
   __syncwarp();
   for (int q0 = 0; q0 < total; q0 += 32) {
     const int q = q0 + lane;
+    int ri = -1, ty = 0;
     if (q < total) {
       int lo = 0, hi = 31;
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (s_incl[mid] > q) hi = mid; else lo = mid + 1;
       }
-      const int excl = lo > 0 ? s_incl[lo - 1] : 0;
-      f(lo, s_own[lo].rc.y + (q - excl));
+      ri = lo;
+      ty = s_own[lo].rc.y + (q - (lo > 0 ? s_incl[lo - 1] : 0));
     }
+    f(ri, ty);
   }
   __syncwarp();
 }
 
-// Exact tile count of each record: one closed-form coverage computation per
-// candidate tile row, the rows of a warp's 32 records spread over its lanes.
-__global__ void __launch_bounds__(kThreads) tile_count_kernel(const float4* __restrict__ bin,
-                                                              const DevCam* __restrict__ cams, int64_t n_gauss,
-                                                              uint32_t n_rec, int tw, int th,
-                                                              int32_t* __restrict__ ntiles,
-                                                              uint32_t* __restrict__ depth_key) {
-  __shared__ RowOwner s_own[kThreads / 32][32];
-  __shared__ int s_incl[kThreads / 32][32], s_cnt[kThreads / 32][32];
+// Work units of the binning: runs of per_unit consecutive entries of the depth order, one
+// warp each.  The counting kernel leaves every unit's first pair position and the writing
+// kernel walks the same units with a running position: no scan over the entries, no 64-bit
+// offset per entry.  Units are small (the entries nearest to the cameras reach hundreds of
+// tiles each: 128 entries per unit instead of 32 made the binning of 500k surfels x 16 views
+// 12 % slower), so their totals are scanned in two levels.
+constexpr uint32_t kMaxUnits = 65536;
+constexpr int kUnitWarps = kThreads / 32;  // units per counting block
+
+// base [units + blocks]: each unit's first position within its counting block, then (from
+// units on) each block's first position; first position of a unit = the sum of both.  The last
+// block to finish scans the blocks' totals and writes their sum to *total (and, with n32,
+// its clamp to cap, raising the capacity bit of *status where it does not fit).
+struct UnitTotals {
+  uint64_t* base;
+  uint32_t* done;   // zeroed
+  uint64_t* total;
+  uint32_t* n32;
+  uint32_t cap;
+  int* status;
+};
+
+__device__ __forceinline__ uint64_t unit_start(const uint64_t* __restrict__ base, uint32_t units, uint32_t unit) {
+  return base[unit] + base[units + unit / kUnitWarps];
+}
+
+// sum: this lane's share of its warp's unit (0 for a warp without one); all threads of the block
+__device__ __forceinline__ void finish_units(const UnitTotals& t, uint32_t units, uint64_t sum) {
+  __shared__ uint64_t s_w[kUnitWarps];
+  __shared__ bool s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t r = blockIdx.x * kThreads + threadIdx.x;
-  int nrows = 0;
-  if (r < n_rec) {
-    const BinView b = load_bin(bin, r);
-    if (b.rc.z >= b.rc.x) {
-      const DevCam& cam = cams[view_of_record(r, n_gauss)];
-      s_own[warp][lane] = RowOwner{support_conic(b.g0, b.g1, b.g2, b.rb), b.rc, cam.tile_offset, cam.tiles_x,
-                                   cam.W, cam.H};
-      nrows = b.rc.w - b.rc.y + 1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+  if (lane == 0) s_w[warp] = sum;
+  __syncthreads();
+  const uint32_t unit = blockIdx.x * kUnitWarps + threadIdx.x;
+  if (threadIdx.x < kUnitWarps && unit < units) {
+    uint64_t e = 0;
+    for (int w = 0; w < (int)threadIdx.x; ++w) e += s_w[w];
+    t.base[unit] = e;
+  }
+  if (threadIdx.x == 0) {
+    uint64_t c = 0;
+    for (int w = 0; w < kUnitWarps; ++w) c += s_w[w];
+    t.base[units + blockIdx.x] = c;
+    __threadfence();
+    s_last = atomicAdd(t.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  uint64_t* blocks = t.base + units;
+  const uint32_t per = (gridDim.x + kThreads - 1) / kThreads;
+  const uint32_t b0 = min(gridDim.x, threadIdx.x * per), b1 = min(gridDim.x, b0 + per);
+  uint64_t mine = 0;
+#pragma unroll 8
+  for (uint32_t b = b0; b < b1; ++b) mine += __ldcg(blocks + b);
+  const uint64_t inc = warp_inclusive_scan<uint64_t>(mine, lane);
+  if (lane == 31) s_w[warp] = inc;
+  __syncthreads();
+  uint64_t run = inc - mine;
+  for (int w = 0; w < warp; ++w) run += s_w[w];
+#pragma unroll 8
+  for (uint32_t b = b0; b < b1; ++b) {
+    const uint64_t c = __ldcg(blocks + b);
+    blocks[b] = run;
+    run += c;
+  }
+  if (threadIdx.x == kThreads - 1) {
+    *t.total = run;
+    if (t.n32) {
+      *t.n32 = (uint32_t)min(run, (uint64_t)t.cap);
+      if (run > (uint64_t)t.cap) atomicOr(t.status, kStatusCapacity);
     }
   }
-  s_cnt[warp][lane] = 0;
-  // the rows of the warp's records, spread over the lanes
-  for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
-    const RowOwner& o = s_own[warp][ri];
-    const int c = row_count(row_runs(o.k, ty, tw, th, o.W, o.H, o.rc));
-    if (c) atomicAdd(&s_cnt[warp][ri], c);
-  });
-  if (r < n_rec) {
-    const int cnt = s_cnt[warp][lane];
-    ntiles[r] = cnt;
-    if (cnt == 0) depth_key[r] = 0xffffffffu;
+}
+
+// This lane's record of a round of 32 entries: publishes it in s_own and returns its
+// candidate rows (0 without a screen box).
+__device__ __forceinline__ int publish_record(uint32_t r, const float4* __restrict__ bin,
+                                              const DevCam* __restrict__ cams, int64_t n_gauss, RowOwner* own) {
+  const BinView b = load_bin(bin, r);
+  if (b.rc.z < b.rc.x) return 0;
+  const DevCam& cam = cams[view_of_record(r, n_gauss)];
+  *own = RowOwner{support_conic(b.g0, b.g1, b.g2, b.rb), b.rc, cam.tile_offset, cam.tiles_x, cam.W, cam.H};
+  return b.rc.w - b.rc.y + 1;
+}
+
+// Pairs of the first n entries of the depth order (at most *d_n, the valid ones): one
+// closed-form coverage computation per candidate tile row, the rows of a warp's 32 records
+// spread over its lanes.
+__global__ void __launch_bounds__(kThreads) bin_count_kernel(const uint32_t* __restrict__ order, uint32_t n,
+                                                             const uint32_t* __restrict__ d_n, uint32_t per_unit,
+                                                             uint32_t units, const float4* __restrict__ bin,
+                                                             const DevCam* __restrict__ cams, int64_t n_gauss, int tw,
+                                                             int th, const UnitTotals totals) {
+  __shared__ RowOwner s_own[kUnitWarps][32];
+  __shared__ int s_incl[kUnitWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t unit = blockIdx.x * kUnitWarps + warp;
+  n = min(n, *d_n);
+  uint64_t sum = 0;
+  if (unit < units) {
+    for (uint32_t k = 0; k < per_unit; k += 32) {
+      const uint64_t i = (uint64_t)unit * per_unit + k + lane;
+      if (__all_sync(kFull, i >= n)) break;
+      const int nrows = i < n ? publish_record(order[i], bin, cams, n_gauss, &s_own[warp][lane]) : 0;
+      for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
+        if (ri < 0) return;
+        const RowOwner& o = s_own[warp][ri];
+        sum += (uint64_t)row_count(row_runs(o.k, ty, tw, th, o.W, o.H, o.rc));
+      });
+    }
+  }
+  finish_units(totals, units, sum);
+}
+
+// A row's pairs are written by its own lane where there are few of them, by the whole warp
+// above this many.
+constexpr int kLongRow = 24;
+
+// Two runs of consecutive values: x_j = a + j for j < la, b + j for la <= j < c.
+struct RowItems {
+  int la, c;
+  uint32_t a, b;
+};
+__device__ __forceinline__ RowItems row_items(uint32_t a, int la, uint32_t b, int lb) {
+  return RowItems{la, la + lb, a, b - (uint32_t)la};
+}
+
+// Writes the pairs of one row per lane, (tile(x_j), r) for its c items, from pos on; pairs at
+// or past n_pairs are dropped.  Consecutive lanes' pairs are adjacent, so the stores of a
+// warp fall into a few neighbouring lines.
+template <class T>
+__device__ __forceinline__ void write_rows(const RowItems& it, uint64_t pos, uint32_t r, uint32_t n_pairs, int lane,
+                                           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, T tile) {
+  const bool is_long = it.c > kLongRow;
+  if (!is_long) {
+    for (int j = 0; j < it.c; ++j)
+      if (pos + (uint64_t)j < (uint64_t)n_pairs) {
+        keys[pos + j] = tile((j < it.la ? it.a : it.b) + (uint32_t)j);
+        vals[pos + j] = r;
+      }
+  }
+  unsigned left = __ballot_sync(kFull, is_long);
+  while (left) {
+    const int src = __ffs(left) - 1;
+    left &= left - 1u;
+    const RowItems o{__shfl_sync(kFull, it.la, src), __shfl_sync(kFull, it.c, src), __shfl_sync(kFull, it.a, src),
+                     __shfl_sync(kFull, it.b, src)};
+    const uint64_t p = __shfl_sync(kFull, pos, src);
+    const uint32_t rr = __shfl_sync(kFull, r, src);
+    for (int j = lane; j < o.c; j += 32)
+      if (p + (uint64_t)j < (uint64_t)n_pairs) {
+        keys[p + j] = tile((j < o.la ? o.a : o.b) + (uint32_t)j);
+        vals[p + j] = rr;
+      }
   }
 }
 
-__device__ __forceinline__ uint64_t write_runs(const RowRuns& rr, uint32_t rowbase, uint32_t r, uint64_t pos,
-                                               uint64_t stop, uint32_t* __restrict__ keys,
-                                               uint32_t* __restrict__ vals) {
-  for (int tx = rr.a0; tx <= rr.a1; ++tx, ++pos)
-    if (pos < stop) { keys[pos] = rowbase + tx; vals[pos] = r; }
-  for (int tx = rr.b0; tx <= rr.b1; ++tx, ++pos)
-    if (pos < stop) { keys[pos] = rowbase + tx; vals[pos] = r; }
-  return pos;
-}
-
-// The (tile, record) pairs, written in depth order: entry i of the depth
-// order (record order[i]) writes its tiles from offsets[i] on, rows in order
-// and tiles left to right, so the runs of consecutive entries are adjacent and
-// a warp's stores are contiguous.  The row runs of the entries that span few
-// rows are computed with those rows spread over the warp; the warp then writes
-// all those entries' tiles as one flat list, 32 consecutive slots per step.  The
-// rows of an entry with many rows are shared out over the warp, with a warp scan
-// of the row counts.
-constexpr int kDupThreads = 128;
-constexpr int kWarpsPerBlock = kDupThreads / 32;
+// The (tile, record) pairs in depth order, entry by entry, rows in order and tiles left to
+// right.  The rows of a warp's 32 records come 32 at a time in exactly that order, so a warp
+// scan of their tile counts gives every row its position and each lane writes its row: no
+// per-entry counts, no search for a pair's row.  What bounds it: the row coverage (ALU) and
+// the scattered stores.  500k surfels x 16 views, 18.6 M pairs: 231 -> 118 us against a
+// search for every pair's entry and row.
+constexpr int kDupThreads = 256;
+constexpr int kDupWarps = kDupThreads / 32;
 
 __global__ void __launch_bounds__(kDupThreads) duplicate_kernel(
-    const uint32_t* __restrict__ order, const uint64_t* __restrict__ offsets, const uint64_t* __restrict__ total,
-    uint32_t n_rec, const float4* __restrict__ bin, const DevCam* __restrict__ cams, int64_t n_gauss, int tw, int th,
-    uint32_t n_pairs, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  __shared__ short4 s_runs[kWarpsPerBlock][kSmallRows][32];  // [row][lane]: lanes in distinct banks
-  __shared__ int s_incl[kWarpsPerBlock][32];
-  __shared__ uint32_t s_rowbase[kWarpsPerBlock][32];  // tile id of (first row, column 0)
-  __shared__ uint32_t s_tilesx[kWarpsPerBlock][32];
-  __shared__ uint32_t s_pos[kWarpsPerBlock][32];
-  __shared__ uint32_t s_rec[kWarpsPerBlock][32];
-  __shared__ RowOwner s_own[kWarpsPerBlock][32];
+    const uint32_t* __restrict__ order, uint32_t n, const uint32_t* __restrict__ d_n, uint32_t per_unit,
+    uint32_t units, const uint64_t* __restrict__ unit_base, const float4* __restrict__ bin,
+    const DevCam* __restrict__ cams, int64_t n_gauss, int tw, int th, uint32_t n_pairs, uint32_t* __restrict__ keys,
+    uint32_t* __restrict__ vals) {
+  __shared__ RowOwner s_own[kDupWarps][32];
+  __shared__ int s_incl[kDupWarps][32];
+  __shared__ uint32_t s_rec[kDupWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t i = blockIdx.x * kDupThreads + threadIdx.x;
-  uint32_t r = 0;
-  int cnt = 0;
-  BinView bv;
-  bv.rc = make_int4(0, 0, -1, -1);
-  uint64_t o = 0;
-  if (i < n_rec) {
-    o = offsets[i];
-    r = order[i];
-  }
-  // this entry's count: the next entry's offset (or the total) minus its own
-  uint64_t o_next = __shfl_down_sync(kFull, o, 1);
-  if (lane == 31 || i + 1 >= n_rec) o_next = (i + 1 < n_rec) ? offsets[i + 1] : *total;
-  if (i < n_rec && o < (uint64_t)n_pairs) {  // entries past a capacity write nothing
-    cnt = (int)(o_next - o);
-    if (cnt > 0) bv = load_bin(bin, r);
-  }
-  const int4 rc = bv.rc;
-  const bool small = cnt > 0 && (rc.w - rc.y + 1) <= kSmallRows;
-  if (small) {
-    const DevCam& cam = cams[view_of_record(r, n_gauss)];
-    s_own[warp][lane] = RowOwner{support_conic(bv.g0, bv.g1, bv.g2, bv.rb), rc, cam.tile_offset, cam.tiles_x, cam.W,
-                                 cam.H};
-    s_rowbase[warp][lane] = (uint32_t)(cam.tile_offset + rc.y * cam.tiles_x);
-    s_tilesx[warp][lane] = (uint32_t)cam.tiles_x;
-    s_pos[warp][lane] = (uint32_t)o;
-    s_rec[warp][lane] = r;
-  }
-  // the row runs of the small entries, the rows spread over the warp
-  for_warp_rows(small ? rc.w - rc.y + 1 : 0, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
-    const RowOwner& ow = s_own[warp][ri];
-    const RowRuns rr = row_runs(ow.k, ty, tw, th, ow.W, ow.H, ow.rc);
-    s_runs[warp][ty - ow.rc.y][ri] = make_short4((short)rr.a0, (short)rr.a1, (short)rr.b0, (short)rr.b1);
-  });
-  // flat walk over the small entries' tiles
-  const int scnt = small ? cnt : 0;
-  int incl = scnt;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int t = __shfl_up_sync(kFull, incl, d);
-    if (lane >= d) incl += t;
-  }
-  s_incl[warp][lane] = incl;
-  const int all = __shfl_sync(kFull, incl, 31);
-  __syncwarp();
-  for (int q0 = 0; q0 < all; q0 += 32) {
-    const int q = q0 + lane;
-    if (q < all) {
-      int lo = 0, hi = 31;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s_incl[warp][mid] > q) hi = mid; else lo = mid + 1;
-      }
-      const int ri = lo;
-      const int excl = ri > 0 ? s_incl[warp][ri - 1] : 0;  // tiles of the warp's earlier small entries
-      int kth = q - excl;
-      int tx = -1, row = 0;
-      for (; row < kSmallRows; ++row) {
-        const short4 ru = s_runs[warp][row][ri];
-        const int la = max(0, (int)ru.y - (int)ru.x + 1), lb = max(0, (int)ru.w - (int)ru.z + 1);
-        if (kth < la) { tx = ru.x + kth; break; }
-        kth -= la;
-        if (kth < lb) { tx = ru.z + kth; break; }
-        kth -= lb;
-      }
-      const uint32_t pos = s_pos[warp][ri] + (uint32_t)(q - excl);
-      if (tx >= 0 && pos < n_pairs) {
-        keys[pos] = s_rowbase[warp][ri] + (uint32_t)row * s_tilesx[warp][ri] + (uint32_t)tx;
-        vals[pos] = s_rec[warp][ri];
-      }
+  const uint32_t unit = blockIdx.x * kDupWarps + warp;
+  if (unit >= units) return;
+  n = min(n, *d_n);
+  uint64_t run = unit_start(unit_base, units, unit);
+  for (uint32_t k = 0; k < per_unit; k += 32) {
+    const uint64_t i = (uint64_t)unit * per_unit + k + lane;
+    if (__all_sync(kFull, i >= n) || run >= (uint64_t)n_pairs) break;
+    int nrows = 0;
+    if (i < n) {
+      const uint32_t r = order[i];
+      s_rec[warp][lane] = r;
+      nrows = publish_record(r, bin, cams, n_gauss, &s_own[warp][lane]);
     }
-  }
-  unsigned big = __ballot_sync(kFull, cnt > 0 && !small);
-  while (big) {
-    const int src = __ffs(big) - 1;
-    big &= big - 1u;
-    const uint32_t rr = __shfl_sync(kFull, r, src);
-    const uint64_t oo = __shfl_sync(kFull, o, src);
-    const int bcnt = __shfl_sync(kFull, cnt, src);
-    const BinView bb = load_bin(bin, rr);
-    const int4 bc = bb.rc;
-    const DevCam& cam = cams[view_of_record(rr, n_gauss)];
-    const SupportConic k = support_conic(bb.g0, bb.g1, bb.g2, bb.rb);
-    const uint64_t stop = min(oo + (uint64_t)bcnt, (uint64_t)n_pairs);
-    uint64_t base = oo;
-    for (int row0 = bc.y; row0 <= bc.w; row0 += 32) {
-      const int ty = row0 + lane;
-      RowRuns runs{1, 0, 1, 0};
-      int c = 0;
-      if (ty <= bc.w) {
-        runs = row_runs(k, ty, tw, th, cam.W, cam.H, bc);
-        c = row_count(runs);
+    for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
+      RowRuns rr{1, 0, 1, 0};
+      uint32_t rowbase = 0, r = 0;
+      if (ri >= 0) {
+        const RowOwner& o = s_own[warp][ri];
+        rr = row_runs(o.k, ty, tw, th, o.W, o.H, o.rc);
+        rowbase = (uint32_t)(o.tile_offset + ty * o.tiles_x);
+        r = s_rec[warp][ri];
       }
-      int inc = c;
-#pragma unroll
-      for (int s2 = 1; s2 < 32; s2 <<= 1) {
-        const int t = __shfl_up_sync(kFull, inc, s2);
-        if (lane >= s2) inc += t;
-      }
-      if (c > 0)
-        write_runs(runs, (uint32_t)(cam.tile_offset + ty * cam.tiles_x), rr, base + (uint64_t)(inc - c), stop, keys,
-                   vals);
-      base += (uint64_t)__shfl_sync(kFull, inc, 31);
-    }
+      const RowItems it = row_items(rowbase + (uint32_t)rr.a0, max(0, rr.a1 - rr.a0 + 1), rowbase + (uint32_t)rr.b0,
+                                    max(0, rr.b1 - rr.b0 + 1));
+      const int inc = warp_inclusive_scan<int>(it.c, lane);
+      write_rows(it, run + (uint64_t)(inc - it.c), r, n_pairs, lane, keys, vals, [](uint32_t x) { return x; });
+      run += (uint64_t)__shfl_sync(kFull, inc, 31);
+    });
   }
 }
 
@@ -711,19 +734,6 @@ __global__ void tile_ranges_kernel(const uint32_t* __restrict__ keys, uint32_t n
   }
 }
 
-// work key for the persistent queue: heaviest tiles first (descending log-scale
-// pair count, one 8-bit radix pass)
-__global__ void tile_work_kernel(const uint2* __restrict__ ranges, const uint2* __restrict__ ranges2, uint32_t n,
-                                 uint32_t* __restrict__ work_key, uint32_t* __restrict__ ids) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const uint2 r = ranges[t];
-  uint32_t len = r.y - r.x;
-  if (ranges2) len += ranges2[t].y - ranges2[t].x;
-  work_key[t] = queue_key(len);
-  ids[t] = t;
-}
-
 }  // namespace
 
 size_t scan_scratch_bytes(uint32_t n) { return scan_levels_bytes<uint64_t>(n) + 256; }
@@ -740,7 +750,7 @@ cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, uint32_t n, ui
 
 namespace {
 
-// Scratch of one sort, zeroed by one memset: digit positions, counters, look-back words.
+// Scratch of one sort (zeroed by the caller): digit positions, counters, look-back words.
 struct RadixScratch {
   uint32_t *base, *done, *next_tile, *words;
   size_t tiles, bytes;
@@ -777,16 +787,12 @@ cudaError_t launch_pass(const Keys& k, const uint32_t* vals, uint32_t* keys_out,
 
 template <int BITS, int PASSES>
 cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
-                        void* scratch, cudaStream_t s, const uint32_t* d_n, bool index_vals) {
+                        void* scratch, cudaStream_t s, const uint32_t* d_n) {
   const RadixScratch w = radix_layout(scratch, n, PASSES, BITS);
-  cudaError_t e = cudaMemsetAsync(scratch, 0, w.bytes, s);
-  if (e != cudaSuccess) return e;
-  e = launch_hist<ArrayKeys, BITS, PASSES, false>(ArrayKeys{keys}, n, d_n, w, nullptr, s);
+  cudaError_t e = launch_hist<ArrayKeys, BITS, PASSES, false>(ArrayKeys{keys}, n, d_n, w, nullptr, s);
   uint32_t *kin = keys, *vin = vals, *kout = keys_alt, *vout = vals_alt;
   for (int p = 0; p < PASSES && e == cudaSuccess; ++p) {
-    e = p == 0 && index_vals
-            ? launch_pass<ArrayKeys, BITS, true, false, true>(ArrayKeys{kin}, nullptr, kout, vout, n, d_n, p, w, s)
-            : launch_pass<ArrayKeys, BITS, false, false, true>(ArrayKeys{kin}, vin, kout, vout, n, d_n, p, w, s);
+    e = launch_pass<ArrayKeys, BITS, false, false, true>(ArrayKeys{kin}, vin, kout, vout, n, d_n, p, w, s);
     std::swap(kin, kout);
     std::swap(vin, vout);
   }
@@ -795,23 +801,22 @@ cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint
 
 }  // namespace
 
-size_t radix_scratch_bytes(uint32_t n) {
-  return radix_layout(nullptr, n, 4, kMaxDigit).bytes;  // the largest of any digit plan
+size_t radix_scratch_bytes(uint32_t n, int n_bits) {
+  if (n <= 1 || n_bits <= 0) return 16;
+  const DigitPlan pl = digit_plan(n_bits);
+  return radix_layout(nullptr, n, pl.passes, pl.bits).bytes;
 }
 
-cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                             uint32_t n, int n_bits, void* scratch, bool* result_in_alt, cudaStream_t s,
-                             const uint32_t* d_n, bool index_vals) {
-  *result_in_alt = false;
-  if (n <= 1 || n_bits <= 0) {
-    if (index_vals && n > 0) return launch_iota(vals, n, s);  // nothing to sort: the values are the indices
-    return cudaSuccess;
-  }
+bool radix_result_in_alt(uint32_t n, int n_bits) {
+  return n > 1 && n_bits > 0 && digit_plan(n_bits).passes % 2 != 0;
+}
+
+cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
+                             int n_bits, void* scratch, cudaStream_t s, const uint32_t* d_n) {
+  if (n <= 1 || n_bits <= 0) return cudaSuccess;
   const DigitPlan pl = digit_plan(n_bits);
-  *result_in_alt = pl.passes % 2 != 0;
 #define OCGS_SORT(B, P) \
-  if (pl.bits == B && pl.passes == P) \
-    return sort_passes<B, P>(keys, vals, keys_alt, vals_alt, n, scratch, s, d_n, index_vals);
+  if (pl.bits == B && pl.passes == P) return sort_passes<B, P>(keys, vals, keys_alt, vals_alt, n, scratch, s, d_n);
   OCGS_SORT(4, 1) OCGS_SORT(5, 1) OCGS_SORT(6, 1) OCGS_SORT(7, 1) OCGS_SORT(8, 1)
   OCGS_SORT(5, 2) OCGS_SORT(6, 2) OCGS_SORT(7, 2) OCGS_SORT(8, 2)
   OCGS_SORT(6, 3) OCGS_SORT(7, 3) OCGS_SORT(8, 3) OCGS_SORT(8, 4)
@@ -819,34 +824,36 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gather_counts(const uint32_t* order, const int32_t* ntiles, uint64_t* counts,
-                                 uint32_t n, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  gather_counts_kernel<<<(n + 255) / 256, 256, 0, s>>>(order, ntiles, counts, n);
-  return launched();
+size_t depth_sort_scratch_bytes(uint32_t n) { return radix_layout(nullptr, n, 4, 8).bytes; }
+
+cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint32_t* order_alt, uint32_t n,
+                       uint32_t* n_valid, void* scratch, cudaStream_t s) {
+  if (n == 0) return cudaMemsetAsync(n_valid, 0, sizeof(uint32_t), s);
+  const RadixScratch w = radix_layout(scratch, n, 4, 8);
+  cudaError_t e = launch_hist<ArrayKeys, 8, 4, true>(ArrayKeys{keys}, n, nullptr, w, n_valid, s);
+  if (e == cudaSuccess)  // the first pass makes the indices and leaves the culled records out
+    e = launch_pass<ArrayKeys, 8, true, true, true>(ArrayKeys{keys}, nullptr, keys_alt, order_alt, n, nullptr, 0, w, s);
+  if (e == cudaSuccess)
+    e = launch_pass<ArrayKeys, 8, false, false, true>(ArrayKeys{keys_alt}, order_alt, keys, order, n, n_valid, 1, w, s);
+  if (e == cudaSuccess)
+    e = launch_pass<ArrayKeys, 8, false, false, true>(ArrayKeys{keys}, order, keys_alt, order_alt, n, n_valid, 2, w, s);
+  if (e == cudaSuccess)
+    e = launch_pass<ArrayKeys, 8, false, false, false>(ArrayKeys{keys_alt}, order_alt, nullptr, order, n, n_valid, 3,
+                                                       w, s);
+  return e;
 }
 
-cudaError_t launch_iota(uint32_t* v, uint32_t n, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  iota_kernel<<<(n + 255) / 256, 256, 0, s>>>(v, n);
-  return launched();
-}
+size_t tile_order_scratch_bytes(uint32_t n_tiles) { return radix_layout(nullptr, n_tiles, 1, 4).bytes; }
 
-cudaError_t launch_tile_count(const float4* bin, const DevCam* cams, int64_t n_gauss, uint32_t n_rec, int tile_w,
-                              int tile_h, int32_t* ntiles, uint32_t* depth_key, cudaStream_t s) {
-  if (n_rec == 0) return cudaSuccess;
-  tile_count_kernel<<<(n_rec + kThreads - 1) / kThreads, kThreads, 0, s>>>(bin, cams, n_gauss, n_rec, tile_w, tile_h,
-                                                                           ntiles, depth_key);
-  return launched();
-}
-
-cudaError_t launch_duplicate(const uint32_t* order, const uint64_t* offsets, const uint64_t* total, uint32_t n_rec,
-                             const float4* bin, const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h,
-                             uint32_t n_pairs, uint32_t* keys, uint32_t* vals, cudaStream_t s) {
-  if (n_pairs == 0 || n_rec == 0) return cudaSuccess;
-  duplicate_kernel<<<(n_rec + kDupThreads - 1) / kDupThreads, kDupThreads, 0, s>>>(
-      order, offsets, total, n_rec, bin, cams, n_gauss, tile_w, tile_h, n_pairs, keys, vals);
-  return launched();
+cudaError_t launch_tile_order(const uint2* ranges, const uint2* ranges2, uint32_t n_tiles, uint32_t* ids,
+                              void* scratch, cudaStream_t s, const uint32_t** n_nonempty) {
+  const RadixScratch w = radix_layout(scratch, n_tiles, 1, 4);
+  if (n_nonempty) *n_nonempty = w.base + 15;  // first position of the empty tiles' class
+  if (n_tiles == 0) return cudaSuccess;
+  const QueueKeys k{ranges, ranges2};
+  const cudaError_t e = launch_hist<QueueKeys, 4, 1, false>(k, n_tiles, nullptr, w, nullptr, s);
+  if (e != cudaSuccess) return e;
+  return launch_pass<QueueKeys, 4, true, false, false>(k, nullptr, nullptr, ids, n_tiles, nullptr, 0, w, s);
 }
 
 cudaError_t launch_tile_ranges(const uint32_t* keys, uint32_t n_pairs, uint2* ranges, cudaStream_t s,
@@ -854,30 +861,6 @@ cudaError_t launch_tile_ranges(const uint32_t* keys, uint32_t n_pairs, uint2* ra
   if (n_pairs == 0) return cudaSuccess;
   const uint32_t blocks = (n_pairs / 4 + 256) / 256;
   tile_ranges_kernel<<<blocks < 152u * 16u ? blocks : 152u * 16u, 256, 0, s>>>(keys, n_pairs, ranges, d_n);
-  return launched();
-}
-
-cudaError_t launch_tile_order(const uint2* ranges, uint32_t n_tiles, uint32_t* work_key, uint32_t* tile_ids,
-                              cudaStream_t s, const uint2* ranges2) {
-  if (n_tiles == 0) return cudaSuccess;
-  tile_work_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(ranges, ranges2, n_tiles, work_key, tile_ids);
-  return launched();
-}
-
-}  // namespace ocgs
-
-namespace ocgs {
-namespace {
-__global__ void clamp_count_kernel(const uint64_t* __restrict__ total, uint32_t cap, uint32_t* __restrict__ n32,
-                                   int* __restrict__ status) {
-  const uint64_t t = *total;
-  *n32 = (uint32_t)(t < (uint64_t)cap ? t : (uint64_t)cap);
-  if (t > (uint64_t)cap) atomicOr(status, kStatusCapacity);
-}
-}  // namespace
-
-cudaError_t launch_clamp_count(const uint64_t* total, uint32_t cap, uint32_t* n32, int* status, cudaStream_t s) {
-  clamp_count_kernel<<<1, 1, 0, s>>>(total, cap, n32, status);
   return launched();
 }
 
@@ -904,129 +887,158 @@ __device__ __forceinline__ int open_in(const uint32_t* __restrict__ P, uint32_t 
   return x1 < x0 ? 0 : (int)(P[rowbase + (uint32_t)x1 + 1u] - P[rowbase + (uint32_t)x0]);
 }
 
-constexpr int kFlatWarps = kThreads / 32;
+// The exclusive prefix P [n + 1] of the open flags and the open tiles in ascending order
+// (open_ids[P[t]] = t for every open tile t), in one kernel: a block scans its tile of
+// kScanTile flags and adds the totals of the tiles before it, found by the look-back of the
+// sorts (a wait that is given up counts the earlier flags instead).
+constexpr int kScanTile = kThreads * 16;
 
-__global__ void __launch_bounds__(kThreads) tile_count_sorted_kernel(const uint32_t* __restrict__ order, uint32_t n,
-                                                                     const float4* __restrict__ bin,
-                                                                     const DevCam* __restrict__ cams, int64_t n_gauss,
-                                                                     int tw, int th, int32_t* __restrict__ ntiles,
-                                                                     uint64_t* __restrict__ counts) {
-  __shared__ RowOwner s_own[kFlatWarps][32];
-  __shared__ int s_incl[kFlatWarps][32], s_cnt[kFlatWarps][32];
+__global__ void __launch_bounds__(kThreads) open_scan_kernel(const uint32_t* __restrict__ open, uint32_t n,
+                                                             uint32_t* __restrict__ P, uint32_t* __restrict__ open_ids,
+                                                             uint32_t* words, uint32_t* next_tile) {
+  static_assert(kScanTile <= kRadixTile, "look-back words");
+  constexpr int kItems16 = kScanTile / kThreads;
+  __shared__ uint32_t s_w[kThreads / 32];
+  __shared__ uint32_t s_tile, s_excl;
+  __shared__ int s_gave_up;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-  uint32_t r = 0;
-  int nrows = 0;
-  if (i < n) {
-    r = order[i];
-    const BinView b = load_bin(bin, r);
-    if (b.rc.z >= b.rc.x) {
-      const DevCam& cam = cams[view_of_record(r, n_gauss)];
-      s_own[warp][lane] = RowOwner{support_conic(b.g0, b.g1, b.g2, b.rb), b.rc, cam.tile_offset, cam.tiles_x,
-                                   cam.W, cam.H};
-      nrows = b.rc.w - b.rc.y + 1;
+  if (threadIdx.x == 0) {
+    s_tile = atomicAdd(next_tile, 1u);
+    s_gave_up = 0;
+  }
+  __syncthreads();
+  const uint32_t tile = s_tile, first = tile * (uint32_t)kScanTile;
+  const uint32_t wbase = first + (uint32_t)warp * 32 * kItems16 + lane;
+  uint32_t f[kItems16], pre[kItems16];
+  uint32_t run = 0;  // open flags of this warp's earlier rounds
+#pragma unroll
+  for (int j = 0; j < kItems16; ++j) f[j] = wbase + j * 32 < n ? open[wbase + j * 32] : 0u;
+#pragma unroll
+  for (int j = 0; j < kItems16; ++j) {
+    const unsigned m = __ballot_sync(kFull, f[j] != 0u);
+    pre[j] = run + (uint32_t)__popc(m & ((1u << lane) - 1u));
+    run += (uint32_t)__popc(m);
+  }
+  if (lane == 0) s_w[warp] = run;
+  __syncthreads();
+  uint32_t off = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; ++w) {
+    off += w < warp ? s_w[w] : 0u;
+    total += s_w[w];
+  }
+  if (threadIdx.x == 0) {
+    store_word(words + tile, tile == 0 ? (uint32_t)(kRadixTile + 2) + total : 1u + total);
+    uint32_t e = 0;
+    if (!look_back<1>(words, tile, &e)) s_gave_up = 1;
+    s_excl = e;
+  }
+  __syncthreads();
+  if (s_gave_up) {
+    if (threadIdx.x == 0) s_excl = 0;
+    __syncthreads();
+    uint32_t c = 0;
+    for (uint32_t i = threadIdx.x; i < first; i += kThreads) c += open[i] ? 1u : 0u;
+    atomicAdd(&s_excl, c);
+    __syncthreads();
+  }
+  const uint32_t excl = s_excl;
+  if (threadIdx.x == 0) {
+    if (tile) store_word(words + tile, (uint32_t)(kRadixTile + 2) + excl + total);
+    if (first + (uint32_t)kScanTile >= n) P[n] = excl + total;
+  }
+#pragma unroll
+  for (int j = 0; j < kItems16; ++j) {
+    const uint32_t t = wbase + j * 32;
+    if (t < n) {
+      const uint32_t q = excl + off + pre[j];
+      P[t] = q;
+      if (f[j]) open_ids[q] = t;
     }
   }
-  s_cnt[warp][lane] = 0;
-  for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
-    const RowOwner& o = s_own[warp][ri];
-    const int c = row_count(row_runs(o.k, ty, tw, th, o.W, o.H, o.rc));
-    if (c) atomicAdd(&s_cnt[warp][ri], c);
-  });
-  if (i < n) {
-    const int cnt = s_cnt[warp][lane];
-    ntiles[r] = cnt;
-    counts[i] = (uint64_t)cnt;
-  }
 }
 
-// number of entries of an ascending array below key: a 32-way search by one warp
-// (each round probes 32 evenly spaced entries of the bracket [lo, hi] that holds
-// the answer and keeps the stretch between the last probe below key and the next)
-__global__ void count_below_kernel(const uint32_t* __restrict__ sorted_keys, uint32_t n, uint32_t key,
-                                   uint32_t* __restrict__ out) {
-  const uint32_t lane = threadIdx.x;
-  uint32_t lo = 0, hi = n;
-  while (hi - lo > 32u) {
-    const uint32_t step = (hi - lo + 31u) / 32u;
-    const uint32_t pos = lo + lane * step;
-    const int c = __popc(__ballot_sync(kFull, pos < hi && sorted_keys[pos] < key));
-    const uint32_t nhi = min(hi, lo + (uint32_t)c * step);
-    lo = c > 0 ? lo + (uint32_t)(c - 1) * step + 1u : lo;
-    hi = nhi;
-  }
-  const uint32_t pos = lo + lane;
-  const int c = __popc(__ballot_sync(kFull, pos < hi && sorted_keys[pos] < key));
-  if (lane == 0) *out = lo + (uint32_t)c;
-}
-
-// Second pass, step 1: flag the entries (records behind the front, in depth
-// order) whose candidate rectangle holds an open tile (row sums of the open
-// flags from their prefix P, all rows loaded independently).
-__global__ void __launch_bounds__(kThreads) open_candidate_kernel(const uint32_t* __restrict__ order, uint32_t n,
-                                                                  const float4* __restrict__ bin,
-                                                                  const DevCam* __restrict__ cams, int64_t n_gauss,
-                                                                  const uint32_t* __restrict__ P,
-                                                                  uint32_t* __restrict__ flag) {
-  const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t r = order[i];
-  const int4 rc = bin_rect(bin[3 * (size_t)r + 2]);
-  int cand = 0;
-  if (rc.z >= rc.x) {
-    const DevCam& cam = cams[view_of_record(r, n_gauss)];
-    const uint32_t base = (uint32_t)(cam.tile_offset + rc.y * cam.tiles_x);
-    for (int ty = rc.y; ty <= rc.w; ++ty)
-      cand += open_in(P, base + (uint32_t)((ty - rc.y) * cam.tiles_x), rc.x, rc.z);
-  }
-  flag[i] = cand > 0 ? 1u : 0u;
-}
-
-// step 2: the flagged entries' records, in depth order (pos: exclusive scan of the flags)
-__global__ void compact_candidates_kernel(const uint32_t* __restrict__ order, uint32_t n,
-                                          const uint32_t* __restrict__ flag, const uint32_t* __restrict__ pos,
-                                          uint32_t* __restrict__ cand) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && flag[i]) cand[pos[i]] = order[i];
-}
-
-// step 3: open tiles reached by each candidate (counts[c] = 0 for c >= *n_cand)
-__global__ void __launch_bounds__(kThreads) open_count_kernel(const uint32_t* __restrict__ cand, uint32_t n,
-                                                              const uint32_t* __restrict__ n_cand,
+// Second pass, candidates and counts: a unit's warp tests its entries (records behind the
+// front, in depth order) for an open tile in their screen box (row sums of the open flags
+// from their prefix P) and collects the few that have one; every 32 of those, their exact
+// open tiles are counted with the rows spread over the lanes.  The unit's candidates and
+// their counts stay in its own stretch [unit * per_unit, ...) of cand and counts, in order,
+// and n_cand[unit] holds their number: nothing is compacted over the whole list.
+__global__ void __launch_bounds__(kThreads) open_count_kernel(const uint32_t* __restrict__ order, uint32_t n,
+                                                              uint32_t per_unit, uint32_t units,
                                                               const float4* __restrict__ bin,
-                                                              const DevCam* __restrict__ cams, int64_t n_gauss,
-                                                              int tw, int th, const uint32_t* __restrict__ P,
-                                                              uint64_t* __restrict__ counts) {
-  __shared__ RowOwner s_own[kFlatWarps][32];
-  __shared__ int s_incl[kFlatWarps][32], s_cnt[kFlatWarps][32];
+                                                              const DevCam* __restrict__ cams, int64_t n_gauss, int tw,
+                                                              int th, const uint32_t* __restrict__ P,
+                                                              uint32_t* __restrict__ cand,
+                                                              uint32_t* __restrict__ counts,
+                                                              uint32_t* __restrict__ n_cand, const UnitTotals totals) {
+  __shared__ RowOwner s_own[kUnitWarps][32];
+  __shared__ int s_incl[kUnitWarps][32], s_cnt[kUnitWarps][32];
+  __shared__ uint32_t s_queue[kUnitWarps][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t c = blockIdx.x * kThreads + threadIdx.x;
-  const uint32_t nc = min(n, *n_cand);
-  int nrows = 0;
-  if (c < nc) {
-    const uint32_t r = cand[c];
-    const BinView b = load_bin(bin, r);
-    const DevCam& cam = cams[view_of_record(r, n_gauss)];
-    s_own[warp][lane] = RowOwner{support_conic(b.g0, b.g1, b.g2, b.rb), b.rc, cam.tile_offset, cam.tiles_x,
-                                 cam.W, cam.H};
-    nrows = max(0, b.rc.w - b.rc.y + 1);
+  const unsigned lt = (1u << lane) - 1u;
+  const uint32_t unit = blockIdx.x * kUnitWarps + warp;
+  uint64_t sum = 0;
+  if (unit < units) {
+    const uint64_t base = (uint64_t)unit * per_unit;
+    uint32_t* queue = s_queue[warp];
+    uint32_t waiting = 0, found = 0;
+    auto count = [&](uint32_t m) {  // the first m <= 32 waiting candidates
+      int nrows = 0;
+      if (lane < (int)m) {
+        const uint32_t r = queue[lane];
+        nrows = publish_record(r, bin, cams, n_gauss, &s_own[warp][lane]);
+        cand[base + found + lane] = r;
+      }
+      s_cnt[warp][lane] = 0;
+      for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
+        if (ri < 0) return;
+        const RowOwner& o = s_own[warp][ri];
+        const RowRuns rr = row_runs(o.k, ty, tw, th, o.W, o.H, o.rc);
+        const uint32_t rowbase = (uint32_t)(o.tile_offset + ty * o.tiles_x);
+        const int c = open_in(P, rowbase, rr.a0, rr.a1) + open_in(P, rowbase, rr.b0, rr.b1);
+        if (c) atomicAdd(&s_cnt[warp][ri], c);
+      });
+      if (lane < (int)m) {
+        counts[base + found + lane] = (uint32_t)s_cnt[warp][lane];
+        sum += (uint64_t)s_cnt[warp][lane];
+      }
+      found += m;
+      __syncwarp();
+    };
+    for (uint32_t k = 0; k < per_unit; k += 32) {
+      const uint64_t i = base + k + lane;
+      if (__all_sync(kFull, i >= n)) break;
+      uint32_t r = 0;
+      bool open_here = false;
+      if (i < n) {
+        r = order[i];
+        const int4 rc = bin_rect(bin[3 * (size_t)r + 2]);
+        if (rc.z >= rc.x) {
+          const DevCam& cam = cams[view_of_record(r, n_gauss)];
+          const uint32_t row0 = (uint32_t)(cam.tile_offset + rc.y * cam.tiles_x);
+          int c = 0;
+          for (int ty = rc.y; ty <= rc.w; ++ty) c += open_in(P, row0 + (uint32_t)((ty - rc.y) * cam.tiles_x), rc.x, rc.z);
+          open_here = c > 0;
+        }
+      }
+      const unsigned m = __ballot_sync(kFull, open_here);
+      if (open_here) queue[waiting + __popc(m & lt)] = r;
+      waiting += (uint32_t)__popc(m);
+      __syncwarp();
+      if (waiting >= 32) {
+        count(32);
+        const uint32_t rest = queue[32 + lane];
+        __syncwarp();
+        queue[lane] = rest;
+        waiting -= 32;
+        __syncwarp();
+      }
+    }
+    if (waiting) count(waiting);
+    if (lane == 0) n_cand[unit] = found;
   }
-  s_cnt[warp][lane] = 0;
-  for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
-    const RowOwner& o = s_own[warp][ri];
-    const RowRuns rr = row_runs(o.k, ty, tw, th, o.W, o.H, o.rc);
-    const uint32_t rowbase = (uint32_t)(o.tile_offset + ty * o.tiles_x);
-    const int cnt = open_in(P, rowbase, rr.a0, rr.a1) + open_in(P, rowbase, rr.b0, rr.b1);
-    if (cnt) atomicAdd(&s_cnt[warp][ri], cnt);
-  });
-  if (c < n) counts[c] = (uint64_t)s_cnt[warp][lane];
-}
-
-// The open tiles, compacted in ascending id: open_ids[P[t]] = t for every open tile t.
-__global__ void open_ids_kernel(const uint32_t* __restrict__ open, const uint32_t* __restrict__ P, uint32_t n,
-                                uint32_t* __restrict__ open_ids) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n && open[t]) open_ids[P[t]] = t;
+  finish_units(totals, units, sum);
 }
 
 // The open tiles of the run [x0, x1] of a tile row are the contiguous slice
@@ -1041,210 +1053,162 @@ __device__ __forceinline__ OpenSlice open_slice(const uint32_t* __restrict__ P, 
   return OpenSlice{a, (int)(P[rowbase + (uint32_t)x1 + 1u] - a)};
 }
 
-constexpr int kOpenThreads = 128;
-constexpr int kOpenWarps = kOpenThreads / 32;
+// The second-pass pairs in depth order, as in duplicate_kernel: each row's open tiles are the
+// slices of its two runs.  A block takes the candidates of kUnitWarps units together: it
+// scans their counts, and its warps take 32 candidates at a time, so that the lanes are full
+// although a unit holds few candidates and the block's units hold unequal numbers.
+constexpr int kGroup = kDupThreads * 4;  // candidates of a block per round
 
-// step 4, the second-pass pairs in depth order: candidate i writes its open
-// tiles from offsets[i] on (rows in order, tiles left to right), each run's open
-// tiles being a slice of open_ids.  A lane finds the slices of its candidate
-// when it spans few rows and the warp writes all those candidates' tiles as one
-// flat list, 32 consecutive slots per step; the rows of a taller candidate are
-// shared out over the warp.
-__global__ void __launch_bounds__(kOpenThreads) duplicate_open_kernel(
-    const uint32_t* __restrict__ order, const uint64_t* __restrict__ offsets, const uint64_t* __restrict__ total,
-    uint32_t n_rec, const uint32_t* __restrict__ n_cand, const float4* __restrict__ bin,
+__global__ void __launch_bounds__(kDupThreads) duplicate_open_kernel(
+    const uint32_t* __restrict__ cand, const uint32_t* __restrict__ counts, const uint32_t* __restrict__ n_cand,
+    uint32_t per_unit, uint32_t units, const uint64_t* __restrict__ unit_base, const float4* __restrict__ bin,
     const DevCam* __restrict__ cams, int64_t n_gauss, int tw, int th, const uint32_t* __restrict__ open_ids,
     const uint32_t* __restrict__ P, uint32_t n_pairs, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  __shared__ uint32_t s_sa[kOpenWarps][kSmallRows][32], s_sb[kOpenWarps][kSmallRows][32];  // [row][lane]
-  __shared__ uint32_t s_cnt[kOpenWarps][kSmallRows][32];  // open tiles of the two runs: a | b << 16
-  __shared__ int s_incl[kOpenWarps][32];
-  __shared__ uint32_t s_pos[kOpenWarps][32];
-  __shared__ uint32_t s_rec[kOpenWarps][32];
+  __shared__ RowOwner s_own[kDupWarps][32];
+  __shared__ int s_incl[kDupWarps][32];
+  __shared__ uint32_t s_first[kUnitWarps + 1];  // first candidate of each unit within the block's list
+  __shared__ uint32_t s_rec[kGroup], s_pos[kGroup], s_w[kDupWarps];
+  static_assert(kDupWarps == kUnitWarps, "one block per counting block");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t i = blockIdx.x * kOpenThreads + threadIdx.x;
-  n_rec = min(n_rec, *n_cand);
-  uint32_t r = 0;
-  uint64_t o = 0;
-  if (i < n_rec) {
-    o = offsets[i];
-    r = order[i];
-  }
-  uint64_t o_next = __shfl_down_sync(kFull, o, 1);
-  if (lane == 31 || i + 1 >= n_rec) o_next = (i + 1 < n_rec) ? offsets[i + 1] : *total;
-  int cnt = 0;
-  int4 rc = make_int4(0, 0, -1, -1);
-  if (i < n_rec && o < (uint64_t)n_pairs) {  // entries past a capacity write nothing
-    cnt = (int)(o_next - o);
-    if (cnt > 0) rc = bin_rect(bin[3 * (size_t)r + 2]);
-  }
-  const bool small = cnt > 0 && (rc.w - rc.y + 1) <= kSmallRows;
-  if (small) {
-    // a lane finds its candidate's slices (the rows spread over the warp measured slower
-    // here, the candidates behind the front spanning few rows)
-    const BinView b = load_bin(bin, r);
-    const DevCam& cam = cams[view_of_record(r, n_gauss)];
-    const SupportConic k = support_conic(b.g0, b.g1, b.g2, b.rb);
-    for (int ty = rc.y; ty <= rc.w; ++ty) {
-      const RowRuns rr = row_runs(k, ty, tw, th, cam.W, cam.H, rc);
-      const uint32_t rowbase = (uint32_t)(cam.tile_offset + ty * cam.tiles_x);
-      const OpenSlice sa = open_slice(P, rowbase, rr.a0, rr.a1), sb = open_slice(P, rowbase, rr.b0, rr.b1);
-      s_sa[warp][ty - rc.y][lane] = sa.start;
-      s_sb[warp][ty - rc.y][lane] = sb.start;
-      s_cnt[warp][ty - rc.y][lane] = (uint32_t)sa.count | ((uint32_t)sb.count << 16);
+  const uint32_t u0 = blockIdx.x * kUnitWarps;
+  if (threadIdx.x == 0) {
+    uint32_t c = 0;
+    for (int u = 0; u < kUnitWarps; ++u) {
+      s_first[u] = c;
+      if (u0 + u < units) c += n_cand[u0 + u];
     }
-    s_pos[warp][lane] = (uint32_t)o;
-    s_rec[warp][lane] = r;
+    s_first[kUnitWarps] = c;
   }
-  // flat walk over the small candidates' open tiles
-  const int scnt = small ? cnt : 0;
-  int incl = scnt;
+  __syncthreads();
+  const uint32_t found = s_first[kUnitWarps];
+  uint64_t start = unit_start(unit_base, units, u0);  // first pair of the group
+  for (uint32_t g0 = 0; g0 < found; g0 += kGroup) {
+    const uint32_t here = min((uint32_t)kGroup, found - g0);
+    // 4 consecutive candidates per thread
+    uint32_t c[4], mine = 0;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int t = __shfl_up_sync(kFull, incl, d);
-    if (lane >= d) incl += t;
-  }
-  s_incl[warp][lane] = incl;
-  const int all = __shfl_sync(kFull, incl, 31);
-  __syncwarp();
-  for (int q0 = 0; q0 < all; q0 += 32) {
-    const int q = q0 + lane;
-    if (q < all) {
-      int lo = 0, hi = 31;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s_incl[warp][mid] > q) hi = mid; else lo = mid + 1;
-      }
-      const int ri = lo;
-      const int excl = ri > 0 ? s_incl[warp][ri - 1] : 0;  // tiles of the warp's earlier small candidates
-      int kth = q - excl;
-      uint32_t slot = 0xffffffffu;
-      for (int row = 0; row < kSmallRows; ++row) {
-        const uint32_t c = s_cnt[warp][row][ri];
-        const int la = (int)(c & 0xffffu), lb = (int)(c >> 16);
-        if (kth < la) { slot = s_sa[warp][row][ri] + (uint32_t)kth; break; }
-        kth -= la;
-        if (kth < lb) { slot = s_sb[warp][row][ri] + (uint32_t)kth; break; }
-        kth -= lb;
-      }
-      const uint32_t pos = s_pos[warp][ri] + (uint32_t)(q - excl);
-      if (slot != 0xffffffffu && pos < n_pairs) {
-        keys[pos] = open_ids[slot];
-        vals[pos] = s_rec[warp][ri];
-      }
-    }
-  }
-  unsigned big = __ballot_sync(kFull, cnt > 0 && !small);
-  while (big) {
-    const int src = __ffs(big) - 1;
-    big &= big - 1u;
-    const uint32_t rr = __shfl_sync(kFull, r, src);
-    const uint64_t oo = __shfl_sync(kFull, o, src);
-    const int bcnt = __shfl_sync(kFull, cnt, src);
-    const BinView bb = load_bin(bin, rr);
-    const int4 bc = bb.rc;
-    const DevCam& cam = cams[view_of_record(rr, n_gauss)];
-    const SupportConic k = support_conic(bb.g0, bb.g1, bb.g2, bb.rb);
-    const uint64_t stop = min(oo + (uint64_t)bcnt, (uint64_t)n_pairs);
-    uint64_t base = oo;
-    for (int row0 = bc.y; row0 <= bc.w; row0 += 32) {
-      const int ty = row0 + lane;
-      OpenSlice sa{0u, 0}, sb{0u, 0};
-      if (ty <= bc.w) {
-        const RowRuns runs = row_runs(k, ty, tw, th, cam.W, cam.H, bc);
-        const uint32_t rowbase = (uint32_t)(cam.tile_offset + ty * cam.tiles_x);
-        sa = open_slice(P, rowbase, runs.a0, runs.a1);
-        sb = open_slice(P, rowbase, runs.b0, runs.b1);
-      }
-      const int c = sa.count + sb.count;
-      int inc = c;
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t q = threadIdx.x * 4 + k;
+      c[k] = 0;
+      if (q < here) {
+        int u = 0;
 #pragma unroll
-      for (int s2 = 1; s2 < 32; s2 <<= 1) {
-        const int t = __shfl_up_sync(kFull, inc, s2);
-        if (lane >= s2) inc += t;
+        for (int v = 1; v < kUnitWarps; ++v) u += s_first[v] <= g0 + q ? 1 : 0;
+        const uint64_t at = (uint64_t)(u0 + u) * per_unit + (g0 + q - s_first[u]);
+        s_rec[q] = cand[at];
+        c[k] = counts[at];
       }
-      uint64_t pos = base + (uint64_t)(inc - c);
-      for (int j = 0; j < sa.count; ++j, ++pos)
-        if (pos < stop) { keys[pos] = open_ids[sa.start + (uint32_t)j]; vals[pos] = rr; }
-      for (int j = 0; j < sb.count; ++j, ++pos)
-        if (pos < stop) { keys[pos] = open_ids[sb.start + (uint32_t)j]; vals[pos] = rr; }
-      base += (uint64_t)__shfl_sync(kFull, inc, 31);
+      mine += c[k];
     }
+    const uint32_t inc = warp_inclusive_scan<uint32_t>(mine, lane);
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t before = inc - mine, total = 0;
+#pragma unroll
+    for (int w = 0; w < kDupWarps; ++w) {
+      before += w < warp ? s_w[w] : 0u;
+      total += s_w[w];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      s_pos[threadIdx.x * 4 + k] = before;
+      before += c[k];
+    }
+    __syncthreads();
+    for (uint32_t q0 = warp * 32; q0 < here; q0 += kDupThreads) {
+      const uint32_t q = q0 + lane;
+      const int nrows = q < here ? publish_record(s_rec[q], bin, cams, n_gauss, &s_own[warp][lane]) : 0;
+      uint64_t run = start + s_pos[q0];
+      for_warp_rows(nrows, lane, s_incl[warp], s_own[warp], [&](int ri, int ty) {
+        OpenSlice sa{0u, 0}, sb{0u, 0};
+        uint32_t r = 0;
+        if (ri >= 0) {
+          const RowOwner& o = s_own[warp][ri];
+          const RowRuns rr = row_runs(o.k, ty, tw, th, o.W, o.H, o.rc);
+          const uint32_t rowbase = (uint32_t)(o.tile_offset + ty * o.tiles_x);
+          sa = open_slice(P, rowbase, rr.a0, rr.a1);
+          sb = open_slice(P, rowbase, rr.b0, rr.b1);
+          r = s_rec[q0 + ri];
+        }
+        const RowItems it = row_items(sa.start, sa.count, sb.start, sb.count);
+        const int row_inc = warp_inclusive_scan<int>(it.c, lane);
+        write_rows(it, run + (uint64_t)(row_inc - it.c), r, n_pairs, lane, keys, vals,
+                   [&](uint32_t x) { return open_ids[x]; });
+        run += (uint64_t)__shfl_sync(kFull, row_inc, 31);
+      });
+    }
+    start += total;
+    __syncthreads();  // the next group overwrites s_rec, s_pos and s_w
   }
 }
 
-// The second pass's queue: tiles with a second-pass segment, longest first (log scale),
-// every other tile last; n_again counts the former.
-__global__ void second_queue_kernel(const uint2* __restrict__ ranges2, uint32_t n_tiles,
-                                    uint32_t* __restrict__ work_key, uint32_t* __restrict__ ids,
-                                    uint32_t* __restrict__ n_again) {
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  const uint2 r2 = ranges2[t];
-  const uint32_t len = r2.y - r2.x;
-  if (len) atomicAdd(n_again, 1u);
-  work_key[t] = queue_key(len);
-  ids[t] = t;
+struct UnitPlan {
+  uint32_t per_unit, units;
+};
+// Rounds of 32 entries per unit so that there are at most kMaxUnits units.
+UnitPlan unit_plan(uint32_t n) {
+  const uint32_t per = 32u * std::max(1u, (uint32_t)(((uint64_t)n + 32ull * kMaxUnits - 1) / (32ull * kMaxUnits)));
+  return UnitPlan{per, (uint32_t)(((uint64_t)n + per - 1) / per)};
 }
 
 }  // namespace
 
-cudaError_t launch_tile_count_sorted(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
-                                     int64_t n_gauss, int tile_w, int tile_h, int32_t* ntiles, uint64_t* counts,
-                                     cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  tile_count_sorted_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(order, n, bin, cams, n_gauss, tile_w,
-                                                                              tile_h, ntiles, counts);
+// (the number of units is not monotonic in n)
+size_t unit_capacity(uint32_t n) { return std::min<size_t>(((size_t)n + 31) / 32, kMaxUnits); }
+size_t unit_base_words(uint32_t n) { return unit_capacity(n) + (unit_capacity(n) + kUnitWarps - 1) / kUnitWarps; }
+
+cudaError_t launch_bin_count(const uint32_t* order, uint32_t n, const uint32_t* d_n, const float4* bin,
+                             const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h, uint64_t* unit_base,
+                             uint32_t* done, uint64_t* total, cudaStream_t s, uint32_t* n32, uint32_t cap,
+                             int* status) {
+  if (n == 0) return cudaMemsetAsync(total, 0, sizeof(uint64_t), s);
+  const UnitPlan u = unit_plan(n);
+  bin_count_kernel<<<(u.units + kUnitWarps - 1) / kUnitWarps, kThreads, 0, s>>>(
+      order, n, d_n, u.per_unit, u.units, bin, cams, n_gauss, tile_w, tile_h,
+      UnitTotals{unit_base, done, total, n32, cap, status});
   return launched();
 }
 
-cudaError_t launch_count_below(const uint32_t* sorted_keys, uint32_t n, uint32_t key, uint32_t* out,
-                               cudaStream_t s) {
-  count_below_kernel<<<1, 32, 0, s>>>(sorted_keys, n, key, out);
+cudaError_t launch_duplicate(const uint32_t* order, uint32_t n, const uint32_t* d_n, const uint64_t* unit_base,
+                             const float4* bin, const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h,
+                             uint32_t n_pairs, uint32_t* keys, uint32_t* vals, cudaStream_t s) {
+  if (n_pairs == 0 || n == 0) return cudaSuccess;
+  const UnitPlan u = unit_plan(n);
+  duplicate_kernel<<<(u.units + kDupWarps - 1) / kDupWarps, kDupThreads, 0, s>>>(
+      order, n, d_n, u.per_unit, u.units, unit_base, bin, cams, n_gauss, tile_w, tile_h, n_pairs, keys, vals);
   return launched();
 }
 
-cudaError_t launch_open_candidates(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
-                                   int64_t n_gauss, const uint32_t* open_prefix, uint32_t* flag, uint32_t* pos,
-                                   uint32_t* cand, uint32_t* n_cand, void* scratch, cudaStream_t s) {
-  if (n == 0) return cudaMemsetAsync(n_cand, 0, sizeof(uint32_t), s);
-  open_candidate_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(order, n, bin, cams, n_gauss,
-                                                                           open_prefix, flag);
-  cudaError_t e = launched();
-  if (e != cudaSuccess) return e;
-  e = scan_exclusive<uint32_t>(flag, pos, n, n_cand, static_cast<char*>(scratch), s);
-  if (e != cudaSuccess) return e;
-  compact_candidates_kernel<<<(n + 255) / 256, 256, 0, s>>>(order, n, flag, pos, cand);
+size_t open_scan_words(uint32_t n_tiles) { return ((size_t)n_tiles + kScanTile - 1) / kScanTile + 1; }
+
+cudaError_t launch_open_scan(const uint32_t* open, uint32_t n_tiles, uint32_t* P, uint32_t* open_ids, uint32_t* words,
+                             cudaStream_t s) {
+  const uint32_t blocks = (uint32_t)open_scan_words(n_tiles) - 1;
+  open_scan_kernel<<<blocks, kThreads, 0, s>>>(open, n_tiles, P, open_ids, words, words + blocks);
   return launched();
 }
 
-cudaError_t launch_open_count(const uint32_t* cand, uint32_t n, const uint32_t* n_cand, const float4* bin,
-                              const DevCam* cams, int64_t n_gauss, int tile_w, int tile_h,
-                              const uint32_t* open_prefix, uint64_t* counts, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  open_count_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(cand, n, n_cand, bin, cams, n_gauss, tile_w,
-                                                                       tile_h, open_prefix, counts);
+cudaError_t launch_open_count(const uint32_t* order, uint32_t n, const float4* bin, const DevCam* cams,
+                              int64_t n_gauss, int tile_w, int tile_h, const uint32_t* P, uint32_t* cand,
+                              uint32_t* counts, uint32_t* n_cand, uint64_t* unit_base, uint32_t* done,
+                              uint64_t* total, cudaStream_t s) {
+  if (n == 0) return cudaMemsetAsync(total, 0, sizeof(uint64_t), s);
+  const UnitPlan u = unit_plan(n);
+  open_count_kernel<<<(u.units + kUnitWarps - 1) / kUnitWarps, kThreads, 0, s>>>(
+      order, n, u.per_unit, u.units, bin, cams, n_gauss, tile_w, tile_h, P, cand, counts, n_cand,
+      UnitTotals{unit_base, done, total, nullptr, 0u, nullptr});
   return launched();
 }
 
-cudaError_t launch_duplicate_open(const uint32_t* cand, const uint64_t* offsets, const uint64_t* total,
-                                  uint32_t n_rec, const uint32_t* n_cand, const float4* bin, const DevCam* cams,
-                                  int64_t n_gauss, int tile_w, int tile_h, const uint32_t* open,
-                                  const uint32_t* open_prefix, uint32_t n_tiles, uint32_t* open_ids, uint32_t n_pairs,
-                                  uint32_t* keys, uint32_t* vals, cudaStream_t s) {
-  if (n_pairs == 0 || n_rec == 0) return cudaSuccess;
-  open_ids_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(open, open_prefix, n_tiles, open_ids);
-  cudaError_t e = launched();
-  if (e != cudaSuccess) return e;
-  duplicate_open_kernel<<<(n_rec + kOpenThreads - 1) / kOpenThreads, kOpenThreads, 0, s>>>(
-      cand, offsets, total, n_rec, n_cand, bin, cams, n_gauss, tile_w, tile_h, open_ids, open_prefix, n_pairs, keys,
-      vals);
-  return launched();
-}
-
-cudaError_t launch_second_queue(const uint2* ranges2, uint32_t n_tiles, uint32_t* work_key, uint32_t* ids,
-                                uint32_t* n_again, cudaStream_t s) {
-  if (n_tiles == 0) return cudaSuccess;
-  second_queue_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(ranges2, n_tiles, work_key, ids, n_again);
+cudaError_t launch_duplicate_open(const uint32_t* cand, uint32_t n, const uint32_t* counts, const uint32_t* n_cand,
+                                  const uint64_t* unit_base, const float4* bin, const DevCam* cams, int64_t n_gauss,
+                                  int tile_w, int tile_h, const uint32_t* open_ids, const uint32_t* P,
+                                  uint32_t n_pairs, uint32_t* keys, uint32_t* vals, cudaStream_t s) {
+  if (n_pairs == 0 || n == 0) return cudaSuccess;
+  const UnitPlan u = unit_plan(n);
+  duplicate_open_kernel<<<(u.units + kDupWarps - 1) / kDupWarps, kDupThreads, 0, s>>>(
+      cand, counts, n_cand, u.per_unit, u.units, unit_base, bin, cams, n_gauss, tile_w, tile_h, open_ids, P, n_pairs,
+      keys, vals);
   return launched();
 }
 
