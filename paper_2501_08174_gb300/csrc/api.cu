@@ -255,7 +255,34 @@ struct LossPlan {
   int blocks = 0;
 };
 
-ocgs_status plan_loss(ocgs_ctx* ctx, const ocgs_camera* cams, int n_views, LossPlan* lp) {
+// A loss's view table and block prefix on the device (one allocation with the loss's scratch,
+// one copy).
+struct LossTables {
+  DevCam* cams = nullptr;
+  int* prefix = nullptr;
+  double* partial = nullptr;
+  float* map = nullptr;
+};
+ocgs_status loss_tables(ocgs_ctx* ctx, Arena& a, const std::vector<DevCam>& cams, const std::vector<int>& prefix,
+                        size_t partials, size_t map_floats, LossTables* t) {
+  const size_t cam_bytes = sizeof(DevCam) * cams.size(), prefix_bytes = sizeof(int) * prefix.size();
+  char* tables;
+  Block b;
+  b.add(&tables, cam_bytes + prefix_bytes);
+  b.add(&t->partial, partials);
+  if (map_floats) b.add(&t->map, map_floats);
+  CK(b.alloc(a, ctx->stream));
+  std::vector<char> h(cam_bytes + prefix_bytes);
+  std::memcpy(h.data(), cams.data(), cam_bytes);
+  std::memcpy(h.data() + cam_bytes, prefix.data(), prefix_bytes);
+  CK(cudaMemcpyAsync(tables, h.data(), h.size(), cudaMemcpyHostToDevice, ctx->stream));
+  t->cams = reinterpret_cast<DevCam*>(tables);
+  t->prefix = reinterpret_cast<int*>(tables + cam_bytes);
+  return OCGS_OK;
+}
+
+ocgs_status plan_loss(ocgs_ctx* ctx, const ocgs_camera* cams, int n_views, LossPlan* lp,
+                      int block_pixels = kLossBlockPixels) {
   if (!cams || n_views < 1 || n_views > 4096) return set_err(ctx, OCGS_ERR_ARG, "bad cameras");
   lp->cams.assign(n_views, DevCam{});
   lp->prefix.assign(n_views + 1, 0);
@@ -275,7 +302,7 @@ ocgs_status plan_loss(ocgs_ctx* ctx, const ocgs_camera* cams, int n_views, LossP
     d.pix_offset = pix;
     const int64_t np = (int64_t)cams[v].width * cams[v].height;
     lp->prefix[v] = blocks;
-    blocks += (int)((np + kLossBlockPixels - 1) / kLossBlockPixels);
+    blocks += (int)((np + block_pixels - 1) / block_pixels);
     pix += np;
   }
   lp->prefix[n_views] = blocks;
@@ -887,16 +914,11 @@ ocgs_status ocgs_background_loss(ocgs_ctx* ctx, const float* alpha, const uint8_
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, lp.blocks));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, lp.prefix, lp.blocks, 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, lp.prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_background_loss(alpha, mask, d_cams, n_views, d_prefix, lp.blocks, gamma, partial, loss, d_alpha, s));
+  CK(launch_background_loss(alpha, mask, lt.cams, n_views, lt.prefix, lp.blocks, gamma, lt.partial, loss, d_alpha, s));
   return OCGS_OK;
 }
 
@@ -911,16 +933,11 @@ ocgs_status ocgs_masked_l1(ocgs_ctx* ctx, const float* rgb, const float* target,
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, lp.blocks));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, lp.prefix, lp.blocks, 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, lp.prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_masked_l1(rgb, target, mask, d_cams, n_views, d_prefix, lp.blocks, weight, partial, loss, d_rgb, s));
+  CK(launch_masked_l1(rgb, target, mask, lt.cams, n_views, lt.prefix, lp.blocks, weight, lt.partial, loss, d_rgb, s));
   return OCGS_OK;
 }
 
@@ -943,18 +960,11 @@ ocgs_status ocgs_ssim(ocgs_ctx* ctx, const float* rgb, const float* target, cons
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  float* gmap = nullptr;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, 3 * (size_t)tiles));
-  if (d_rgb) CK(tmp.alloc(&gmap, 9 * (size_t)P));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, prefix, 3 * (size_t)tiles, d_rgb ? 9 * (size_t)P : 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_ssim(rgb, target, mask, d_cams, n_views, d_prefix, tiles, P, weight, partial, gmap, ssim, ssim_masked,
+  CK(launch_ssim(rgb, target, mask, lt.cams, n_views, lt.prefix, tiles, P, weight, lt.partial, lt.map, ssim, ssim_masked,
                  d_rgb, s));
   return OCGS_OK;
 }
@@ -965,21 +975,16 @@ ocgs_status ocgs_masked_psnr(ocgs_ctx* ctx, const float* rgb, const float* targe
   if (!rgb || !target || !mask || !psnr) return set_err(ctx, OCGS_ERR_ARG, "rgb, target, mask and psnr must be non-NULL");
   if (!(std::isfinite(max_i) && max_i > 0.f)) return set_err(ctx, OCGS_ERR_ARG, "max_i must be finite and > 0");
   LossPlan lp;
-  ocgs_status r = plan_loss(ctx, cams, n_views, &lp);
+  ocgs_status r = plan_loss(ctx, cams, n_views, &lp, kPsnrBlockPixels);
   if (r != OCGS_OK) return r;
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, 2 * (size_t)lp.blocks));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, lp.prefix, 2 * (size_t)lp.blocks, 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, lp.prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_masked_psnr(rgb, target, mask, d_cams, n_views, d_prefix, lp.blocks, (double)max_i, partial, psnr, s));
+  CK(launch_masked_psnr(rgb, target, mask, lt.cams, n_views, lt.prefix, lp.blocks, (double)max_i, lt.partial, psnr, s));
   return OCGS_OK;
 }
 
@@ -997,16 +1002,11 @@ ocgs_status ocgs_depth_distortion(ocgs_ctx* ctx, const float* alpha, const float
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, lp.blocks));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, lp.prefix, lp.blocks, 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, lp.prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_depth_distortion(alpha, depth, depth2, d_cams, n_views, d_prefix, lp.blocks, weight, partial, loss,
+  CK(launch_depth_distortion(alpha, depth, depth2, lt.cams, n_views, lt.prefix, lp.blocks, weight, lt.partial, loss,
                              d_alpha, d_depth, d_depth2, s));
   return OCGS_OK;
 }
@@ -1032,19 +1032,12 @@ ocgs_status ocgs_normal_consistency(ocgs_ctx* ctx, const float* alpha, const flo
   CK(cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   Arena tmp(ctx);
-  DevCam* d_cams;
-  int* d_prefix;
-  double* partial;
-  float* gmap = nullptr;
-  CK(tmp.alloc(&d_cams, n_views));
-  CK(tmp.alloc(&d_prefix, n_views + 1));
-  CK(tmp.alloc(&partial, lp.blocks));
-  if (d_alpha) CK(tmp.alloc(&gmap, 6 * (size_t)P));
+  LossTables lt;
+  r = loss_tables(ctx, tmp, lp.cams, lp.prefix, lp.blocks, d_alpha ? 6 * (size_t)P : 0, &lt);
+  if (r != OCGS_OK) return r;
   StageTimer t(ctx, OCGS_STAGE_LOSS);
-  CK(cudaMemcpyAsync(d_cams, lp.cams.data(), sizeof(DevCam) * n_views, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_prefix, lp.prefix.data(), sizeof(int) * (n_views + 1), cudaMemcpyHostToDevice, s));
-  CK(launch_normal_consistency(alpha, depth, normal, d_cams, n_views, d_prefix, lp.blocks, weight, a_min, partial,
-                               gmap, loss, d_alpha, d_depth, d_normal, s));
+  CK(launch_normal_consistency(alpha, depth, normal, lt.cams, n_views, lt.prefix, lp.blocks, weight, a_min, lt.partial,
+                               lt.map, loss, d_alpha, d_depth, d_normal, s));
   return OCGS_OK;
 }
 

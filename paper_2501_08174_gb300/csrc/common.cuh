@@ -462,6 +462,7 @@ struct RasterBwdArgs {
 };
 cudaError_t launch_raster_backward(const RasterBwdArgs& a, int tile_w, int tile_h, int ppt, int batch,
                                    cudaStream_t s);
+constexpr int kPsnrBlockPixels = 1024;
 // sum of the per-pixel blended-prefix lengths (the pairs both passes must evaluate)
 cudaError_t launch_sum_u32(const uint32_t* v, int64_t n, unsigned long long* out, cudaStream_t s);
 
@@ -631,7 +632,7 @@ cudaError_t launch_normal_consistency(const float* alpha, const float* depth, co
                                       int n_views, const int* block_prefix, int n_blocks, float weight, float a_min,
                                       double* partial, float* gmap, double* loss, float* d_alpha, float* d_depth,
                                       float* d_normal, cudaStream_t s);
-// PSNR over the loss blocks (kLossBlockPixels per block); partial holds 2 doubles per block
+// PSNR over blocks of kPsnrBlockPixels; partial holds 2 doubles per block
 cudaError_t launch_masked_psnr(const float* rgb, const float* target, const uint8_t* mask, const DevCam* cams,
                                int n_views, const int* block_prefix, int n_blocks, double max_i, double* partial,
                                double* psnr, cudaStream_t s);

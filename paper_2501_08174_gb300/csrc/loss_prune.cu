@@ -11,6 +11,7 @@ namespace ocgs {
 namespace {
 
 constexpr int kLossThreads = 256;
+constexpr int kLossLoads = 2;  // pixels per thread whose loads are in flight together
 
 // Each block reduces kLossBlockPixels pixels of one view, in a fixed order
 // (compensated float32 sums per thread, merged into one FP64 partial per block),
@@ -28,11 +29,21 @@ __global__ void __launch_bounds__(kLossThreads) bg_loss_partial_kernel(
   const int64_t hi = (lo + kLossBlockPixels < npix) ? lo + kLossBlockPixels : npix;
   const float g = gamma / (float)npix;
   CompSum acc[1];
-  for (int64_t k = lo + threadIdx.x; k < hi; k += kLossThreads) {
-    const int64_t p = cam.pix_offset + k;
-    const float bg = mask[p] ? 0.f : 1.f;
-    acc[0].add(alpha[p] * bg);  // alpha (1 - M) is exact
-    if (d_alpha) d_alpha[p] += g * bg;
+  for (int64_t k0 = lo + threadIdx.x; k0 < hi; k0 += kLossLoads * kLossThreads) {
+    float a[kLossLoads], d[kLossLoads];
+    bool bg[kLossLoads];
+#pragma unroll
+    for (int u = 0; u < kLossLoads; ++u) {
+      const int64_t k = k0 + u * kLossThreads, p = cam.pix_offset + k;
+      bg[u] = k < hi && !mask[p];
+      a[u] = k < hi ? alpha[p] : 0.f;
+      d[u] = bg[u] && d_alpha ? d_alpha[p] : 0.f;  // (1 - M) adds nothing to the others
+    }
+#pragma unroll
+    for (int u = 0; u < kLossLoads; ++u) {
+      acc[0].add(a[u] * (bg[u] ? 1.f : 0.f));  // alpha (1 - M) is exact
+      if (bg[u] && d_alpha) d_alpha[cam.pix_offset + k0 + u * kLossThreads] = d[u] + g;
+    }
   }
   block_comp_sums<kLossThreads, 1>(acc, partial + b);
 }
@@ -55,15 +66,35 @@ __global__ void __launch_bounds__(kLossThreads) l1_partial_kernel(
   const int64_t hi = (lo + kLossBlockPixels < npix) ? lo + kLossBlockPixels : npix;
   const float g = weight / (3.0f * (float)npix);
   CompSum acc[1];
-  for (int64_t k = lo + threadIdx.x; k < hi; k += kLossThreads) {
-    const int64_t p = cam.pix_offset + k;
-    if (!mask[p]) continue;
+  for (int64_t k0 = lo + threadIdx.x; k0 < hi; k0 += kLossLoads * kLossThreads) {
+    bool m[kLossLoads];
+    float x[kLossLoads][3], y[kLossLoads][3], q[kLossLoads][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float e;
-      const float d = two_sum(rgb[3 * p + c], -target[3 * p + c], e);
-      acc[0].add(fabsf(d), d > 0.f ? e : -e);
-      if (d_rgb) d_rgb[3 * p + c] += d > 0.f ? g : (d < 0.f ? -g : 0.f);
+    for (int u = 0; u < kLossLoads; ++u) {
+      const int64_t k = k0 + u * kLossThreads;
+      m[u] = k < hi && mask[cam.pix_offset + k];
+    }
+#pragma unroll
+    for (int u = 0; u < kLossLoads; ++u) {
+      const int64_t p = cam.pix_offset + k0 + u * kLossThreads;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        x[u][c] = m[u] ? rgb[3 * p + c] : 0.f;
+        y[u][c] = m[u] ? target[3 * p + c] : 0.f;
+        q[u][c] = m[u] && d_rgb ? d_rgb[3 * p + c] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kLossLoads; ++u) {
+      if (!m[u]) continue;
+      const int64_t p = cam.pix_offset + k0 + u * kLossThreads;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float e;
+        const float d = two_sum(x[u][c], -y[u][c], e);
+        acc[0].add(fabsf(d), d > 0.f ? e : -e);
+        if (d_rgb) d_rgb[3 * p + c] = q[u][c] + (d > 0.f ? g : (d < 0.f ? -g : 0.f));
+      }
     }
   }
   block_comp_sums<kLossThreads, 1>(acc, partial + b);
@@ -72,17 +103,12 @@ __global__ void __launch_bounds__(kLossThreads) l1_partial_kernel(
 // one CTA per view
 __global__ void __launch_bounds__(kViewSumThreads) bg_loss_final_kernel(const double* __restrict__ partial,
                                                                        const int* __restrict__ block_prefix,
-                                                                       const DevCam* __restrict__ cams,
+                                                                       const DevCam* __restrict__ cams, double scale,
                                                                        double* __restrict__ loss) {
   const int v = blockIdx.x;
   double t;
   view_block_sums<1>(partial, block_prefix[v], block_prefix[v + 1], &t);
-  if (threadIdx.x == 0) loss[v] = t / ((double)cams[v].W * (double)cams[v].H);
-}
-
-__global__ void scale_kernel(double* __restrict__ x, int n, double f) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] *= f;
+  if (threadIdx.x == 0) loss[v] = t / ((double)cams[v].W * (double)cams[v].H) * scale;
 }
 
 __global__ void prune_flags_kernel(const float* __restrict__ score, uint32_t n, float tau,
@@ -127,7 +153,7 @@ cudaError_t launch_background_loss(const float* alpha, const uint8_t* mask, cons
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
   }
-  bg_loss_final_kernel<<<n_views, kViewSumThreads, 0, s>>>(partial, block_prefix, cams, loss);
+  bg_loss_final_kernel<<<n_views, kViewSumThreads, 0, s>>>(partial, block_prefix, cams, 1.0, loss);
   return launched();
 }
 
@@ -141,10 +167,7 @@ cudaError_t launch_masked_l1(const float* rgb, const float* target, const uint8_
     if (e != cudaSuccess) return e;
   }
   // the final pass divides by h*w; the L1 mean is over 3*h*w values
-  bg_loss_final_kernel<<<n_views, kViewSumThreads, 0, s>>>(partial, block_prefix, cams, loss);
-  cudaError_t e = launched();
-  if (e != cudaSuccess) return e;
-  scale_kernel<<<(n_views + 127) / 128, 128, 0, s>>>(loss, n_views, 1.0 / 3.0);
+  bg_loss_final_kernel<<<n_views, kViewSumThreads, 0, s>>>(partial, block_prefix, cams, 1.0 / 3.0, loss);
   return launched();
 }
 

@@ -17,7 +17,8 @@ namespace ocgs {
 namespace {
 
 constexpr int kRegThreads = 256;
-constexpr int kNcUnroll = 2;  // pixels per thread whose stencil loads are in flight together
+constexpr int kDistLoads = 4;  // pixels per thread of the distortion whose loads are in flight together
+constexpr int kNcUnroll = 2;   // pixels per thread whose stencil loads are in flight together
 
 struct Block {
   int v;
@@ -50,20 +51,40 @@ __global__ void __launch_bounds__(kRegThreads) depth_distortion_kernel(
   const DevCam& cam = cams[b.v];
   const float k = weight / ((float)cam.W * (float)cam.H);
   CompSum acc[1];
-  for (int64_t i = b.lo + threadIdx.x; i < b.hi; i += kRegThreads) {
-    const int64_t p = cam.pix_offset + i;
-    const float A = alpha[p], D = depth[p], Q = depth2[p];
-    // A Q - D^2 from the exact products, so that its cancellation (the blended depths
-    // close together) costs no accuracy: (aq + ea) - (dd + ed), the leading difference
-    // kept exactly by two_sum
-    float ea, ed, es;
-    const float aq = two_prod(A, Q, ea), dd = two_prod(D, D, ed);
-    const float s0 = two_sum(aq, -dd, es);
-    acc[0].add(2.f * s0, 2.f * __fadd_rn(es, __fsub_rn(ea, ed)));
-    if (d_alpha) {
-      d_alpha[p] += k * 2.f * Q;
-      d_depth[p] += k * -4.f * D;
-      d_depth2[p] += k * 2.f * A;
+  // kDistLoads pixels per round, every load of the round issued before any is used
+  for (int64_t i0 = b.lo + threadIdx.x; i0 < b.hi; i0 += kDistLoads * kRegThreads) {
+    float A[kDistLoads], D[kDistLoads], Q[kDistLoads], ga[kDistLoads], gd[kDistLoads], gq[kDistLoads];
+#pragma unroll
+    for (int u = 0; u < kDistLoads; ++u) {
+      const int64_t i = i0 + u * kRegThreads, p = cam.pix_offset + i;
+      A[u] = D[u] = Q[u] = ga[u] = gd[u] = gq[u] = 0.f;
+      if (i < b.hi) {
+        A[u] = alpha[p];
+        D[u] = depth[p];
+        Q[u] = depth2[p];
+        if (d_alpha) {
+          ga[u] = d_alpha[p];
+          gd[u] = d_depth[p];
+          gq[u] = d_depth2[p];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kDistLoads; ++u) {
+      const int64_t i = i0 + u * kRegThreads, p = cam.pix_offset + i;
+      if (i >= b.hi) break;
+      // A Q - D^2 from the exact products, so that its cancellation (the blended depths
+      // close together) costs no accuracy: (aq + ea) - (dd + ed), the leading difference
+      // kept exactly by two_sum
+      float ea, ed, es;
+      const float aq = two_prod(A[u], Q[u], ea), dd = two_prod(D[u], D[u], ed);
+      const float s0 = two_sum(aq, -dd, es);
+      acc[0].add(2.f * s0, 2.f * __fadd_rn(es, __fsub_rn(ea, ed)));
+      if (d_alpha) {
+        d_alpha[p] = ga[u] + k * 2.f * Q[u];
+        d_depth[p] = gd[u] + k * -4.f * D[u];
+        d_depth2[p] = gq[u] + k * 2.f * A[u];
+      }
     }
   }
   block_comp_sums<kRegThreads, 1>(acc, partial + blockIdx.x);
@@ -88,7 +109,8 @@ __device__ __forceinline__ Pt surface_point(float A, float D, const DevCam& cam,
 }
 
 // Alpha and depth of the five stencil pixels (centre, x + 1, x - 1, y + 1, y - 1) of
-// pixel (x, y) and its accumulated normal, NaN alpha outside the image.
+// pixel (x, y) and its accumulated normal, NaN alpha outside the image.  A centre that
+// does not count (its alpha A0 at most a_min) loads nothing more.
 struct Stencil {
   float A[5], D[5];
   float3 Nr;
@@ -98,10 +120,13 @@ __host__ __device__ constexpr int stencil_dy(int j) { return (j == 3) - (j == 4)
 
 __device__ __forceinline__ void load_stencil(const float* __restrict__ alpha, const float* __restrict__ depth,
                                              const float* __restrict__ normal, const DevCam& cam, int x, int y,
-                                             Stencil& st) {
+                                             float A0, float a_min, Stencil& st) {
   const int64_t p = cam.pix_offset + (int64_t)y * cam.W + x;
+  st.A[0] = A0;
+  if (!(A0 > a_min)) return;
+  st.D[0] = depth[p];
 #pragma unroll
-  for (int j = 0; j < 5; ++j) {
+  for (int j = 1; j < 5; ++j) {
     const int xx = x + stencil_dx(j), yy = y + stencil_dy(j);
     st.A[j] = __int_as_float(0x7fc00000);
     st.D[j] = 0.f;
@@ -120,7 +145,8 @@ __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
   return make_float3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
 
-// gmap [P][6] (or NULL): d(weight term)/d(dx) and d/d(dy) of the pixel's central differences
+// gmap [P][6] (or NULL): d(weight term)/d(dx) and d/d(dy) of the pixel's central differences,
+// written for the pixels above a_min only (the gather reads no other)
 __global__ void __launch_bounds__(kRegThreads, 4) normal_consistency_kernel(
     const float* __restrict__ alpha, const float* __restrict__ depth, const float* __restrict__ normal,
     const DevCam* __restrict__ cams, int n_views, const int* __restrict__ block_prefix, float weight, float a_min,
@@ -133,17 +159,27 @@ __global__ void __launch_bounds__(kRegThreads, 4) normal_consistency_kernel(
   // kNcUnroll pixels per round, every load of the round issued before any is used
   for (int64_t i0 = b.lo + threadIdx.x; i0 < b.hi; i0 += kNcUnroll * kRegThreads) {
     Stencil st[kNcUnroll];
+    float A0[kNcUnroll];
 #pragma unroll
     for (int u = 0; u < kNcUnroll; ++u) {
       const int64_t i = i0 + u * kRegThreads;
-      if (i < b.hi) load_stencil(alpha, depth, normal, cam, (int)(i % cam.W), (int)(i / cam.W), st[u]);
+      A0[u] = i < b.hi ? alpha[cam.pix_offset + i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kNcUnroll; ++u) {
+      const int64_t i = i0 + u * kRegThreads;
+      if (i < b.hi)
+        load_stencil(alpha, depth, normal, cam, (int)((uint32_t)i % (uint32_t)cam.W), (int)((uint32_t)i / (uint32_t)cam.W),
+                     A0[u], a_min, st[u]);
     }
 #pragma unroll
     for (int u = 0; u < kNcUnroll; ++u) {
       const int64_t i = i0 + u * kRegThreads;
       if (i >= b.hi) break;
+      // a pixel without coverage counts in no stencil, so its map entry is never read
+      if (!(A0[u] > a_min)) continue;
       const int64_t p = cam.pix_offset + i;
-      const int x = (int)(i % cam.W), y = (int)(i / cam.W);
+      const int x = (int)((uint32_t)i % (uint32_t)cam.W), y = (int)((uint32_t)i / (uint32_t)cam.W);
       float g6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const Pt c = surface_point(st[u].A[0], st[u].D[0], cam, x, y, a_min);
       const Pt xp = surface_point(st[u].A[1], st[u].D[1], cam, x + 1, y, a_min);
@@ -218,12 +254,15 @@ __global__ void __launch_bounds__(kRegThreads, 4) normal_consistency_gather_kern
       for (int j = 0; j < 12; ++j) m[u][j] = 0.f;
       if (i < b.hi && A[u] > a_min) {  // else not a point of any counted stencil
         const int64_t q = cam.pix_offset + i;
-        const int x = (int)(i % cam.W), y = (int)(i / cam.W);
+        const int x = (int)((uint32_t)i % (uint32_t)cam.W), y = (int)((uint32_t)i / (uint32_t)cam.W);
         const int64_t nb[4] = {q - 1, q + 1, q - cam.W, q + cam.W};
         const bool in[4] = {x > 0, x + 1 < cam.W, y > 0, y + 1 < cam.H};
+        float nbA[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) nbA[n] = in[n] ? alpha[nb[n]] : 0.f;
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-          if (in[n]) {
+          if (in[n] && nbA[n] > a_min) {  // else it counts in no stencil and has no entry
             const float* e = gmap + 6 * nb[n] + (n < 2 ? 0 : 3);
             m[u][3 * n] = e[0];
             m[u][3 * n + 1] = e[1];
@@ -237,7 +276,7 @@ __global__ void __launch_bounds__(kRegThreads, 4) normal_consistency_gather_kern
       const int64_t i = i0 + u * kRegThreads;
       if (i >= b.hi || !(A[u] > a_min)) continue;
       const int64_t q = cam.pix_offset + i;
-      const int x = (int)(i % cam.W), y = (int)(i / cam.W);
+      const int x = (int)((uint32_t)i % (uint32_t)cam.W), y = (int)((uint32_t)i / (uint32_t)cam.W);
       // the same sums as term by term over the present neighbours (an absent one adds +0)
       float3 g = make_float3(0.f, 0.f, 0.f);
       g.x += m[u][0]; g.y += m[u][1]; g.z += m[u][2];

@@ -90,6 +90,28 @@ __global__ void __launch_bounds__(kThreadsSsim, 4) ssim_stats_kernel(
   const int col = tid % kT, r0 = (tid / kT) * kSeg;  // second pass: 4 rows of one column
   CompSum sums[2];  // S over all values, S over the mask values
   int cnt = 0;      // mask values
+  // A patch without a mask pixel holds two zero images: S is its value at zero
+  // statistics for every pixel of the tile, and the tile's adjoint maps are not written,
+  // since no pixel whose gradient is not masked away lies within the window's reach of
+  // them.  Three tiles in four of an object-centric view are such tiles.
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < kPatchLoads; ++k) {
+    const int i = tid + k * kThreadsSsim;
+    const int gy = y0 - kR + i / kP, gx = x0 - kR + i % kP;
+    if (i < kP * kP && gy >= 0 && gy < cam.H && gx >= 0 && gx < cam.W)
+      any = any || mask[cam.pix_offset + (int64_t)gy * cam.W + gx] != 0;
+  }
+  if (!__syncthreads_or(any ? 1 : 0)) {
+    if (tid == 0) {
+      const int w = min(kT, cam.W - x0), h = min(kT, cam.H - y0);
+      const float S = kC1 * kC2 * (1.f / (kC1 * kC2));  // ssim_value at zero statistics
+      partial[3 * blockIdx.x] = 3.0 * (double)(w * h) * (double)S;
+      partial[3 * blockIdx.x + 1] = 0.0;
+      partial[3 * blockIdx.x + 2] = 0.0;
+    }
+    return;
+  }
   for (int c = 0; c < 3; ++c) {
     if (c > 0) __syncthreads();  // the previous channel's second pass is done with sx and h
     // the patch in groups of kLoadGroup values per thread, each group's loads issued
@@ -220,6 +242,14 @@ __global__ void __launch_bounds__(kThreadsSsim) ssim_grad_kernel(
   const int tid = threadIdx.x;
   const int col = tid % kT, r0 = (tid / kT) * kSeg;
   const float coef = -weight / (3.f * (float)cam.W * (float)cam.H);
+  // x2 = R M: a tile without a mask pixel has no gradient to add
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < kSeg; ++k) {
+    const int gx = x0 + col, gy = y0 + r0 + k;
+    if (gx < cam.W && gy < cam.H) any = any || mask[cam.pix_offset + (int64_t)gy * cam.W + gx] != 0;
+  }
+  if (!__syncthreads_or(any ? 1 : 0)) return;
   for (int c = 0; c < 3; ++c) {
     if (c > 0) __syncthreads();
     // each plane's patch in one group: its loads in flight together, then the stores
@@ -301,30 +331,55 @@ __global__ void __launch_bounds__(kViewSumThreads) ssim_final_kernel(const doubl
 }
 
 // partial[2 b]: sum of squared masked differences, partial[2 b + 1]: mask values
-__global__ void __launch_bounds__(256) psnr_partial_kernel(const float* __restrict__ rgb,
+// Bound by the FP64 rate (about two operations per cycle and SM) where the mask is: blocks of
+// 1024 pixels spread the masked ones over the SMs (blocks of 4096 took 36 us for one view of
+// 717k pixels: X_PSNR), and the loads of a thread's four pixels are in flight together.
+constexpr int kPsnrThreads = 256, kPsnrLoads = kPsnrBlockPixels / kPsnrThreads;
+__global__ void __launch_bounds__(kPsnrThreads) psnr_partial_kernel(const float* __restrict__ rgb,
                                                            const float* __restrict__ target,
                                                            const uint8_t* __restrict__ mask,
                                                            const DevCam* __restrict__ cams, int n_views,
                                                            const int* __restrict__ block_prefix,
                                                            double* __restrict__ partial) {
-  __shared__ double red[2][8];
+  __shared__ double red[2][kPsnrThreads / 32];
   const int b = blockIdx.x;
   const int v = view_of_tile(block_prefix, n_views, b);
   const DevCam& cam = cams[v];
   const int64_t npix = (int64_t)cam.W * cam.H;
-  const int64_t lo = (int64_t)(b - block_prefix[v]) * kLossBlockPixels;
-  const int64_t hi = (lo + kLossBlockPixels < npix) ? lo + kLossBlockPixels : npix;
-  double se = 0.0, n = 0.0;
-  for (int64_t k = lo + threadIdx.x; k < hi; k += 256) {
-    const int64_t p = cam.pix_offset + k;
-    if (!mask[p]) continue;
+  const int64_t lo = (int64_t)(b - block_prefix[v]) * kPsnrBlockPixels;
+  const int64_t hi = (lo + kPsnrBlockPixels < npix) ? lo + kPsnrBlockPixels : npix;
+  double se = 0.0;
+  int pixels = 0;
+  {
+    const int64_t k0 = lo + threadIdx.x;
+    bool m[kPsnrLoads];
+    float x[kPsnrLoads][3], y[kPsnrLoads][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double d = (double)target[3 * p + c] - (double)rgb[3 * p + c];
-      se += d * d;
+    for (int u = 0; u < kPsnrLoads; ++u) {
+      const int64_t k = k0 + u * kPsnrThreads;
+      m[u] = k < hi && mask[cam.pix_offset + k];
     }
-    n += 3.0;
+#pragma unroll
+    for (int u = 0; u < kPsnrLoads; ++u) {
+      const int64_t p = cam.pix_offset + k0 + u * kPsnrThreads;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        x[u][c] = m[u] ? target[3 * p + c] : 0.f;
+        y[u][c] = m[u] ? rgb[3 * p + c] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPsnrLoads; ++u) {
+      if (!m[u]) continue;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double d = (double)x[u][c] - (double)y[u][c];
+        se += d * d;
+      }
+      ++pixels;
+    }
   }
+  double n = 3.0 * (double)pixels;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     se += __shfl_down_sync(0xffffffffu, se, o);
@@ -337,7 +392,7 @@ __global__ void __launch_bounds__(256) psnr_partial_kernel(const float* __restri
   __syncthreads();
   if (threadIdx.x < 2) {
     double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+    for (int w = 0; w < kPsnrThreads / 32; ++w) t += red[threadIdx.x][w];
     partial[2 * b + threadIdx.x] = t;
   }
 }
@@ -392,7 +447,7 @@ cudaError_t launch_masked_psnr(const float* rgb, const float* target, const uint
                                int n_views, const int* block_prefix, int n_blocks, double max_i, double* partial,
                                double* psnr, cudaStream_t s) {
   if (n_blocks > 0) {
-    psnr_partial_kernel<<<n_blocks, 256, 0, s>>>(rgb, target, mask, cams, n_views, block_prefix, partial);
+    psnr_partial_kernel<<<n_blocks, kPsnrThreads, 0, s>>>(rgb, target, mask, cams, n_views, block_prefix, partial);
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
   }
