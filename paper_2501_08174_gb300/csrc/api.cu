@@ -1184,21 +1184,16 @@ ocgs_status ocgs_prune(ocgs_ctx* ctx, const float* score, float threshold, const
   cudaStream_t s = ctx->stream;
   const uint32_t n = (uint32_t)in->n;
   Arena tmp(ctx);
-  uint32_t *keep, *keep_pos, *border, *border_pos;
-  CK(tmp.alloc(&keep, n));
-  CK(tmp.alloc(&keep_pos, n));
-  CK(tmp.alloc(&border, n));
-  CK(tmp.alloc(&border_pos, n));
-  char* scratch;
-  CK(tmp.alloc(&scratch, scan_scratch_bytes(n)));
+  uint32_t *words, *done;
+  Block b;
+  b.add(&words, prune_words(n));
+  b.zeroed(&done, 1);
+  CK(b.alloc(tmp, s));
   uint32_t* totals = reinterpret_cast<uint32_t*>(ctx->d_scalar);
   StageTimer t(ctx, OCGS_STAGE_PRUNE);
-  CK(launch_prune_flags(score, n, threshold, keep, border, s));
-  CK(scan_exclusive_u32(keep, keep_pos, n, totals, scratch, s));
-  CK(scan_exclusive_u32(border, border_pos, n, totals + 1, scratch, s));
   GaussOut go{out->xyz, out->quat, out->scale, out->opacity, out->sh};
-  CK(launch_prune_compact(gptrs(in), n, in->sh_degree, keep, keep_pos, border, border_pos, go,
-                          borderline_cap > 0 ? borderline : nullptr, borderline_cap, s));
+  CK(launch_prune(score, n, threshold, gptrs(in), in->sh_degree, go, borderline_cap > 0 ? borderline : nullptr,
+                  borderline_cap, words, done, totals, s));
   t.stop();
   CK(cudaMemcpyAsync(ctx->h_scalar, totals, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));

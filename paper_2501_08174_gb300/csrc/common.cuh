@@ -356,13 +356,6 @@ size_t depth_sort_scratch_bytes(uint32_t n);
 cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint32_t* order_alt, uint32_t n,
                        uint32_t* n_valid, void* scratch, cudaStream_t s);
 
-// exclusive scan of n uint64 values (in may equal out); the total is written to *d_total.
-size_t scan_scratch_bytes(uint32_t n);
-cudaError_t scan_exclusive_u64(const uint64_t* in, uint64_t* out, uint32_t n, uint64_t* d_total,
-                               void* scratch, cudaStream_t s);
-cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* d_total,
-                               void* scratch, cudaStream_t s);
-
 // Binning of the depth order (entries order[0 .. min(n, *d_n))) in work units of consecutive
 // entries.  unit_base [unit_base_words(n)]: first pair of each unit, *total = the pairs (row_runs
 // over every record's candidate rows).  With n32, *n32 = min(*total, cap), and kStatusCapacity is
@@ -462,7 +455,6 @@ struct RasterBwdArgs {
 };
 cudaError_t launch_raster_backward(const RasterBwdArgs& a, int tile_w, int tile_h, int ppt, int batch,
                                    cudaStream_t s);
-constexpr int kPsnrBlockPixels = 1024;
 // sum of the per-pixel blended-prefix lengths (the pairs both passes must evaluate)
 cudaError_t launch_sum_u32(const uint32_t* v, int64_t n, unsigned long long* out, cudaStream_t s);
 
@@ -470,6 +462,7 @@ cudaError_t launch_background_loss(const float* alpha, const uint8_t* mask, cons
                                    int n_views, const int* block_prefix, int n_blocks, float gamma,
                                    double* partial, double* loss, float* d_alpha, cudaStream_t s);
 constexpr int kLossBlockPixels = 4096;
+constexpr int kPsnrBlockPixels = 1024;
 
 // Packed FP32x2 arithmetic: pfma / pmul / padd round each lane as the scalar
 // operation does, so a pair gives two scalar results bit for bit whether it runs
@@ -591,12 +584,13 @@ cudaError_t launch_masked_l1(const float* rgb, const float* target, const uint8_
                              int n_views, const int* block_prefix, int n_blocks, float weight, double* partial,
                              double* loss, float* d_rgb, cudaStream_t s);
 
-cudaError_t launch_prune_flags(const float* score, uint32_t n, float threshold, uint32_t* keep,
-                               uint32_t* border, cudaStream_t s);
-cudaError_t launch_prune_compact(const GaussPtrs& in, uint32_t n, int sh_degree, const uint32_t* keep,
-                                 const uint32_t* keep_pos, const uint32_t* border,
-                                 const uint32_t* border_pos, GaussOut out, int64_t* border_idx,
-                                 int64_t border_cap, cudaStream_t s);
+// Keep-set {score > threshold}, in order: kept rows of every parameter array into out, the
+// indices with |score - threshold| <= 1e-6 into border_idx (the first border_cap of them), both
+// numbers into n_out[0], n_out[1].  words: prune_words(n); done: one zeroed word.
+size_t prune_words(uint32_t n);
+cudaError_t launch_prune(const float* score, uint32_t n, float threshold, const GaussPtrs& in, int sh_degree,
+                         GaussOut out, int64_t* border_idx, int64_t border_cap, uint32_t* words, uint32_t* done,
+                         uint32_t* n_out, cudaStream_t s);
 
 // Adam (adam.cu): one segment per parameter array
 struct AdamSeg {

@@ -1,11 +1,12 @@
 // Background loss (Eq. 1) with its fused adjoint, and the pruning keep-set
 // compaction (Sec. 4.3).
-#include "common.cuh"
+#include "lookback.cuh"
 #include "ocgs.h"
 
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 namespace ocgs {
 namespace {
@@ -111,35 +112,149 @@ __global__ void __launch_bounds__(kViewSumThreads) bg_loss_final_kernel(const do
   if (threadIdx.x == 0) loss[v] = t / ((double)cams[v].W * (double)cams[v].H) * scale;
 }
 
-__global__ void prune_flags_kernel(const float* __restrict__ score, uint32_t n, float tau,
-                                   uint32_t* __restrict__ keep, uint32_t* __restrict__ border) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float s = score[i];
-  keep[i] = s > tau ? 1u : 0u;
-  border[i] = fabsf(s - tau) <= 1e-6f ? 1u : 0u;
+// ----------------------------------------------------------------------------- pruning
+using namespace lookback;
+
+constexpr int kPruneThreads = 256;  // Gaussians per block
+
+// Rows list[0 .. kept) of an array of W floats per Gaussian, to the rows from base on: the
+// block's kept rows are contiguous in the output, so the stores are coalesced, and each
+// source row is read by neighbouring lanes.
+template <int W, typename V>
+__device__ __forceinline__ void copy_rows_as(const float* __restrict__ in, float* __restrict__ out, int64_t i0,
+                                             const uint16_t* list, int kept, int64_t base) {
+  constexpr int Q = W * sizeof(float) / sizeof(V);  // vectors per row
+  const V* src = reinterpret_cast<const V*>(in) + i0 * Q;
+  V* dst = reinterpret_cast<V*>(out) + base * Q;
+  constexpr int kBatch = Q >= 4 ? 4 : 1;  // loads in flight per thread
+  const int total = kept * Q;
+  for (int k0 = threadIdx.x; k0 < total; k0 += kBatch * kPruneThreads) {
+    V v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int k = k0 + u * kPruneThreads;
+      if (k < total) v[u] = __ldcs(src + ((int)list[k / Q] * Q + k % Q));
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int k = k0 + u * kPruneThreads;
+      if (k < total) __stcs(dst + k, v[u]);
+    }
+  }
+}
+template <int W>
+__device__ __forceinline__ void copy_rows(const float* __restrict__ in, float* __restrict__ out, int64_t i0,
+                                          const uint16_t* list, int kept, int64_t base) {
+  const uintptr_t both = reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out);
+  if (W % 4 == 0 && both % 16 == 0) copy_rows_as<W, typename std::conditional<W % 4 == 0, float4, float>::type>(in, out, i0, list, kept, base);
+  else if (W % 2 == 0 && both % 8 == 0) copy_rows_as<W, typename std::conditional<W % 2 == 0, float2, float>::type>(in, out, i0, list, kept, base);
+  else copy_rows_as<W, float>(in, out, i0, list, kept, base);
 }
 
-__global__ void prune_compact_kernel(GaussPtrs in, uint32_t n, int k3, const uint32_t* __restrict__ keep,
-                                     const uint32_t* __restrict__ keep_pos, const uint32_t* __restrict__ border,
-                                     const uint32_t* __restrict__ border_pos, GaussOut out,
-                                     int64_t* __restrict__ border_idx, int64_t border_cap) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (keep[i]) {
-    const int64_t j = keep_pos[i];
-    out.xyz[3 * j + 0] = in.xyz[3 * (int64_t)i + 0];
-    out.xyz[3 * j + 1] = in.xyz[3 * (int64_t)i + 1];
-    out.xyz[3 * j + 2] = in.xyz[3 * (int64_t)i + 2];
-    reinterpret_cast<float4*>(out.quat)[j] = reinterpret_cast<const float4*>(in.quat)[i];
-    reinterpret_cast<float2*>(out.scale)[j] = reinterpret_cast<const float2*>(in.scale)[i];
-    out.opacity[j] = in.opacity[i];
-    for (int k = 0; k < k3; ++k) out.sh[j * k3 + k] = in.sh[(int64_t)i * k3 + k];
+__device__ __forceinline__ bool is_kept(float s, float tau) { return s > tau; }
+__device__ __forceinline__ bool is_border(float s, float tau) { return fabsf(s - tau) <= 1e-6f; }
+
+// Kept and border counts of every kPruneThreads Gaussians, one warp each, into kept[tiles] and
+// border[tiles]; the last block to finish turns both into exclusive prefixes and writes the
+// totals to n_out.
+__global__ void __launch_bounds__(kPruneThreads) prune_count_kernel(const float* __restrict__ score, uint32_t n,
+                                                                    float tau, uint32_t tiles, uint32_t* kept,
+                                                                    uint32_t* border, uint32_t* done,
+                                                                    uint32_t* __restrict__ n_out) {
+  constexpr int kWarps = kPruneThreads / 32, kRounds = kPruneThreads / 32;
+  __shared__ uint32_t s_w[kWarps];
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tile = blockIdx.x * kWarps + warp;
+  if (tile < tiles) {
+    const int64_t i0 = (int64_t)tile * kPruneThreads + lane;
+    float s[kRounds];
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) s[r] = i0 + 32 * r < n ? score[i0 + 32 * r] : __int_as_float(0x7fc00000);
+    uint32_t ck = 0, cb = 0;  // NaN is neither kept nor at the border
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      ck += (uint32_t)__popc(__ballot_sync(kFull, is_kept(s[r], tau)));
+      cb += (uint32_t)__popc(__ballot_sync(kFull, is_border(s[r], tau)));
+    }
+    if (lane == 0) {
+      kept[tile] = ck;
+      border[tile] = cb;
+    }
   }
-  if (border_idx && border[i]) {
-    const int64_t j = border_pos[i];
-    if (j < border_cap) border_idx[j] = i;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const uint32_t per = (tiles + kPruneThreads - 1) / kPruneThreads;
+  const uint32_t t0 = min(tiles, threadIdx.x * per), t1 = min(tiles, t0 + per);
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    uint32_t* c = which ? border : kept;
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t t = t0; t < t1; ++t) sum += __ldcg(c + t);
+    const uint32_t inc = warp_inclusive_scan<uint32_t>(sum, lane);
+    __syncthreads();  // s_w of the other count has been read
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t run = inc - sum;
+    for (int w = 0; w < warp; ++w) run += s_w[w];
+#pragma unroll 8
+    for (uint32_t t = t0; t < t1; ++t) {
+      const uint32_t x = __ldcg(c + t);
+      c[t] = run;
+      run += x;
+    }
+    if (threadIdx.x == kPruneThreads - 1) n_out[which] = run;
   }
+}
+
+// Stable compaction: a block lists its kept Gaussians and copies their rows.
+//
+// What bounds it: HBM (464 bytes per kept Gaussian of degree 3).  One thread per Gaussian
+// copying its 48 coefficients at a stride of 192 bytes took 292 us for 1M Gaussians of which
+// 69 % are kept; finding the positions by a look-back inside this kernel 143 us (its blocks
+// waited for one another more than they copied); this form 72 us with its count kernel.
+template <int DEG>
+__global__ void __launch_bounds__(kPruneThreads) prune_copy_kernel(const float* __restrict__ score, uint32_t n,
+                                                                   float tau, const GaussPtrs in, GaussOut out,
+                                                                   int64_t* __restrict__ border_idx,
+                                                                   int64_t border_cap,
+                                                                   const uint32_t* __restrict__ kept_before,
+                                                                   const uint32_t* __restrict__ border_before) {
+  constexpr int kWarps = kPruneThreads / 32;
+  __shared__ uint16_t s_list[kPruneThreads];
+  __shared__ uint32_t s_k[kWarps], s_b[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t i0 = (int64_t)blockIdx.x * kPruneThreads, i = i0 + threadIdx.x;
+  const uint32_t bk = kept_before[blockIdx.x], bb = border_before[blockIdx.x];
+  const float s = i < n ? score[i] : __int_as_float(0x7fc00000);
+  const bool keep = is_kept(s, tau), border = is_border(s, tau);
+  const unsigned mk = __ballot_sync(kFull, keep), mb = __ballot_sync(kFull, border);
+  if (lane == 0) {
+    s_k[warp] = (uint32_t)__popc(mk);
+    s_b[warp] = (uint32_t)__popc(mb);
+  }
+  __syncthreads();
+  uint32_t ok = (uint32_t)__popc(mk & lt), ob = (uint32_t)__popc(mb & lt), kept = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    ok += w < warp ? s_k[w] : 0u;
+    ob += w < warp ? s_b[w] : 0u;
+    kept += s_k[w];
+  }
+  if (keep) s_list[ok] = (uint16_t)threadIdx.x;
+  if (border && border_idx && (int64_t)(bb + ob) < border_cap) border_idx[bb + ob] = i;
+  __syncthreads();
+  copy_rows<3 * (DEG + 1) * (DEG + 1)>(in.sh, out.sh, i0, s_list, (int)kept, bk);
+  copy_rows<4>(in.quat, out.quat, i0, s_list, (int)kept, bk);
+  copy_rows<3>(in.xyz, out.xyz, i0, s_list, (int)kept, bk);
+  copy_rows<2>(in.scale, out.scale, i0, s_list, (int)kept, bk);
+  copy_rows<1>(in.opacity, out.opacity, i0, s_list, (int)kept, bk);
 }
 
 }  // namespace
@@ -171,21 +286,27 @@ cudaError_t launch_masked_l1(const float* rgb, const float* target, const uint8_
   return launched();
 }
 
-cudaError_t launch_prune_flags(const float* score, uint32_t n, float threshold, uint32_t* keep,
-                               uint32_t* border, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  prune_flags_kernel<<<(n + 255) / 256, 256, 0, s>>>(score, n, threshold, keep, border);
-  return launched();
-}
+size_t prune_words(uint32_t n) { return 2 * (((size_t)n + kPruneThreads - 1) / kPruneThreads); }
 
-cudaError_t launch_prune_compact(const GaussPtrs& in, uint32_t n, int sh_degree, const uint32_t* keep,
-                                 const uint32_t* keep_pos, const uint32_t* border,
-                                 const uint32_t* border_pos, GaussOut out, int64_t* border_idx,
-                                 int64_t border_cap, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  const int k3 = 3 * (sh_degree + 1) * (sh_degree + 1);
-  prune_compact_kernel<<<(n + 255) / 256, 256, 0, s>>>(in, n, k3, keep, keep_pos, border, border_pos, out,
-                                                       border_idx, border_cap);
+cudaError_t launch_prune(const float* score, uint32_t n, float threshold, const GaussPtrs& in, int sh_degree,
+                         GaussOut out, int64_t* border_idx, int64_t border_cap, uint32_t* words, uint32_t* done,
+                         uint32_t* n_out, cudaStream_t s) {
+  if (n == 0) return cudaMemsetAsync(n_out, 0, 2 * sizeof(uint32_t), s);
+  const uint32_t tiles = (uint32_t)(((uint64_t)n + kPruneThreads - 1) / kPruneThreads);
+  uint32_t *kept = words, *border = words + tiles;
+  prune_count_kernel<<<(tiles + kPruneThreads / 32 - 1) / (kPruneThreads / 32), kPruneThreads, 0, s>>>(
+      score, n, threshold, tiles, kept, border, done, n_out);
+  const cudaError_t e = launched();
+  if (e != cudaSuccess) return e;
+#define OCGS_PRUNE(D) \
+  prune_copy_kernel<D><<<tiles, kPruneThreads, 0, s>>>(score, n, threshold, in, out, border_idx, border_cap, kept, border)
+  switch (sh_degree) {
+    case 0: OCGS_PRUNE(0); break;
+    case 1: OCGS_PRUNE(1); break;
+    case 2: OCGS_PRUNE(2); break;
+    default: OCGS_PRUNE(3); break;
+  }
+#undef OCGS_PRUNE
   return launched();
 }
 
