@@ -8,132 +8,22 @@
 // stably sorted by global tile id.  Within a tile the list is therefore in
 // ascending (depth, Gaussian index) order, and only ceil(log2 tiles) key bits
 // are sorted per pair instead of tile+depth bits.
-#include "common.cuh"
+#include "lookback.cuh"
 
 #include <algorithm>
 #include <type_traits>
 
 namespace ocgs {
 namespace {
-
-constexpr int kBlock = 256;
-constexpr int kItems = 16;
-constexpr int kChunk = kBlock * kItems;  // items per block in scans and sort passes
-constexpr unsigned kFull = 0xffffffffu;
-
-template <typename T>
-__device__ __forceinline__ T warp_inclusive_scan(T v, int lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const T t = __shfl_up_sync(kFull, v, o);
-    if (lane >= o) v += t;
-  }
-  return v;
-}
-
-// ------------------------------------------------------------------ scan
-template <typename T>
-__global__ void __launch_bounds__(kBlock) scan_reduce_kernel(const T* __restrict__ in, uint32_t n,
-                                                             T* __restrict__ block_sums) {
-  __shared__ T warp_sums[kBlock / 32];
-  const uint32_t base = blockIdx.x * kChunk;
-  T s = 0;
-#pragma unroll 4
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = base + j * kBlock + threadIdx.x;
-    if (k < n) s += in[k];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) warp_sums[warp] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    T t = 0;
-    for (int w = 0; w < kBlock / 32; ++w) t += warp_sums[w];
-    block_sums[blockIdx.x] = t;
-  }
-}
-
-// exclusive scan of one chunk per block, each warp owning a contiguous 32*kItems slice
-template <typename T>
-__global__ void __launch_bounds__(kBlock) scan_chunk_kernel(const T* in, T* out, uint32_t n,
-                                                            const T* __restrict__ block_offsets,
-                                                            T* __restrict__ d_total) {
-  __shared__ T warp_tot[kBlock / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t wbase = blockIdx.x * kChunk + warp * 32 * kItems;
-  T vals[kItems];
-  T run = 0;
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    const T x = k < n ? in[k] : T(0);
-    const T inc = warp_inclusive_scan<T>(x, lane);
-    vals[j] = run + inc - x;  // exclusive within the warp slice
-    run += __shfl_sync(kFull, inc, 31);
-  }
-  if (lane == 0) warp_tot[warp] = run;
-  __syncthreads();
-  T off = block_offsets ? block_offsets[blockIdx.x] : T(0);
-  T tot = 0;
-  for (int w = 0; w < kBlock / 32; ++w) {
-    if (w < warp) off += warp_tot[w];
-    tot += warp_tot[w];
-  }
-#pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t k = wbase + j * 32 + lane;
-    if (k < n) out[k] = off + vals[j];
-  }
-  if (d_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-    const T first = block_offsets ? block_offsets[blockIdx.x] : T(0);
-    *d_total = first + tot;
-  }
-}
-
-template <typename T>
-size_t scan_levels_bytes(uint32_t n) {
-  size_t bytes = 0;
-  while (n > (uint32_t)kChunk) {
-    n = (n + kChunk - 1) / kChunk;
-    bytes += ((size_t)n * sizeof(T) + 255) & ~(size_t)255;
-  }
-  return bytes;
-}
-
-template <typename T>
-cudaError_t scan_exclusive(const T* in, T* out, uint32_t n, T* d_total, char* scratch, cudaStream_t s) {
-  if (n == 0) {
-    if (d_total) return cudaMemsetAsync(d_total, 0, sizeof(T), s);
-    return cudaSuccess;
-  }
-  const uint32_t nb = (n + kChunk - 1) / kChunk;
-  if (nb == 1) {
-    scan_chunk_kernel<T><<<1, kBlock, 0, s>>>(in, out, n, nullptr, d_total);
-    return launched();
-  }
-  T* sums = reinterpret_cast<T*>(scratch);
-  char* rest = scratch + (((size_t)nb * sizeof(T) + 255) & ~(size_t)255);
-  scan_reduce_kernel<T><<<nb, kBlock, 0, s>>>(in, n, sums);
-  cudaError_t e = launched();
-  if (e != cudaSuccess) return e;
-  e = scan_exclusive<T>(sums, sums, nb, nullptr, rest, s);  // in place over the block sums
-  if (e != cudaSuccess) return e;
-  scan_chunk_kernel<T><<<nb, kBlock, 0, s>>>(in, out, n, sums, d_total);
-  return launched();
-}
+using namespace lookback;
 
 // ------------------------------------------------------------------ radix sort
 // Stable LSD sort, one kernel per digit (the single-pass scatter with decoupled
-// look-back of Adinets and Merrill, "Onesweep", 2022): a first kernel reads the
-// keys once and counts the digits of every pass; each pass then reads its items
-// once and writes them once.  A block orders its tile by digit in shared memory,
-// publishes its digit counts and adds up those of the tiles before it until one
-// has published its running total.  Tiles are handed out by a counter, so the
-// tiles a block waits for are resident and never wait for a later one; a wait
-// that reaches kSpinLimit polls all the same is given up, and the block counts
-// the digits of all earlier keys itself, so the result never depends on a wait.
+// look-back of Adinets and Merrill, "Onesweep", 2022; see lookback.cuh): a first
+// kernel reads the keys once and counts the digits of every pass; each pass then
+// reads its items once and writes them once, a block ordering its tile by digit in
+// shared memory.  A look-back that is given up is replaced by counting the digits
+// of all earlier keys.
 //
 // What bounds it: HBM at full size (16 bytes per item and pass), the launch and
 // the look-back latency below about a million items.
@@ -145,14 +35,13 @@ cudaError_t scan_exclusive(const T* in, T* out, uint32_t n, T* d_total, char* sc
 constexpr int kRadixThreads = 384;
 constexpr int kRadixItems = 18;
 constexpr int kRadixBlocks = 3;  // resident per SM
-constexpr int kRadixTile = kRadixThreads * kRadixItems;
 constexpr int kRadixWarps = kRadixThreads / 32;
-#ifndef OCGS_SPIN_LIMIT
-#define OCGS_SPIN_LIMIT (1u << 20)
-#endif
-constexpr uint32_t kSpinLimit = OCGS_SPIN_LIMIT;
-constexpr int kLookBack = 16;  // tiles per round trip of a look-back (4 to 32 measured within 3 %)
-
+static_assert(kRadixThreads * kRadixItems <= kMaxTileCount, "look-back words");
+// Where tiles of 18 items would leave SMs idle, tiles of 4: a pass over few items is the
+// latency of one tile, and that of its serial ranking rounds (a pass over 2,000 records: 8.2
+// -> 5.5 us; the depth sort of 100k: 52 -> 43 us).
+constexpr int kSmallItems = 4;
+constexpr uint32_t kSmallSort = 152u * kRadixThreads * kSmallItems;  // at most one small tile per SM
 // Digits of a sort of n_bits key bits: equal widths of 4 to 8 bits.  (Two digits of 10
 // bits instead of three of 7 took 17.6 against 6.0 ms on 480k tiles: runs of a few items
 // per digit and tile, and four times the look-back words.)
@@ -262,45 +151,6 @@ __global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const Keys ke
   }
 }
 
-// Look-back word of one (tile, digit): 0 = nothing yet, 1 + c = the tile's count c
-// (at most kRadixTile), kRadixTile + 2 + t = the total t of the tiles up to it.
-__device__ __forceinline__ uint32_t load_word(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void store_word(uint32_t* p, uint32_t v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Sum of the tiles before `tile` for this thread's digit (words: the digit's column,
-// R apart).  False if the wait was given up.
-template <int R>
-__device__ __forceinline__ bool look_back(const uint32_t* words, uint32_t tile, uint32_t* excl) {
-  uint32_t sum = 0, polls = 0;
-  int64_t t = (int64_t)tile - 1;
-  while (t >= 0) {
-    uint32_t w[kLookBack];
-#pragma unroll
-    for (int k = 0; k < kLookBack; ++k) w[k] = t - k >= 0 ? load_word(words + (t - k) * R) : 0u;
-    int used = 0;
-#pragma unroll
-    for (int k = 0; k < kLookBack; ++k) {
-      if (used != k || w[k] == 0u) continue;
-      if (w[k] > (uint32_t)kRadixTile + 1u) {
-        *excl = sum + (w[k] - (uint32_t)(kRadixTile + 2));
-        return true;
-      }
-      sum += w[k] - 1u;
-      used = k + 1;
-    }
-    t -= used;
-    if (used == 0 && ++polls > kSpinLimit) return false;
-  }
-  *excl = sum;
-  return true;
-}
-
 // One pass.  Warp w of a block owns the contiguous slice [w * 32 * kRadixItems, ...)
 // of its tile.  The warps first count their digits with shared-memory atomics, so
 // that the tile's counts are published before the ranking: the look-back of the
@@ -310,16 +160,17 @@ __device__ __forceinline__ bool look_back(const uint32_t* words, uint32_t tile, 
 // digit order in shared memory; the tile is written in digit runs, so the global
 // stores are coalesced.  INDEX: the values are the items' indices (vals_in is not
 // read).  DROP: see radix_hist_kernel.
-template <class Keys, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
+template <class Keys, int ITEMS, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
 __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel(
     const Keys keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
     uint32_t* __restrict__ vals_out, uint32_t n, const uint32_t* __restrict__ d_n, int shift,
     const uint32_t* __restrict__ base, uint32_t* words, uint32_t* next_tile) {
+  constexpr int TILE = kRadixThreads * ITEMS;
   constexpr int R = 1 << BITS, PER = (R + kRadixThreads - 1) / kRadixThreads;
   __shared__ uint32_t whist[kRadixWarps][R];
   __shared__ uint32_t gofs[R];  // global position minus tile position of each digit's run
   __shared__ uint32_t s_w[kRadixWarps];
-  __shared__ uint32_t sk[kRadixTile], sv[kRadixTile];
+  __shared__ uint32_t sk[TILE], sv[TILE];
   __shared__ uint32_t s_tile, s_items;
   __shared__ int s_gave_up;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -331,24 +182,24 @@ __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel
   if (d_n) n = min(n, *d_n);
   __syncthreads();
   const uint32_t tile = s_tile;
-  const uint64_t first = (uint64_t)tile * kRadixTile;
+  const uint64_t first = (uint64_t)tile * TILE;
   if (first >= n) return;  // capacity launches: no tile after this one waits for it
-  const uint32_t here = (uint32_t)min((uint64_t)kRadixTile, n - first);
-  const uint32_t slice = (uint32_t)warp * 32 * kRadixItems + lane;
+  const uint32_t here = (uint32_t)min((uint64_t)TILE, n - first);
+  const uint32_t slice = (uint32_t)warp * 32 * ITEMS + lane;
   const unsigned lt = (1u << lane) - 1u;
-  uint32_t key[kRadixItems];
+  uint32_t key[ITEMS];
 #pragma unroll
-  for (int j = 0; j < kRadixItems; ++j) {
+  for (int j = 0; j < ITEMS; ++j) {
     const uint32_t k = slice + j * 32;
     key[j] = k < here ? keys_in((uint32_t)first + k) : 0xffffffffu;
   }
   auto valid = [&](int j) { return slice + j * 32 < here && (!DROP || key[j] != 0xffffffffu); };
 #pragma unroll
-  for (int j = 0; j < kRadixItems; ++j)
+  for (int j = 0; j < ITEMS; ++j)
     if (valid(j)) atomicAdd(&whist[warp][(key[j] >> shift) & (R - 1)], 1u);
-  uint32_t val[kRadixItems];
+  uint32_t val[ITEMS];
 #pragma unroll
-  for (int j = 0; j < kRadixItems; ++j) {
+  for (int j = 0; j < ITEMS; ++j) {
     const uint32_t k = slice + j * 32;
     val[j] = INDEX ? (uint32_t)first + k : k < here ? vals_in[first + k] : 0u;
   }
@@ -365,7 +216,7 @@ __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel
 #pragma unroll
         for (int w = 0; w < kRadixWarps; ++w) c += whist[w][d];
         cnt[k] = c;
-        store_word(words + (size_t)tile * R + d, tile == 0 ? (uint32_t)(kRadixTile + 2) + c : 1u + c);
+        store_word(words + (size_t)tile * R + d, tile == 0 ? total_word(c) : count_word(c));
       }
     }
     e = block_exclusive<PER>(cnt, s_w);
@@ -386,7 +237,7 @@ __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < kRadixItems; ++j) {
+  for (int j = 0; j < ITEMS; ++j) {
     const uint32_t d = (key[j] >> shift) & (R - 1);
     unsigned peers = DROP ? __ballot_sync(kFull, valid(j)) : kFull;
 #pragma unroll
@@ -432,7 +283,7 @@ __global__ void __launch_bounds__(kRadixThreads, kRadixBlocks) radix_pass_kernel
   for (int k = 0; k < PER; ++k) {
     const int d = threadIdx.x * PER + k;
     if (d < R) {
-      if (tile) store_word(words + (size_t)tile * R + d, (uint32_t)(kRadixTile + 2) + excl[k] + cnt[k]);
+      if (tile) store_word(words + (size_t)tile * R + d, total_word(excl[k] + cnt[k]));
       gofs[d] = base[d] + excl[k] - e;
     }
     e += cnt[k];
@@ -736,18 +587,6 @@ __global__ void tile_ranges_kernel(const uint32_t* __restrict__ keys, uint32_t n
 
 }  // namespace
 
-size_t scan_scratch_bytes(uint32_t n) { return scan_levels_bytes<uint64_t>(n) + 256; }
-
-cudaError_t scan_exclusive_u64(const uint64_t* in, uint64_t* out, uint32_t n, uint64_t* d_total,
-                               void* scratch, cudaStream_t s) {
-  return scan_exclusive<uint64_t>(in, out, n, d_total, static_cast<char*>(scratch), s);
-}
-
-cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* d_total,
-                               void* scratch, cudaStream_t s) {
-  return scan_exclusive<uint32_t>(in, out, n, d_total, static_cast<char*>(scratch), s);
-}
-
 namespace {
 
 // Scratch of one sort (zeroed by the caller): digit positions, counters, look-back words.
@@ -757,8 +596,8 @@ struct RadixScratch {
 };
 RadixScratch radix_layout(void* scratch, uint32_t n, int passes, int bits) {
   RadixScratch w;
-  const size_t R = (size_t)1 << bits;
-  w.tiles = ((size_t)n + kRadixTile - 1) / kRadixTile;
+  const size_t R = (size_t)1 << bits, tile = (size_t)kRadixThreads * (n <= kSmallSort ? kSmallItems : kRadixItems);
+  w.tiles = ((size_t)n + tile - 1) / tile;
   w.base = static_cast<uint32_t*>(scratch);
   w.done = w.base + passes * R;
   w.next_tile = w.done + 1;
@@ -770,8 +609,9 @@ RadixScratch radix_layout(void* scratch, uint32_t n, int passes, int bits) {
 template <class Keys, int BITS, int PASSES, bool DROP>
 cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const RadixScratch& w, uint32_t* n_valid,
                         cudaStream_t s) {
-  // about 16 keys per thread, at most four blocks per SM
-  const uint32_t blocks = (uint32_t)std::min<size_t>((size_t)152 * 4, ((size_t)n + 16 * kRadixThreads - 1) / (16 * kRadixThreads));
+  // at least four keys per thread, at most four blocks per SM
+  const size_t per_block = 4 * kRadixThreads;
+  const uint32_t blocks = (uint32_t)std::min<size_t>((size_t)152 * 4, ((size_t)n + per_block - 1) / per_block);
   radix_hist_kernel<Keys, BITS, PASSES, DROP><<<blocks, kRadixThreads, 0, s>>>(k, n, d_n, w.base, w.done, n_valid);
   return launched();
 }
@@ -779,9 +619,11 @@ cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const Ra
 template <class Keys, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
 cudaError_t launch_pass(const Keys& k, const uint32_t* vals, uint32_t* keys_out, uint32_t* vals_out, uint32_t n,
                         const uint32_t* d_n, int p, const RadixScratch& w, cudaStream_t s) {
-  radix_pass_kernel<Keys, BITS, INDEX, DROP, KEYS_OUT><<<(unsigned)w.tiles, kRadixThreads, 0, s>>>(
-      k, vals, keys_out, vals_out, n, d_n, p * BITS, w.base + (size_t)p * (1 << BITS),
-      w.words + (size_t)p * w.tiles * (1 << BITS), w.next_tile + p);
+  auto pass = n <= kSmallSort ? radix_pass_kernel<Keys, kSmallItems, BITS, INDEX, DROP, KEYS_OUT>
+                              : radix_pass_kernel<Keys, kRadixItems, BITS, INDEX, DROP, KEYS_OUT>;
+  pass<<<(unsigned)w.tiles, kRadixThreads, 0, s>>>(k, vals, keys_out, vals_out, n, d_n, p * BITS,
+                                                   w.base + (size_t)p * (1 << BITS),
+                                                   w.words + (size_t)p * w.tiles * (1 << BITS), w.next_tile + p);
   return launched();
 }
 
@@ -896,7 +738,7 @@ constexpr int kScanTile = kThreads * 16;
 __global__ void __launch_bounds__(kThreads) open_scan_kernel(const uint32_t* __restrict__ open, uint32_t n,
                                                              uint32_t* __restrict__ P, uint32_t* __restrict__ open_ids,
                                                              uint32_t* words, uint32_t* next_tile) {
-  static_assert(kScanTile <= kRadixTile, "look-back words");
+  static_assert(kScanTile <= kMaxTileCount, "look-back words");
   constexpr int kItems16 = kScanTile / kThreads;
   __shared__ uint32_t s_w[kThreads / 32];
   __shared__ uint32_t s_tile, s_excl;
@@ -927,11 +769,14 @@ __global__ void __launch_bounds__(kThreads) open_scan_kernel(const uint32_t* __r
     off += w < warp ? s_w[w] : 0u;
     total += s_w[w];
   }
-  if (threadIdx.x == 0) {
-    store_word(words + tile, tile == 0 ? (uint32_t)(kRadixTile + 2) + total : 1u + total);
+  if (warp == 0) {
+    if (lane == 0) store_word(words + tile, tile == 0 ? total_word(total) : count_word(total));
     uint32_t e = 0;
-    if (!look_back<1>(words, tile, &e)) s_gave_up = 1;
-    s_excl = e;
+    const bool found = look_back_warp(words, tile, lane, &e);
+    if (lane == 0) {
+      if (!found) s_gave_up = 1;
+      s_excl = e;
+    }
   }
   __syncthreads();
   if (s_gave_up) {
@@ -944,7 +789,7 @@ __global__ void __launch_bounds__(kThreads) open_scan_kernel(const uint32_t* __r
   }
   const uint32_t excl = s_excl;
   if (threadIdx.x == 0) {
-    if (tile) store_word(words + tile, (uint32_t)(kRadixTile + 2) + excl + total);
+    if (tile) store_word(words + tile, total_word(excl + total));
     if (first + (uint32_t)kScanTile >= n) P[n] = excl + total;
   }
 #pragma unroll
