@@ -329,6 +329,28 @@ bool valid_tile(int tw, int th, int ppt, int batch) {
   return batch == 32 || ((batch == 16 || batch == 64) && small_big);
 }
 
+// Pixels per thread and records per batch a rasterizer launch takes: the options', or fewer
+// pixels per thread where those would leave too few warps to fill the SMs (a warp walks its
+// band's list alone, so a render of few tiles takes as long as its longest list).  No result
+// depends on either.  Measured on 16x16 tiles of one to five views, forward / backward, us:
+//   4 -> 2 below 64 warps per SM (4,864 tiles): 3,072 tiles 311 -> 270 / 546 -> 517, 625 tiles
+//     296 -> 222 / 509 -> 335; at 7,500 tiles 352 against 359 / 699 against 804.
+//   2 -> 1, forward, up to 16 warps per SM (608 tiles): 251 tiles 314 -> 244, 361 tiles 181 ->
+//     168; at 625 tiles 134 against 138.  Backward up to 8 warps per SM (304 tiles), plain grids:
+//     251 tiles 375 -> 337; at 361 tiles 342 against 372, and with a queue 464 against 560.
+struct LaunchShape {
+  int ppt, batch;
+};
+LaunchShape launch_shape(int tw, int th, int ppt, int batch, int64_t tiles, int sm_count, bool persistent,
+                         bool backward) {
+  const int64_t px = tiles * tw * th;
+  LaunchShape s{ppt, batch};
+  if (s.ppt == 4 && px / (32 * 4) < 64ll * sm_count) s.ppt = 2;
+  if (s.ppt == 2 && px / (32 * 2) <= (backward ? (persistent ? 0ll : 8ll) : 16ll) * sm_count) s.ppt = 1;
+  if (!valid_tile(tw, th, s.ppt, s.batch)) s.batch = 32;
+  return s;
+}
+
 GaussPtrs gptrs(const ocgs_gaussians* g) { return GaussPtrs{g->xyz, g->quat, g->scale, g->opacity, g->sh}; }
 
 void free_state(ocgs_fwd_state* st) {
@@ -370,6 +392,7 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
     M = (uint32_t)std::min<double>((double)VN, std::max(1.0, front));
   }
   const int tbits = bits_for((uint64_t)pl.tiles);
+  const LaunchShape shape = launch_shape(tw, th, st->ppt, st->batch, pl.tiles, ctx->sm_count, st->persistent != 0, false);
 
   char* tables;  // the cameras, then the tile prefix
   const size_t cam_bytes = (sizeof(DevCam) * V + 255) & ~(size_t)255;
@@ -513,12 +536,12 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
   ra.score = score;
   ra.tile_order = ids;
   ra.queue = queue;
-  ra.persistent_ctas = st->persistent ? ctx->sm_count * (2048 * st->ppt / (tw * th)) : 0;
+  ra.persistent_ctas = st->persistent ? ctx->sm_count * (2048 * shape.ppt / (tw * th)) : 0;
   ra.open = open;
   ra.done = done;
   {
     StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
-    CK(launch_raster_forward(ra, tw, th, st->ppt, st->batch, img, s));
+    CK(launch_raster_forward(ra, tw, th, shape.ppt, shape.batch, img, s));
   }
 
   uint32_t K2 = 0;
@@ -577,7 +600,7 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
       rb.open = nullptr;
       {
         StageTimer t(ctx, OCGS_STAGE_RASTER_FWD);
-        CK(launch_raster_forward(rb, tw, th, st->ppt, st->batch, img, s));
+        CK(launch_raster_forward(rb, tw, th, shape.ppt, shape.batch, img, s));
       }
     }
   }
@@ -666,7 +689,9 @@ cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_
 // word's capacity bit and the result must then be discarded).
 ocgs_status enqueue_sweep_chunk(ocgs_ctx* ctx, const ocgs_gaussians* g, int V, const DevCam* d_cams,
                                 const int* d_prefix, int64_t n_tiles, SweepWs& w, float* score, cudaStream_t s) {
-  const int tw = ctx->opts.tile_w, th = ctx->opts.tile_h, ppt = ctx->opts.pixels_per_thread;
+  const int tw = ctx->opts.tile_w, th = ctx->opts.tile_h;
+  const LaunchShape shape = launch_shape(tw, th, ctx->opts.pixels_per_thread, ctx->opts.batch, n_tiles, ctx->sm_count,
+                                         ctx->opts.persistent != 0, false);
   const int64_t N = g->n;
   const uint32_t VN = (uint32_t)(N * V);
   const int tbits = bits_for((uint64_t)n_tiles);
@@ -695,9 +720,9 @@ ocgs_status enqueue_sweep_chunk(ocgs_ctx* ctx, const ocgs_gaussians* g, int V, c
     CK(launch_tile_order(w.ranges, nullptr, (uint32_t)n_tiles, w.ids, w.oscratch, s));
     ra.tile_order = w.ids;
     ra.queue = w.queue;
-    ra.persistent_ctas = ctx->sm_count * (2048 * ppt / (tw * th));
+    ra.persistent_ctas = ctx->sm_count * (2048 * shape.ppt / (tw * th));
   }
-  CK(launch_raster_forward(ra, tw, th, ppt, ctx->opts.batch, false, s));
+  CK(launch_raster_forward(ra, tw, th, shape.ppt, shape.batch, false, s));
   return OCGS_OK;
 }
 
@@ -857,9 +882,12 @@ ocgs_status ocgs_render_backward(ocgs_ctx* ctx, const ocgs_fwd_state* st, const 
   Arena tmp(ctx);
   const uint64_t VN = (uint64_t)st->N * st->V;
   float* grad_rec;
-  CK(tmp.alloc(&grad_rec, VN * kGradStride));
+  uint32_t* queue;
   StageTimer t_bwd(ctx, OCGS_STAGE_RASTER_BWD);
-  CK(cudaMemsetAsync(grad_rec, 0, VN * kGradStride * sizeof(float), s));
+  Block b;
+  b.zeroed(&grad_rec, VN * kGradStride);
+  b.zeroed(&queue, 1);
+  CK(b.alloc(tmp, s));
   RasterBwdArgs ba{};
   ba.cams = st->d_cams;
   ba.tile_prefix = st->d_tile_prefix;
@@ -876,14 +904,11 @@ ocgs_status ocgs_render_backward(ocgs_ctx* ctx, const ocgs_fwd_state* st, const 
   ba.d_out = ImgPtrs{d_out->rgb, d_out->alpha, d_out->depth, d_out->normal, d_out->depth2};
   ba.grad_rec = grad_rec;
   ba.tile_order = st->tile_order;
-  uint32_t* queue = nullptr;
-  if (st->persistent) {
-    CK(tmp.alloc(&queue, 1));
-    CK(cudaMemsetAsync(queue, 0, sizeof(uint32_t), s));
-    ba.persistent_ctas = ctx->sm_count * (2048 * st->ppt / (st->tile_w * st->tile_h));
-  }
+  const LaunchShape shape = launch_shape(st->tile_w, st->tile_h, st->ppt, st->batch, st->n_tiles, ctx->sm_count,
+                                         st->persistent != 0, true);
+  if (st->persistent) ba.persistent_ctas = ctx->sm_count * (2048 * shape.ppt / (st->tile_w * st->tile_h));
   ba.queue = queue;
-  CK(launch_raster_backward(ba, st->tile_w, st->tile_h, st->ppt, st->batch, s));
+  CK(launch_raster_backward(ba, st->tile_w, st->tile_h, shape.ppt, shape.batch, s));
   t_bwd.stop();
   GaussOut go{d_params->xyz, d_params->quat, d_params->scale, d_params->opacity, d_params->sh};
   {
