@@ -26,11 +26,6 @@ namespace ocgs {
 constexpr float kRhoCut = 9.0f;            // support cut-off rho <= 9 (3 sigma)
 constexpr float kAlphaMin = 1.0f / 255.0f;  // skip below this opacity
 constexpr float kAlphaMax = 0.99f;          // opacity clamp
-// Opacity below which the 0.99 clamp of alpha never applies: G = exp(-rho/2) <= 1
-// for rho >= 0 (the base-2 exponential's relative error is about 2^-22), so o G <
-// 0.989 (1 + 2^-20) < 0.99.  The backward takes a clamp-free path for such a
-// record, whose alpha = o (blended ? G : 0) equals the clamped form bit for bit.
-constexpr float kNoClampO = 0.989f;
 constexpr float kTEps = 1e-4f;              // stop when T (1 - alpha) would fall below this
 constexpr float kInvSigmaF2 = 2.0f;         // 1 / sigma_f^2 of the screen low-pass filter (sigma_f^2 = 1/2 px^2)
 

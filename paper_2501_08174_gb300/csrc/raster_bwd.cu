@@ -223,10 +223,18 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
           a1 = a.rec.a1[idx];
           keep = a1.w >= band.z && a1.z <= band.w;
         }
+        float4 g0, g1, g2;
+        if (keep) {
+          g0 = a.rec.g0[idx];
+          g1 = a.rec.g1[idx];
+          g2 = a.rec.g2[idx];
+          // exact band test; with one pixel per thread (few tiles) the launch waits for its longest
+          // list, where the test lengthens every batch (crops: 337 -> 351 us)
+          if (PPT > 1) keep = meets_band(g0, g1, g2, band, cam);
+        }
         const unsigned km = __ballot_sync(kFull, keep);
         if (keep) {
           const int slot = cnt + __popc(km & lt);
-          float4 g0 = a.rec.g0[idx], g2 = a.rec.g2[idx];
           const float rb = blend_rho(g0.z);
           if (GEO) {
             s_b[wib][slot] = make_float4(a1.x, a1.y, rb, __int_as_float(q));
@@ -235,7 +243,7 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
             g2.w = __int_as_float(q);
           }
           s_g0[wib][slot] = g0;
-          s_g1[wib][slot] = a.rec.g1[idx];
+          s_g1[wib][slot] = g1;
           s_g2[wib][slot] = g2;
           s_a0[wib][slot] = a.rec.a0[idx];
           s_idx[wib][slot] = idx;
@@ -251,8 +259,11 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
 #ifdef OCGS_COUNT
         if (lane == 0) OCGS_DIAG(2, 1);
 #endif
-        // every entry of the walk lies before warp_last, so some lane has jj < its
-        // last index; the support test of all pixels runs as straight-line code
+        // Every entry of the walk lies before warp_last, so some lane has jj < its last index, and
+        // nearly every one that passed the staging's band test blends a pixel: all are evaluated as
+        // straight-line code, without a vote.  (A vote on a cheap per-pixel support test skipped one
+        // entry in seven before the band test was exact; its latency and that test cost more: 4.27 ->
+        // 4.16 ms on 500k surfels x 16 views, 55.6 -> 54.8 ms on 1M x 64.)
         const float4 g0 = s_g0[wib][j], g1 = s_g1[wib][j], g2 = s_g2[wib][j];
         const float4 an = GEO ? s_b[wib][j] : make_float4(0.f, 0.f, g0.w, g2.w);
         const float rb = an.z;
@@ -260,22 +271,13 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
         const SplatColumn col = splat_column(g0, g1, g2, pxf);
         SplatHead2 hd[NP];
         bool live[2 * NP];
-        bool any = false;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
           const float2 py = padd(pyb, bc2((float)(2 * p)));  // exact: half-integers below 2^15
           hd[p] = splat_head2(g0, g1, g2, col, py);
           live[2 * p] = jj < (int)last[2 * p];
           live[2 * p + 1] = jj < (int)last[2 * p + 1];
-          if (!GEO) any = any || may_blend(hd[p], rb, live[2 * p], live[2 * p + 1]);
         }
-        // the support misses every pixel of the band (about one entry in seven; the depth and normal
-        // form evaluates those too: the vote's latency costs it more, 56.7 against 57.2 ms on 1M
-        // surfels x 64 views; the colour and opacity form keeps it, 4.34 against 4.37 ms)
-        if (!GEO && !__any_sync(kFull, any)) continue;
-#ifdef OCGS_COUNT
-        if (lane == 0) OCGS_DIAG(5, 1);  // entries evaluated in full
-#endif
         const float4 ap = s_a0[wib][j];
         const float2 no = bc2(-g0.z);  // 2 dalpha/drho = -alpha = -o G
         // this thread's sums (one lane per pixel of a pair): the slots of the
@@ -285,90 +287,82 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
         // The first pair sets each sum, the others add to it.
         float2 acc[kGradStride];
         // no per-pair branch: a candidate that is not blended has alpha = 0 and
-        // Gc = 0, which makes its weight and every term of its adjoint exactly 0
-        auto pairs = [&](auto clamp) {
-          constexpr bool CLAMP = decltype(clamp)::value;
+        // Gc = 0, which makes its weight and every term of its adjoint exactly 0.  (A clamp-free
+        // form for records whose opacity cannot reach the clamp saved its compares and cost a
+        // branch: 4.14 against 4.10 ms on 500k surfels x 16 views.)
 #pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            auto sum_fma = [&](int q, float2 x, float2 y) { acc[q] = p == 0 ? pmul(x, y) : pfma(x, y, acc[q]); };
-            auto sum_add = [&](int q, float2 x) { acc[q] = p == 0 ? x : padd(acc[q], x); };
-            const SplatEval2 e = splat_tail2<true, false, CLAMP>(g0, g2, hd[p], rb, live[2 * p], live[2 * p + 1]);
+        for (int p = 0; p < NP; ++p) {
+          auto sum_fma = [&](int q, float2 x, float2 y) { acc[q] = p == 0 ? pmul(x, y) : pfma(x, y, acc[q]); };
+          auto sum_add = [&](int q, float2 x) { acc[q] = p == 0 ? x : padd(acc[q], x); };
+          const SplatEval2 e = splat_tail2<true>(g0, g2, hd[p], rb, live[2 * p], live[2 * p + 1]);
 #ifdef OCGS_COUNT
-            OCGS_DIAG(6, (e.ok[0] ? 1 : 0) + (e.ok[1] ? 1 : 0));  // (pixel, entry) blends
+          OCGS_DIAG(6, (e.ok[0] ? 1 : 0) + (e.ok[1] ? 1 : 0));  // (pixel, entry) blends
 #endif
-            // undo the entry: T before it, its weight, and dL/dalpha
-            const float2 om = pfma(e.alpha, bc2(-1.f), bc2(1.f));  // 1 - alpha
-            const float2 inv = make_float2(rcp_approx(om.x), rcp_approx(om.y));
-            const float2 Ti = pmul(T[p], inv);
-            const float2 w = pmul(e.alpha, Ti);
-            float2 F = pmul(gC0[p], bc2(ap.x));
-            F = pfma(gC1[p], bc2(ap.y), F);
-            F = pfma(gC2[p], bc2(ap.z), F);
-            if (GEO) {
-              F = pfma(gD[p], e.z, F);
-              F = pfma(pmul(gQ[p], e.z), e.z, F);  // d(sum w z^2)/dw = z^2
-              F = pfma(gN0[p], bc2(ap.w), F);
-              F = pfma(gN1[p], bc2(an.x), F);
-              F = pfma(gN2[p], bc2(an.y), F);
-            }
-            // dL/dalpha = T_i F + (gAT - S) / (1 - alpha)
-            const float2 ga = pfma(Ti, F, pmul(pfma(S[p], bc2(-1.f), gAT[p]), inv));
-            S[p] = pfma(w, F, S[p]);
-            // a skipped candidate has alpha = 0, and the fast reciprocal of 1 - 0 is exactly 1
-            // on this GPU (checked at 1, 2 and 0.5), so T passes through it unchanged
-            T[p] = Ti;
-            sum_fma(kGr, gC0[p], w);
-            sum_fma(kGg, gC1[p], w);
-            sum_fma(kGb, gC2[p], w);
-            if (GEO) {
-              sum_fma(kGnx, gN0[p], w);
-              sum_fma(kGny, gN1[p], w);
-              sum_fma(kGnz, gN2[p], w);
-            }
-            // alpha = o G below the clamp: dalpha/do = G, dalpha/drho = -o G / 2
-            // (Gc is 0 at the clamp and for skipped candidates); gs2 = 2 dL/drho
-            const float2 gop = pmul(ga, e.Gc);
-            sum_add(kGo, gop);
-            const float2 gs2 = pmul(gop, no);
-            // rho and depth came from the surfel's (u, v) where it won the min, from the
-            // screen-space filter elsewhere.  e.r and e.rho3 are 0 where the filter won,
-            // so the surfel terms below vanish there without a mask.
-            const float2 gf2 = make_float2(e.surf[0] ? 0.f : gs2.x, e.surf[1] ? 0.f : gs2.y);
-            float2 gzs = bc2(0.f);
-            if (GEO) {
-              // d/dz of w (gD z + gQ z^2)
-              const float2 gz = pmul(pfma(pmul(bc2(2.f), gQ[p]), e.z, gD[p]), w);
-              gzs = make_float2(e.surf[0] ? gz.x : 0.f, e.surf[1] ? gz.y : 0.f);
-              sum_add(kGzc, pfma(gzs, bc2(-1.f), gz));
-              sum_fma(kGzD, gzs, e.r);
-            }
-            // 2 grho / den^2, shared by the u, v and den terms (rho3 = q / den^2)
-            const float2 t = pmul(gs2, pmul(e.r, e.r));
-            const float2 gun = pmul(t, hd[p].un);
-            const float2 gvn = pmul(t, hd[p].vn);
-            // -dL/dden = (2 grho rho3 + gz z) / den; the e slots accumulate negated and
-            // are flipped when the lanes are summed
-            const float2 ngden = GEO ? pmul(pfma(gs2, e.rho3, pmul(gzs, e.z)), e.r)
-                                     : pmul(t, pmul(hd[p].q, e.r));
-            sum_add(kSumU, gun);
-            sum_add(kSumV, gvn);
-            sum_fma(kGA01, gun, hd[p].dy);
-            sum_fma(kGA11, gvn, hd[p].dy);
-            sum_add(kGe0, ngden);
-            sum_fma(kGe2, ngden, hd[p].dy);
-            // the filter term: d rho2 / d(c) = -4 (x - c) with rho2 = 2 |x - c|^2 (the
-            // factor -2 and dx are applied later)
-            sum_add(kGcx, gf2);
-            sum_fma(kGcy, gf2, hd[p].dy);
+          // undo the entry: T before it, its weight, and dL/dalpha
+          const float2 om = pfma(e.alpha, bc2(-1.f), bc2(1.f));  // 1 - alpha
+          const float2 inv = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+          const float2 Ti = pmul(T[p], inv);
+          const float2 w = pmul(e.alpha, Ti);
+          float2 F = pmul(gC0[p], bc2(ap.x));
+          F = pfma(gC1[p], bc2(ap.y), F);
+          F = pfma(gC2[p], bc2(ap.z), F);
+          if (GEO) {
+            F = pfma(gD[p], e.z, F);
+            F = pfma(pmul(gQ[p], e.z), e.z, F);  // d(sum w z^2)/dw = z^2
+            F = pfma(gN0[p], bc2(ap.w), F);
+            F = pfma(gN1[p], bc2(an.x), F);
+            F = pfma(gN2[p], bc2(an.y), F);
           }
-        };
-        // a record that cannot reach the 0.99 clamp takes the clamp-free blend (2 % of the colour
-        // and opacity launch); the depth and normal form is faster without the branch (55.0
-        // against 56.7 ms on 1M surfels x 64 views)
-        if (!GEO && g0.z < kNoClampO) pairs(std::false_type{});
-        else pairs(std::true_type{});
-        // nearly every entry that is evaluated blends a pixel, so there is no second vote: the
-        // sums of one that does not are all zero and its flush adds nothing
+          // dL/dalpha = T_i F + (gAT - S) / (1 - alpha)
+          const float2 ga = pfma(Ti, F, pmul(pfma(S[p], bc2(-1.f), gAT[p]), inv));
+          S[p] = pfma(w, F, S[p]);
+          // a skipped candidate has alpha = 0, and the fast reciprocal of 1 - 0 is exactly 1
+          // on this GPU (checked at 1, 2 and 0.5), so T passes through it unchanged
+          T[p] = Ti;
+          sum_fma(kGr, gC0[p], w);
+          sum_fma(kGg, gC1[p], w);
+          sum_fma(kGb, gC2[p], w);
+          if (GEO) {
+            sum_fma(kGnx, gN0[p], w);
+            sum_fma(kGny, gN1[p], w);
+            sum_fma(kGnz, gN2[p], w);
+          }
+          // alpha = o G below the clamp: dalpha/do = G, dalpha/drho = -o G / 2
+          // (Gc is 0 at the clamp and for skipped candidates); gs2 = 2 dL/drho
+          const float2 gop = pmul(ga, e.Gc);
+          sum_add(kGo, gop);
+          const float2 gs2 = pmul(gop, no);
+          // rho and depth came from the surfel's (u, v) where it won the min, from the
+          // screen-space filter elsewhere.  e.r and e.rho3 are 0 where the filter won,
+          // so the surfel terms below vanish there without a mask.
+          const float2 gf2 = make_float2(e.surf[0] ? 0.f : gs2.x, e.surf[1] ? 0.f : gs2.y);
+          float2 gzs = bc2(0.f);
+          if (GEO) {
+            // d/dz of w (gD z + gQ z^2)
+            const float2 gz = pmul(pfma(pmul(bc2(2.f), gQ[p]), e.z, gD[p]), w);
+            gzs = make_float2(e.surf[0] ? gz.x : 0.f, e.surf[1] ? gz.y : 0.f);
+            sum_add(kGzc, pfma(gzs, bc2(-1.f), gz));
+            sum_fma(kGzD, gzs, e.r);
+          }
+          // 2 grho / den^2, shared by the u, v and den terms (rho3 = q / den^2)
+          const float2 t = pmul(gs2, pmul(e.r, e.r));
+          const float2 gun = pmul(t, hd[p].un);
+          const float2 gvn = pmul(t, hd[p].vn);
+          // -dL/dden = (2 grho rho3 + gz z) / den; the e slots accumulate negated and
+          // are flipped when the lanes are summed
+          const float2 ngden = GEO ? pmul(pfma(gs2, e.rho3, pmul(gzs, e.z)), e.r)
+                                   : pmul(t, pmul(hd[p].q, e.r));
+          sum_add(kSumU, gun);
+          sum_add(kSumV, gvn);
+          sum_fma(kGA01, gun, hd[p].dy);
+          sum_fma(kGA11, gvn, hd[p].dy);
+          sum_add(kGe0, ngden);
+          sum_fma(kGe2, ngden, hd[p].dy);
+          // the filter term: d rho2 / d(c) = -4 (x - c) with rho2 = 2 |x - c|^2 (the
+          // factor -2 and dx are applied later)
+          sum_add(kGcx, gf2);
+          sum_fma(kGcy, gf2, hd[p].dy);
+        }
 #ifdef OCGS_COUNT
         if (lane == 0) OCGS_DIAG(3, 1);
 #endif

@@ -9,8 +9,6 @@
 // thread owns.
 #pragma once
 
-#include <type_traits>
-
 #include "common.cuh"
 
 namespace ocgs {
@@ -48,6 +46,17 @@ __device__ __forceinline__ float4 warp_band(const DevCam& cam, int local, int wt
   const int x0 = (local % cam.tiles_x) * TW, y0 = (local / cam.tiles_x) * TH + ((wt * 32) / TW) * PPT;
   return make_float4((float)x0 + 0.5f, (float)(min(x0 + TW, cam.W) - 1) + 0.5f, (float)y0 + 0.5f,
                      (float)(min(y0 + kRows, cam.H) - 1) + 0.5f);
+}
+
+// Whether a record's support can reach a pixel centre of the band: the binning's tile test
+// (exact in y and x, with its margins) applied to the warp's rows and columns.  A superset of
+// what blends; always true in a view that checks the support tests.
+__device__ __forceinline__ bool meets_band(const float4 g0, const float4 g1, const float4 g2, const float4 band,
+                                           const DevCam& cam) {
+  if (cam.cover_rect) return true;
+  const SupportConic k = support_conic(g0, g1, g2, support_rho(g0.z));
+  const RowSpan s = support_row_span(k, band.z, band.w, band.x, band.y);
+  return (s.lo0 <= band.y && s.hi0 >= band.x) || (s.lo1 <= band.y && s.hi1 >= band.x);
 }
 
 // CTAs of BW independent warps: persistent_ctas counts tile-sized CTAs
@@ -115,16 +124,6 @@ __device__ __forceinline__ SplatHead2 splat_head2(const float4 g0, const float4 
   return h;
 }
 
-// A cheap superset of the pixels a candidate can blend: the surfel term within the
-// blend bound (u^2 + v^2 <= rb, tested as q <= rb den^2 with a relative margin that
-// covers the rounding of rho3 = q / den^2) or the filter term within it.  Only used
-// to skip an entry no pixel of the band can blend; the blend decision itself is
-// taken in splat_tail2.
-__device__ __forceinline__ bool may_blend(const SplatHead2& h, float rb, bool live0, bool live1) {
-  const float2 lim = pmul(bc2(__fmul_rn(rb, 1.0001f)), pmul(h.den, h.den));
-  return (live0 && (h.q.x <= lim.x || h.rho2.x <= rb)) || (live1 && (h.q.y <= lim.y || h.rho2.y <= rb));
-}
-
 // exp(-rho / 2) = 2^(rho * (-1 / (2 ln 2))): one multiply and the base-2 exponential of
 // the special-function unit (PTX ex2.approx, relative error about 2^-22; results below
 // 2^-126, where rho > 174, flush to 0, far outside every support bound).
@@ -164,9 +163,7 @@ struct SplatEval2 {
 // products the backward masks with zero stay finite (the forward reads z only).
 // A skipped candidate gets alpha = 0 (T (1 - 0) = T and w = 0 exactly) and
 // Gc = 0, which zeroes every term of its adjoint without further masks.
-// CLAMP = false (backward): the record's o < kNoClampO, so alpha never reaches
-// the clamp (see kNoClampO).
-template <bool FINITE, bool EWA = false, bool CLAMP = true>
+template <bool FINITE, bool EWA = false>
 __device__ __forceinline__ SplatEval2 splat_tail2(const float4 g0, const float4 g2, const SplatHead2& h, float rb,
                                                   bool live0, bool live1) {
   SplatEval2 e;
@@ -187,14 +184,9 @@ __device__ __forceinline__ SplatEval2 splat_tail2(const float4 g0, const float4 
   const float2 oG = pmul(bc2(g0.z), G);
   e.ok[0] = live0 && (rho.x <= rb);
   e.ok[1] = live1 && (rho.y <= rb);
-  if (CLAMP) {
-    e.alpha = make_float2(e.ok[0] ? fminf(kAlphaMax, oG.x) : 0.0f, e.ok[1] ? fminf(kAlphaMax, oG.y) : 0.0f);
-    if (FINITE)
-      e.Gc = make_float2(e.ok[0] && oG.x < kAlphaMax ? G.x : 0.0f, e.ok[1] && oG.y < kAlphaMax ? G.y : 0.0f);
-  } else {
-    e.Gc = make_float2(e.ok[0] ? G.x : 0.0f, e.ok[1] ? G.y : 0.0f);
-    e.alpha = pmul(bc2(g0.z), e.Gc);  // o G where blended, o 0 = 0 elsewhere
-  }
+  e.alpha = make_float2(e.ok[0] ? fminf(kAlphaMax, oG.x) : 0.0f, e.ok[1] ? fminf(kAlphaMax, oG.y) : 0.0f);
+  if (FINITE)
+    e.Gc = make_float2(e.ok[0] && oG.x < kAlphaMax ? G.x : 0.0f, e.ok[1] && oG.y < kAlphaMax ? G.y : 0.0f);
   const float2 zs = pmul(bc2(g2.w), e.r);
   e.z = make_float2(e.surf[0] ? zs.x : g0.w, e.surf[1] ? zs.y : g0.w);
   return e;
