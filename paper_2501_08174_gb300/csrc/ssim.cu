@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kViewSumThreads) ssim_final_kernel(const doubl
 // partial[2 b]: sum of squared masked differences, partial[2 b + 1]: mask values
 // Bound by the FP64 rate (about two operations per cycle and SM) where the mask is: blocks of
 // 1024 pixels spread the masked ones over the SMs (blocks of 4096 took 36 us for one view of
-// 717k pixels: X_PSNR), and the loads of a thread's four pixels are in flight together.
+// 717k pixels, these 25), and the loads of a thread's four pixels are in flight together.
 constexpr int kPsnrThreads = 256, kPsnrLoads = kPsnrBlockPixels / kPsnrThreads;
 __global__ void __launch_bounds__(kPsnrThreads) psnr_partial_kernel(const float* __restrict__ rgb,
                                                            const float* __restrict__ target,
