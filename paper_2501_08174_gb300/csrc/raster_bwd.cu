@@ -25,15 +25,13 @@ using namespace raster;
 __device__ unsigned long long g_diag[8];
 #endif
 
-// Resident warps per SM the compiler is asked to fit (caps registers per thread):
-// 20 leaves 96 registers (4 bytes spilled), measured 1.4 % faster than 16 at 119
-// registers on 500k surfels x 16 views
+// Resident warps per SM the compiler is asked to fit (caps registers per thread): 20 leaves
+// 96 registers; 16 measured 0.4 % and 24 (spills) 5 % slower on 500k surfels x 16 views
 #ifndef OCGS_BWD_WARPS
 #define OCGS_BWD_WARPS 20
 #endif
-// With depth and normal cotangents: 16 resident warps leave 128 registers (no spill;
-// 20 would spill 176 bytes), measured 4.7 % faster than 12 at 151 registers on the
-// 1M-surfel, 64-view iteration
+// With depth and normal cotangents: 16 resident warps leave 128 registers; 20 spill (62.8
+// against 54.9 ms on 1M surfels x 64 views)
 #ifndef OCGS_BWD_WARPS_GEO
 #define OCGS_BWD_WARPS_GEO 16
 #endif
