@@ -256,21 +256,21 @@ def algorithmic(stage: str, N: int, V: int, P: int, K: int, T: int, E: int, tile
     first of two passes, 0 for one pass)."""
     VN = V * N
     if M:
-        # front: counts (order, 48 B record, count, ntiles), scan, duplication; behind the front:
-        # the open-tile test (order, 16 B box, flag), its scan and compaction, the counts and their
-        # scan (the candidates' coverage reads are left out: a lower bound); pairs and tile
-        # ranges of both passes, the open flags and their prefix
-        binning = (M * (64 + 16 + 60) + (VN - M) * (24 + 12 + 24) + K * 12 + T * 32)
+        # front: counts and duplication (order and 48 B record each); behind the front: the
+        # open-tile test (order, 16 B box; the candidates' coverage reads are left out: a lower
+        # bound); pairs (8 B out, 4 B read for the ranges) and tile ranges of both passes, the
+        # open flags and their prefix
+        binning = M * (52 + 52) + (VN - M) * 20 + K * 12 + T * 32
     else:
-        # counts (48 B record in, 8 B out), count gather + scan (28 B), duplication (60 B in per
-        # record, 8 B out per pair), tile ranges (4 B per pair, 8 B per tile)
-        binning = VN * (56 + 28 + 60) + K * 12 + T * 8
+        # counts and duplication (order and 48 B record each, 8 B out per pair), tile ranges
+        # (4 B per pair, 8 B per tile)
+        binning = VN * (52 + 52) + K * 12 + T * 8
     ssim_px = 24 + 1 + 36 + 36 + 24 + 24  # images + mask, adjoint maps out and back, images again, d_rgb
     b = {
         "preprocess": N * 232 + VN * (72 + 4 + 48 + 4),   # record, ntiles, binning record, depth key
-        "depth_sort": VN * 4 + 4 * VN * 20,
+        "depth_sort": VN * (4 + 12 + 3 * 16),             # histograms, first pass (index implied), three more
         "binning": binning,
-        "tile_sort": tile_passes * K * 20,
+        "tile_sort": K * (4 + tile_passes * 16),          # histograms, then key and value in and out
         "raster_fwd": VN * 72 + K * 4 + P * 40,
         "loss": P * (4 + 1 + 8) + P * (12 + 12 + 1 + 24) + (ssim_px * P if prune_calls > 1 else 0),
         "raster_bwd": VN * (72 + 80) + K * 4 + P * 40,
