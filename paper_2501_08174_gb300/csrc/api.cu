@@ -122,6 +122,10 @@ class Block {
   void add(T** p, size_t count) { parts_.push_back({reinterpret_cast<void**>(p), bytes_of(count * sizeof(T))}); }
   template <typename T>
   void zeroed(T** p, size_t count) { zero_.push_back({reinterpret_cast<void**>(p), bytes_of(count * sizeof(T))}); }
+  void zeroed(Scratch* x, size_t bytes) {
+    x->bytes = bytes;
+    zeroed(&x->p, bytes);
+  }
   cudaError_t alloc(Arena& a, cudaStream_t s) {
     size_t total = 0, clear = 0;
     for (const Part& q : zero_) clear += q.bytes;
@@ -400,7 +404,7 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
   float4* bin;
   uint32_t *dkey, *dkey_alt, *order, *order_alt, *done1;
   uint64_t* unit_base;
-  char* dscratch;
+  Scratch dscratch;
   {
     Block b;
     b.add(&tables, table_bytes);
@@ -470,7 +474,7 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
   uint32_t *open = nullptr, *prefix = nullptr, *open_ids = nullptr, *open_words = nullptr, *done2 = nullptr;
   uint32_t* n_cand = nullptr;
   uint8_t* done = nullptr;
-  char *pscratch, *oscratch = nullptr, *qscratch = nullptr, *bscratch = nullptr;
+  Scratch pscratch, oscratch, qscratch, bscratch;
   // the second pass continues from T (and, with images, the last blended position)
   float* t_fin = keep_state && img ? st->t_final : nullptr;
   uint32_t* lst = keep_state && img ? st->last : nullptr;
@@ -562,7 +566,7 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
     K2 = (uint32_t)K2_64;
     if (K2) {
       uint32_t *qkey, *qval, *qkey_alt, *qval_alt;
-      char* pscratch2;
+      Scratch pscratch2;
       const bool alt2 = radix_result_in_alt(K2, tbits);
       {
         Block b;
@@ -637,7 +641,7 @@ struct SweepWs {
   // cleared at the start of every chunk: [zero, zero + zero_bytes)
   char* zero = nullptr;
   size_t zero_bytes = 0;
-  char *dscratch = nullptr, *pscratch = nullptr, *oscratch = nullptr;
+  Scratch dscratch, pscratch, oscratch;
   uint32_t *queue = nullptr, *done = nullptr;
   uint32_t vn_max = 0, cap = 0;
   int64_t tiles_max = 0;
@@ -649,6 +653,7 @@ cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_
   w.cap = cap;
   const int tbits = bits_for((uint64_t)tiles_max);
   Block b;
+  // every scratch serves the chunks of fewer records or tiles too (see Scratch)
   b.zeroed(&w.dscratch, depth_sort_scratch_bytes(vn_max));
   // a chunk with fewer tiles may sort fewer bits in fewer passes: any plan up to tbits fits
   size_t psort = 0;
@@ -679,8 +684,8 @@ cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_
   b.add(&w.pval_alt, cap);
   b.add(&w.ids, tiles_max);
   const cudaError_t e = b.alloc(a, s);
-  w.zero = w.dscratch;
-  w.zero_bytes = (size_t)(reinterpret_cast<char*>(w.rec.g0) - w.dscratch);
+  w.zero = w.dscratch.p;
+  w.zero_bytes = (size_t)(reinterpret_cast<char*>(w.rec.g0) - w.zero);
   return e;
 }
 

@@ -336,20 +336,29 @@ cudaError_t launch_preprocess_backward(const GaussPtrs& g, int64_t n, int sh_deg
                                        const DevCam* cams, int n_views, const float* grad_rec,
                                        const int32_t* ntiles, GaussOut out, cudaStream_t s);
 
+// Scratch of a sort and the bytes it has: zeroed by the caller before every sort.  A scratch of
+// the *_scratch_bytes of n items serves a sort of any m <= n (a workspace laid out for the largest
+// of several sorts); a sort that needs more than its scratch has returns cudaErrorInvalidValue
+// and launches nothing.
+struct Scratch {
+  char* p = nullptr;
+  size_t bytes = 0;
+};
+
 // Stable LSD radix sort of (key, value) 32-bit pairs on key bits [0, n_bits) in ping-pong
-// buffers; the result is in the alternate ones if radix_result_in_alt.  scratch holds
-// radix_scratch_bytes and is zeroed by the caller.  d_n (optional): device-side item count,
-// read by the kernels and clamped to n (n sizes the launch: a capacity).
+// buffers; the result is in the alternate ones if radix_result_in_alt.  scratch:
+// radix_scratch_bytes.  d_n (optional): device-side item count, read by the kernels and clamped
+// to n (n sizes the launch: a capacity).
 size_t radix_scratch_bytes(uint32_t n, int n_bits);
 bool radix_result_in_alt(uint32_t n, int n_bits);
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
-                             int n_bits, void* scratch, cudaStream_t s, const uint32_t* d_n = nullptr);
+                             int n_bits, const Scratch& scratch, cudaStream_t s, const uint32_t* d_n = nullptr);
 // The records in depth order: order[0 .. *n_valid) are the indices of the keys other than
 // 0xffffffff, ascending by key, ties by index.  keys and the alternates are overwritten;
-// scratch holds depth_sort_scratch_bytes and is zeroed by the caller.
+// scratch: depth_sort_scratch_bytes.
 size_t depth_sort_scratch_bytes(uint32_t n);
 cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint32_t* order_alt, uint32_t n,
-                       uint32_t* n_valid, void* scratch, cudaStream_t s);
+                       uint32_t* n_valid, const Scratch& scratch, cudaStream_t s);
 
 // Binning of the depth order (entries order[0 .. min(n, *d_n))) in work units of consecutive
 // entries.  unit_base [unit_base_words(n)]: first pair of each unit, *total = the pairs (row_runs
@@ -371,11 +380,11 @@ cudaError_t launch_tile_ranges(const uint32_t* keys, uint32_t n_pairs, uint2* ra
 // (queue_class; ranges2: an optional second segment of each tile's list, counted with the
 // first).  A strict view-by-view order left SMs idle at the end of each launch, each view's
 // heavy tiles starting late (backward active warps 15.6 -> 14.6 per SM on a 4-view case).
-// scratch: zeroed, tile_order_scratch_bytes; *n_nonempty: device count of the tiles with pairs
+// scratch: tile_order_scratch_bytes; *n_nonempty: device count of the tiles with pairs
 // (in scratch), which come first.
 size_t tile_order_scratch_bytes(uint32_t n_tiles);
 cudaError_t launch_tile_order(const uint2* ranges, const uint2* ranges2, uint32_t n_tiles, uint32_t* ids,
-                              void* scratch, cudaStream_t s, const uint32_t** n_nonempty = nullptr);
+                              const Scratch& scratch, cudaStream_t s, const uint32_t** n_nonempty = nullptr);
 
 // Two-pass binning (front records first, then the records behind them into the tiles left open).
 // P [n_tiles + 1]: exclusive prefix of the 0/1 open flags; open_ids: the open tiles, ascending;

@@ -9,6 +9,7 @@
 // ascending (depth, Gaussian index) order, and only ceil(log2 tiles) key bits
 // are sorted per pair instead of tile+depth bits.
 #include "lookback.cuh"
+#include "sort_layout.h"
 
 #include <algorithm>
 #include <type_traits>
@@ -16,6 +17,7 @@
 namespace ocgs {
 namespace {
 using namespace lookback;
+using namespace sort_layout;
 
 // ------------------------------------------------------------------ radix sort
 // Stable LSD sort, one kernel per digit (the single-pass scatter with decoupled
@@ -27,21 +29,10 @@ using namespace lookback;
 //
 // What bounds it: HBM at full size (16 bytes per item and pass), the launch and
 // the look-back latency below about a million items.
-// 384 threads x 18 items at three blocks per SM (56 registers, 69 KB) was the fastest of
-// 256 to 512 threads x 10 to 24 items: 36 resident warps hide the ranking's shared-memory
-// latency and few tiles keep the look-back short (tile sorts of 500k surfels x 16 views,
-// 28 M pairs: 376 us against 400 to 516 with the others, 584 with a histogram, a scan and
-// a scatter kernel per digit; depth sort of 8 M records: 230 against 390).
-constexpr int kRadixThreads = 384;
-constexpr int kRadixItems = 18;
+// (The sizes of a tile: sort_layout.h.)
 constexpr int kRadixBlocks = 3;  // resident per SM
 constexpr int kRadixWarps = kRadixThreads / 32;
 static_assert(kRadixThreads * kRadixItems <= kMaxTileCount, "look-back words");
-// Where tiles of 18 items would leave SMs idle, tiles of 4: a pass over few items is the
-// latency of one tile, and that of its serial ranking rounds (a pass over 2,000 records: 8.2
-// -> 5.5 us; the depth sort of 100k: 52 -> 43 us).
-constexpr int kSmallItems = 4;
-constexpr uint32_t kSmallSort = 152u * kRadixThreads * kSmallItems;  // at most one small tile per SM
 // Digits of a sort of n_bits key bits: equal widths of 4 to 8 bits.  (Two digits of 10
 // bits instead of three of 7 took 17.6 against 6.0 ms on 480k tiles: runs of a few items
 // per digit and tile, and four times the look-back words.)
@@ -589,25 +580,25 @@ __global__ void tile_ranges_kernel(const uint32_t* __restrict__ keys, uint32_t n
 
 namespace {
 
-// Scratch of one sort (zeroed by the caller): digit positions, counters, look-back words.
-struct RadixScratch {
+// Places of one sort within its scratch (zeroed by the caller): digit positions, counters,
+// look-back words.  The scratch may be that of a larger sort; one that is too small is refused
+// before any launch.
+struct RadixPlaces {
   uint32_t *base, *done, *next_tile, *words;
-  size_t tiles, bytes;
+  size_t tiles;
 };
-RadixScratch radix_layout(void* scratch, uint32_t n, int passes, int bits) {
-  RadixScratch w;
-  const size_t R = (size_t)1 << bits, tile = (size_t)kRadixThreads * (n <= kSmallSort ? kSmallItems : kRadixItems);
-  w.tiles = ((size_t)n + tile - 1) / tile;
-  w.base = static_cast<uint32_t*>(scratch);
-  w.done = w.base + passes * R;
-  w.next_tile = w.done + 1;
-  w.words = w.base + passes * R + 64;
-  w.bytes = sizeof(uint32_t) * (passes * R + 64 + passes * w.tiles * R);
-  return w;
+cudaError_t radix_places(const Scratch& scratch, uint32_t n, int passes, int bits, RadixPlaces* w) {
+  if (bytes_used(n, passes, bits) > scratch.bytes) return cudaErrorInvalidValue;
+  w->tiles = tile_count(n);
+  w->base = reinterpret_cast<uint32_t*>(scratch.p);
+  w->done = w->base + ((size_t)passes << bits);
+  w->next_tile = w->done + 1;
+  w->words = w->done + kCounterWords;
+  return cudaSuccess;
 }
 
 template <class Keys, int BITS, int PASSES, bool DROP>
-cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const RadixScratch& w, uint32_t* n_valid,
+cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const RadixPlaces& w, uint32_t* n_valid,
                         cudaStream_t s) {
   // at least four keys per thread, at most four blocks per SM
   const size_t per_block = 4 * kRadixThreads;
@@ -618,7 +609,7 @@ cudaError_t launch_hist(const Keys& k, uint32_t n, const uint32_t* d_n, const Ra
 
 template <class Keys, int BITS, bool INDEX, bool DROP, bool KEYS_OUT>
 cudaError_t launch_pass(const Keys& k, const uint32_t* vals, uint32_t* keys_out, uint32_t* vals_out, uint32_t n,
-                        const uint32_t* d_n, int p, const RadixScratch& w, cudaStream_t s) {
+                        const uint32_t* d_n, int p, const RadixPlaces& w, cudaStream_t s) {
   auto pass = n <= kSmallSort ? radix_pass_kernel<Keys, kSmallItems, BITS, INDEX, DROP, KEYS_OUT>
                               : radix_pass_kernel<Keys, kRadixItems, BITS, INDEX, DROP, KEYS_OUT>;
   pass<<<(unsigned)w.tiles, kRadixThreads, 0, s>>>(k, vals, keys_out, vals_out, n, d_n, p * BITS,
@@ -629,9 +620,10 @@ cudaError_t launch_pass(const Keys& k, const uint32_t* vals, uint32_t* keys_out,
 
 template <int BITS, int PASSES>
 cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
-                        void* scratch, cudaStream_t s, const uint32_t* d_n) {
-  const RadixScratch w = radix_layout(scratch, n, PASSES, BITS);
-  cudaError_t e = launch_hist<ArrayKeys, BITS, PASSES, false>(ArrayKeys{keys}, n, d_n, w, nullptr, s);
+                        const Scratch& scratch, cudaStream_t s, const uint32_t* d_n) {
+  RadixPlaces w;
+  cudaError_t e = radix_places(scratch, n, PASSES, BITS, &w);
+  if (e == cudaSuccess) e = launch_hist<ArrayKeys, BITS, PASSES, false>(ArrayKeys{keys}, n, d_n, w, nullptr, s);
   uint32_t *kin = keys, *vin = vals, *kout = keys_alt, *vout = vals_alt;
   for (int p = 0; p < PASSES && e == cudaSuccess; ++p) {
     e = launch_pass<ArrayKeys, BITS, false, false, true>(ArrayKeys{kin}, vin, kout, vout, n, d_n, p, w, s);
@@ -646,7 +638,7 @@ cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint
 size_t radix_scratch_bytes(uint32_t n, int n_bits) {
   if (n <= 1 || n_bits <= 0) return 16;
   const DigitPlan pl = digit_plan(n_bits);
-  return radix_layout(nullptr, n, pl.passes, pl.bits).bytes;
+  return bytes_for(n, pl.passes, pl.bits);
 }
 
 bool radix_result_in_alt(uint32_t n, int n_bits) {
@@ -654,7 +646,7 @@ bool radix_result_in_alt(uint32_t n, int n_bits) {
 }
 
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
-                             int n_bits, void* scratch, cudaStream_t s, const uint32_t* d_n) {
+                             int n_bits, const Scratch& scratch, cudaStream_t s, const uint32_t* d_n) {
   if (n <= 1 || n_bits <= 0) return cudaSuccess;
   const DigitPlan pl = digit_plan(n_bits);
 #define OCGS_SORT(B, P) \
@@ -666,13 +658,14 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
   return cudaErrorInvalidValue;
 }
 
-size_t depth_sort_scratch_bytes(uint32_t n) { return radix_layout(nullptr, n, 4, 8).bytes; }
+size_t depth_sort_scratch_bytes(uint32_t n) { return bytes_for(n, 4, 8); }
 
 cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint32_t* order_alt, uint32_t n,
-                       uint32_t* n_valid, void* scratch, cudaStream_t s) {
+                       uint32_t* n_valid, const Scratch& scratch, cudaStream_t s) {
   if (n == 0) return cudaMemsetAsync(n_valid, 0, sizeof(uint32_t), s);
-  const RadixScratch w = radix_layout(scratch, n, 4, 8);
-  cudaError_t e = launch_hist<ArrayKeys, 8, 4, true>(ArrayKeys{keys}, n, nullptr, w, n_valid, s);
+  RadixPlaces w;
+  cudaError_t e = radix_places(scratch, n, 4, 8, &w);
+  if (e == cudaSuccess) e = launch_hist<ArrayKeys, 8, 4, true>(ArrayKeys{keys}, n, nullptr, w, n_valid, s);
   if (e == cudaSuccess)  // the first pass makes the indices and leaves the culled records out
     e = launch_pass<ArrayKeys, 8, true, true, true>(ArrayKeys{keys}, nullptr, keys_alt, order_alt, n, nullptr, 0, w, s);
   if (e == cudaSuccess)
@@ -685,15 +678,17 @@ cudaError_t depth_sort(uint32_t* keys, uint32_t* keys_alt, uint32_t* order, uint
   return e;
 }
 
-size_t tile_order_scratch_bytes(uint32_t n_tiles) { return radix_layout(nullptr, n_tiles, 1, 4).bytes; }
+size_t tile_order_scratch_bytes(uint32_t n_tiles) { return bytes_for(n_tiles, 1, 4); }
 
 cudaError_t launch_tile_order(const uint2* ranges, const uint2* ranges2, uint32_t n_tiles, uint32_t* ids,
-                              void* scratch, cudaStream_t s, const uint32_t** n_nonempty) {
-  const RadixScratch w = radix_layout(scratch, n_tiles, 1, 4);
+                              const Scratch& scratch, cudaStream_t s, const uint32_t** n_nonempty) {
+  RadixPlaces w;
+  cudaError_t e = radix_places(scratch, n_tiles, 1, 4, &w);
+  if (e != cudaSuccess) return e;
   if (n_nonempty) *n_nonempty = w.base + 15;  // first position of the empty tiles' class
   if (n_tiles == 0) return cudaSuccess;
   const QueueKeys k{ranges, ranges2};
-  const cudaError_t e = launch_hist<QueueKeys, 4, 1, false>(k, n_tiles, nullptr, w, nullptr, s);
+  e = launch_hist<QueueKeys, 4, 1, false>(k, n_tiles, nullptr, w, nullptr, s);
   if (e != cudaSuccess) return e;
   return launch_pass<QueueKeys, 4, true, false, false>(k, nullptr, nullptr, ids, n_tiles, nullptr, 0, w, s);
 }
