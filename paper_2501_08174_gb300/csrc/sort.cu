@@ -33,17 +33,6 @@ using namespace sort_layout;
 constexpr int kRadixBlocks = 3;  // resident per SM
 constexpr int kRadixWarps = kRadixThreads / 32;
 static_assert(kRadixThreads * kRadixItems <= kMaxTileCount, "look-back words");
-// Digits of a sort of n_bits key bits: equal widths of 4 to 8 bits.  (Two digits of 10
-// bits instead of three of 7 took 17.6 against 6.0 ms on 480k tiles: runs of a few items
-// per digit and tile, and four times the look-back words.)
-constexpr int kMinDigit = 4, kMaxDigit = 8;
-struct DigitPlan {
-  int passes, bits;
-};
-DigitPlan digit_plan(int n_bits) {
-  const int passes = (n_bits + kMaxDigit - 1) / kMaxDigit;
-  return DigitPlan{passes, std::max(kMinDigit, (n_bits + passes - 1) / passes)};
-}
 
 // Where the keys of a sort come from: an array, or (queue orders) the tiles' pair counts.
 struct ArrayKeys {
@@ -633,6 +622,18 @@ cudaError_t sort_passes(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint
   return e;
 }
 
+// The sort of each key width by its digit plan: every width from N to 32 bits is built, so no
+// plan is without its kernels.
+template <int N>
+cudaError_t sort_width(int n_bits, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
+                       const Scratch& scratch, cudaStream_t s, const uint32_t* d_n) {
+  constexpr DigitPlan plan = digit_plan(N);
+  static_assert(plan.bits <= kMaxDigit && plan.bits * plan.passes >= N, "digits of the key");
+  if (n_bits == N) return sort_passes<plan.bits, plan.passes>(keys, vals, keys_alt, vals_alt, n, scratch, s, d_n);
+  if constexpr (N < 32) return sort_width<N + 1>(n_bits, keys, vals, keys_alt, vals_alt, n, scratch, s, d_n);
+  return cudaErrorInvalidValue;
+}
+
 }  // namespace
 
 size_t radix_scratch_bytes(uint32_t n, int n_bits) {
@@ -648,14 +649,7 @@ bool radix_result_in_alt(uint32_t n, int n_bits) {
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
                              int n_bits, const Scratch& scratch, cudaStream_t s, const uint32_t* d_n) {
   if (n <= 1 || n_bits <= 0) return cudaSuccess;
-  const DigitPlan pl = digit_plan(n_bits);
-#define OCGS_SORT(B, P) \
-  if (pl.bits == B && pl.passes == P) return sort_passes<B, P>(keys, vals, keys_alt, vals_alt, n, scratch, s, d_n);
-  OCGS_SORT(4, 1) OCGS_SORT(5, 1) OCGS_SORT(6, 1) OCGS_SORT(7, 1) OCGS_SORT(8, 1)
-  OCGS_SORT(5, 2) OCGS_SORT(6, 2) OCGS_SORT(7, 2) OCGS_SORT(8, 2)
-  OCGS_SORT(6, 3) OCGS_SORT(7, 3) OCGS_SORT(8, 3) OCGS_SORT(8, 4)
-#undef OCGS_SORT
-  return cudaErrorInvalidValue;
+  return sort_width<1>(n_bits, keys, vals, keys_alt, vals_alt, n, scratch, s, d_n);
 }
 
 size_t depth_sort_scratch_bytes(uint32_t n) { return bytes_for(n, 4, 8); }

@@ -1,4 +1,5 @@
-// Sizes of the radix sorts of the binning: the items of a tile and the scratch of a sort.
+// Sizes of the radix sorts of the binning: the items of a tile, the digits of a key and the
+// scratch of a sort.
 // Plain C++, so that a program on the CPU can check them.
 #pragma once
 
@@ -29,6 +30,18 @@ inline size_t tile_count(uint32_t n) {
 }
 // The most tiles a sort of any m <= n items has.
 inline size_t tile_bound(uint32_t n) { return std::max(tile_count(n), tile_count(std::min(n, kSmallSort))); }
+
+// Digits of a sort of n_bits key bits: equal widths of 4 to 8 bits.  (Two digits of 10
+// bits instead of three of 7 took 17.6 against 6.0 ms on 480k tiles: runs of a few items
+// per digit and tile, and four times the look-back words.)
+constexpr int kMinDigit = 4, kMaxDigit = 8;
+struct DigitPlan {
+  int passes, bits;
+};
+constexpr DigitPlan digit_plan(int n_bits) {
+  const int passes = (n_bits + kMaxDigit - 1) / kMaxDigit;
+  return DigitPlan{passes, std::max(kMinDigit, (n_bits + passes - 1) / passes)};
+}
 
 // Scratch words of a sort: the digit positions of every pass, 64 words of counters, and one
 // look-back word per pass, tile and digit.

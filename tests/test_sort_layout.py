@@ -48,3 +48,12 @@ def test_scratch_of_n_items_holds_every_smaller_sort(tmp_path):
 def test_last_chunk_fits_the_workspace_of_the_first(tmp_path, n, views):
     """Depth-sort scratch of a sweep of more than 16 views: chunks of 16, a shorter last one."""
     run_program(tmp_path, f"  return bytes_for({16 * n}u, 4, 8) < bytes_used({(views - 16) * n}u, 4, 8);\n")
+
+
+def test_digit_plan_covers_every_key_width(tmp_path):
+    run_program(tmp_path, """
+  for (int n = 1; n <= 32; ++n) {
+    const DigitPlan p = digit_plan(n);
+    if (p.passes * p.bits < n || p.bits < kMinDigit || p.bits > kMaxDigit || p.passes != (n + 7) / 8) return 1;
+  }
+""")
