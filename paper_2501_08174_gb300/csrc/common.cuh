@@ -112,6 +112,10 @@ __device__ __forceinline__ float fast_sqrt(float x) { return x > 0.f ? __fmul_rn
 //      (A00 dx + A01 dy)^2 + (A10 dx + A11 dy)^2 <= rt (e0 + e1 dx + e2 dy)^2
 //    in (dx, dy) = x - c, written a dx^2 + 2 b dx dy + c dy^2 + 2 d dx + 2 e dy + f <= 0
 //    and, about its centre m, a u^2 + 2 b u v + c v^2 <= kappa.
+// The map (A and e) is first scaled by the power of two that brings the largest |A| into
+// [1, 2): the support does not change, no mantissa does either, and the products below (a
+// kappa is of the sixth power of the surfel's size and the focal length) stay within float32
+// for scenes in any unit of length.
 struct SupportConic {
   float cx, cy, r2f;
   float a, b, c;
@@ -120,8 +124,15 @@ struct SupportConic {
   bool ellipse;             // a > 0, det > 0, kappa > 0 and finite
 };
 
-__device__ __forceinline__ SupportConic support_conic(const float4 g0, const float4 g1, const float4 g2, float rb) {
+__device__ __forceinline__ SupportConic support_conic(const float4 g0, const float4 g1_raw, const float4 g2_raw,
+                                                      float rb) {
   SupportConic k;
+  const float m = fmaxf(fmaxf(fabsf(g1_raw.x), fabsf(g1_raw.y)), fmaxf(fabsf(g1_raw.z), fabsf(g1_raw.w)));
+  // 2^-exponent(m) (a non-finite m makes every coefficient non-finite: no ellipse)
+  const float f = __uint_as_float(0x7f000000u - (__float_as_uint(m) & 0x7f800000u));
+  const float4 g1 = make_float4(__fmul_rn(f, g1_raw.x), __fmul_rn(f, g1_raw.y), __fmul_rn(f, g1_raw.z),
+                                __fmul_rn(f, g1_raw.w));
+  const float4 g2 = make_float4(__fmul_rn(f, g2_raw.x), __fmul_rn(f, g2_raw.y), __fmul_rn(f, g2_raw.z), 0.f);
   const float rt = __fadd_rn(__fmul_rn(rb, 1.001f), 1e-3f);
   k.cx = g0.x;
   k.cy = g0.y;
@@ -149,6 +160,7 @@ __device__ __forceinline__ SupportConic support_conic(const float4 g0, const flo
     k.umax = fast_sqrt(__fdividef(__fmul_rn(k.kappa, k.c), k.det));
     k.vmax = fast_sqrt(__fdividef(__fmul_rn(k.kappa, k.a), k.det));
     k.vstar = __fdividef(-__fmul_rn(k.b, k.umax), k.c);
+    k.ellipse = isfinite(k.umax) && isfinite(k.vmax);
   }
   return k;
 }
