@@ -56,3 +56,21 @@ def test_prune_none_and_all(value):
     for k in KEYS:
         assert torch.equal(kept[k], g[k][:kept[k].shape[0]])
     rast.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [524_288, 524_289, 1_300_003])
+def test_prune_over_many_count_blocks(n):
+    """More than 256 blocks of 2,048: the last block scans several totals per thread."""
+    from paper_2501_08174_gb300 import Rasterizer
+    rast = Rasterizer(0)
+    g = arrays(n, 0, 0, rast.device)
+    gen = torch.Generator(device=rast.device).manual_seed(n)
+    s = torch.rand(n, generator=gen, device=rast.device)
+    s[::1000] = 0.5
+    kept, border, n_border = rast.prune(g, s, 0.5, borderline_cap=n)
+    for k in KEYS:
+        assert torch.equal(kept[k], g[k][s > 0.5]), k
+    want = torch.nonzero((s - 0.5).abs() <= 1e-6).reshape(-1)
+    assert n_border == len(want) and torch.equal(border, want)
+    rast.close()
