@@ -267,7 +267,7 @@ def algorithmic(stage: str, N: int, V: int, P: int, K: int, T: int, E: int, tile
         binning = VN * (52 + 52) + K * 12 + T * 8
     ssim_px = 24 + 1 + 36 + 36 + 24 + 24  # images + mask, adjoint maps out and back, images again, d_rgb
     b = {
-        "preprocess": N * 232 + VN * (72 + 4 + 48 + 4),   # record, ntiles, binning record, depth key
+        "preprocess": N * 232 + VN * (72 + 48 + 4),       # record, binning record, depth key
         "depth_sort": VN * (4 + 12 + 3 * 16),             # histograms, first pass (index implied), three more
         "binning": binning,
         "tile_sort": K * (4 + tile_passes * 16),          # histograms, then key and value in and out

@@ -56,7 +56,6 @@ struct ocgs_fwd_state {
   DevCam* d_cams = nullptr;
   int* d_tile_prefix = nullptr;
   RecPtrs rec{};
-  int32_t* ntiles = nullptr;
   uint32_t* vals = nullptr;
   uint2* ranges = nullptr;
   uint2* ranges2 = nullptr;   // two-pass renders: second segment of each tile's list
@@ -413,7 +412,6 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
     b.add(&st->rec.g2, VN);
     b.add(&st->rec.a0, VN);
     b.add(&st->rec.a1, VN);
-    b.add(&st->ntiles, VN);
     b.zeroed(&st->ranges, n_t);
     if (keep_state) {
       b.add(&st->t_final, pl.P);
@@ -442,10 +440,10 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
   {
     StageTimer t(ctx, OCGS_STAGE_PREPROCESS);
     if (ewa)
-      CK(launch_preprocess_ewa(gptrs(g), N, g->sh_degree, st->d_cams, V, tw, th, st->rec, st->ntiles, bin, dkey,
+      CK(launch_preprocess_ewa(gptrs(g), N, g->sh_degree, st->d_cams, V, tw, th, st->rec, bin, dkey,
                                ctx->d_status, s));
     else
-      CK(launch_preprocess(gptrs(g), N, g->sh_degree, st->d_cams, V, tw, th, st->rec, st->ntiles, bin, dkey,
+      CK(launch_preprocess(gptrs(g), N, g->sh_degree, st->d_cams, V, tw, th, st->rec, bin, dkey,
                            ctx->d_status, s));
   }
   uint32_t* d_valid = reinterpret_cast<uint32_t*>(ctx->d_scalar + kValid);  // records with a non-empty screen box
@@ -631,7 +629,6 @@ ocgs_status forward_pass(ocgs_ctx* ctx, const ocgs_gaussians* g, const ocgs_came
 // allocation, host copy or host synchronisation (and hence captured).
 struct SweepWs {
   RecPtrs rec{};
-  int32_t* ntiles = nullptr;
   uint2* ranges = nullptr;
   float4* bin = nullptr;
   uint32_t *dkey = nullptr, *order = nullptr, *dkey_alt = nullptr, *order_alt = nullptr;
@@ -668,7 +665,6 @@ cudaError_t alloc_sweep_ws(Arena& a, SweepWs& w, uint32_t vn_max, int64_t tiles_
   b.add(&w.rec.g2, vn_max);
   b.add(&w.rec.a0, vn_max);
   b.add(&w.rec.a1, vn_max);
-  b.add(&w.ntiles, vn_max);
   b.add(&w.bin, 3 * (size_t)vn_max);
   b.add(&w.dkey, vn_max);
   b.add(&w.order, vn_max);
@@ -701,7 +697,7 @@ ocgs_status enqueue_sweep_chunk(ocgs_ctx* ctx, const ocgs_gaussians* g, int V, c
   const uint32_t VN = (uint32_t)(N * V);
   const int tbits = bits_for((uint64_t)n_tiles);
   CK(cudaMemsetAsync(w.zero, 0, w.zero_bytes, s));
-  CK(launch_preprocess(gptrs(g), N, g->sh_degree, d_cams, V, tw, th, w.rec, w.ntiles, w.bin, w.dkey, ctx->d_status,
+  CK(launch_preprocess(gptrs(g), N, g->sh_degree, d_cams, V, tw, th, w.rec, w.bin, w.dkey, ctx->d_status,
                        s));
   CK(depth_sort(w.dkey, w.dkey_alt, w.order, w.order_alt, VN, w.n_valid, w.dscratch, s));
   CK(launch_bin_count(w.order, VN, w.n_valid, w.bin, d_cams, N, tw, th, w.unit_base, w.done, w.total, s, w.n32,
@@ -918,7 +914,7 @@ ocgs_status ocgs_render_backward(ocgs_ctx* ctx, const ocgs_fwd_state* st, const 
   GaussOut go{d_params->xyz, d_params->quat, d_params->scale, d_params->opacity, d_params->sh};
   {
     StageTimer t(ctx, OCGS_STAGE_PREPROCESS_BWD);
-    CK(launch_preprocess_backward(gptrs(g), st->N, st->deg, st->d_cams, st->V, grad_rec, st->ntiles, go, s));
+    CK(launch_preprocess_backward(gptrs(g), st->N, st->deg, st->d_cams, st->V, grad_rec, go, s));
   }
   return OCGS_OK;
 }

@@ -337,16 +337,16 @@ inline cudaError_t launched() {
 }
 
 cudaError_t launch_preprocess(const GaussPtrs& g, int64_t n, int sh_degree, const DevCam* cams,
-                              int n_views, int tile_w, int tile_h, RecPtrs rec, int32_t* ntiles,
-                              float4* bin, uint32_t* depth_key, int* status, cudaStream_t s);
+                              int n_views, int tile_w, int tile_h, RecPtrs rec, float4* bin, uint32_t* depth_key,
+                              int* status, cudaStream_t s);
 
 // EWA projection of 3D Gaussians (scale [n,3]) into the same record format
 cudaError_t launch_preprocess_ewa(const GaussPtrs& g, int64_t n, int sh_degree, const DevCam* cams, int n_views,
-                                  int tile_w, int tile_h, RecPtrs rec, int32_t* ntiles, float4* bin,
+                                  int tile_w, int tile_h, RecPtrs rec, float4* bin,
                                   uint32_t* depth_key, int* status, cudaStream_t s);
 cudaError_t launch_preprocess_backward(const GaussPtrs& g, int64_t n, int sh_degree,
                                        const DevCam* cams, int n_views, const float* grad_rec,
-                                       const int32_t* ntiles, GaussOut out, cudaStream_t s);
+                                       GaussOut out, cudaStream_t s);
 
 // Scratch of a sort and the bytes it has: zeroed by the caller before every sort.  A scratch of
 // the *_scratch_bytes of n items serves a sort of any m <= n (a workspace laid out for the largest

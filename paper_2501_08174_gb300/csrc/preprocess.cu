@@ -321,7 +321,6 @@ template <int DEG>
 __global__ void __launch_bounds__(128) preprocess_kernel(GaussPtrs g, int64_t n,
                                                          const DevCam* __restrict__ cams, int n_views,
                                                          int tile_w, int tile_h, RecPtrs rec,
-                                                         int32_t* __restrict__ ntiles,
                                                          float4* __restrict__ bin,
                                                          uint32_t* __restrict__ depth_key,
                                                          int* __restrict__ status) {
@@ -390,12 +389,10 @@ __global__ void __launch_bounds__(128) preprocess_kernel(GaussPtrs g, int64_t n,
       }
     }
     if (culled) {
-      ntiles[idx] = 0;
       depth_key[idx] = 0xffffffffu;
       bin[3 * idx + 2] = make_float4(0.f, 0.f, __uint_as_float(pack_i16x2(0, 0)), __uint_as_float(pack_i16x2(-1, -1)));
       continue;
     }
-    ntiles[idx] = (rc.z - rc.x + 1) * (rc.w - rc.y + 1);
     depth_key[idx] = depth_key_of(cam, X);
     const float pz = G.p[2];
     const float e0 = G.a * G.d - G.b * G.c;
@@ -427,7 +424,6 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(GaussPtrs g, int64_
                                                              const DevCam* __restrict__ cams,
                                                              int n_views,
                                                              const float* __restrict__ grad_rec,
-                                                             const int32_t* __restrict__ ntiles,
                                                              GaussOut out) {
   constexpr int K = (DEG + 1) * (DEG + 1);
   __shared__ __align__(16) float s_rows[ShRows<3 * K>::kFloats];
@@ -454,23 +450,21 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(GaussPtrs g, int64_
 #pragma unroll
   for (int k = 0; k < 3 * K; ++k) gsh[k] = 0.f;
 
-  // the tile counts and record gradients of the next two views are requested before
-  // the current view is processed, so their memory latency overlaps its arithmetic
+  // the record gradients of the next two views are requested before the current view
+  // is processed, so their memory latency overlaps its arithmetic
   constexpr int NQ = kGradStride / 4;
-  int nt_next = 0, nt_next2 = 0;
   float4 g_next[NQ], g_next2[NQ];
-  auto request = [&](int v, int& nt, float4* gv) {
+  auto request = [&](int v, float4* gv) {
     const int64_t idx = (int64_t)v * n + i;
-    nt = ntiles[idx];
     const float4* gr4 = reinterpret_cast<const float4*>(grad_rec + idx * kGradStride);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) gv[q] = gr4[q];
   };
-  if (n_views > 0) request(0, nt_next, g_next);
-  if (n_views > 1) request(1, nt_next2, g_next2);
+  if (n_views > 0) request(0, g_next);
+  if (n_views > 1) request(1, g_next2);
   for (int v = 0; v < n_views; ++v) {
-    const int nt = nt_next;
     float gq[kGradStride];
+    unsigned bits = 0;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       gq[4 * q] = g_next[q].x;
@@ -479,9 +473,12 @@ __global__ void __launch_bounds__(128) preprocess_bwd_kernel(GaussPtrs g, int64_
       gq[4 * q + 3] = g_next[q].w;
       g_next[q] = g_next2[q];
     }
-    nt_next = nt_next2;
-    if (v + 2 < n_views) request(v + 2, nt_next2, g_next2);
-    if (nt == 0) continue;
+    if (v + 2 < n_views) request(v + 2, g_next2);
+    // a record without gradient adds nothing: the chain rule through a record that blends no
+    // pixel (culled, or far outside the image) may be infinite
+#pragma unroll
+    for (int q = 0; q < kGradSlots; ++q) bits |= __float_as_uint(gq[q]);
+    if ((bits & 0x7fffffffu) == 0u) continue;
     const DevCam& cam = vcams[v];
     const float g_cx = gq[kGcx], g_cy = gq[kGcy], g_o = gq[kGo], g_zc = gq[kGzc];
     const float gA00 = gq[kGA00], gA01 = gq[kGA01], gA10 = gq[kGA10], gA11 = gq[kGA11];
@@ -606,7 +603,6 @@ template <int DEG>
 __global__ void __launch_bounds__(128) preprocess_ewa_kernel(GaussPtrs g, int64_t n,
                                                              const DevCam* __restrict__ cams, int n_views,
                                                              int tile_w, int tile_h, RecPtrs rec,
-                                                             int32_t* __restrict__ ntiles,
                                                              float4* __restrict__ bin,
                                                              uint32_t* __restrict__ depth_key,
                                                              int* __restrict__ status) {
@@ -695,12 +691,10 @@ __global__ void __launch_bounds__(128) preprocess_ewa_kernel(GaussPtrs g, int64_
       }
     }
     if (culled) {
-      ntiles[idx] = 0;
       depth_key[idx] = 0xffffffffu;
       bin[3 * idx + 2] = make_float4(0.f, 0.f, __uint_as_float(pack_i16x2(0, 0)), __uint_as_float(pack_i16x2(-1, -1)));
       continue;
     }
-    ntiles[idx] = (rc.z - rc.x + 1) * (rc.w - rc.y + 1);
     depth_key[idx] = depth_key_of(cam, X);
     float dirn[3], dlen, raw[3];
     view_colour<DEG>(cam, X, sh, dirn, &dlen, raw);
@@ -723,31 +717,31 @@ __global__ void __launch_bounds__(128) preprocess_ewa_kernel(GaussPtrs g, int64_
 }  // namespace
 
 cudaError_t launch_preprocess(const GaussPtrs& g, int64_t n, int sh_degree, const DevCam* cams,
-                              int n_views, int tile_w, int tile_h, RecPtrs rec, int32_t* ntiles,
+                              int n_views, int tile_w, int tile_h, RecPtrs rec,
                               float4* bin, uint32_t* depth_key, int* status, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int bs = kPreThreads;
   const unsigned grid = (unsigned)((n + bs - 1) / bs);
   switch (sh_degree) {
-    case 0: preprocess_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    case 1: preprocess_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    case 2: preprocess_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    default: preprocess_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
+    case 0: preprocess_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    case 1: preprocess_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    case 2: preprocess_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    default: preprocess_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
   }
   return launched();
 }
 
 cudaError_t launch_preprocess_backward(const GaussPtrs& g, int64_t n, int sh_degree,
                                        const DevCam* cams, int n_views, const float* grad_rec,
-                                       const int32_t* ntiles, GaussOut out, cudaStream_t s) {
+                                       GaussOut out, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int bs = kPreThreads;
   const unsigned grid = (unsigned)((n + bs - 1) / bs);
   switch (sh_degree) {
-    case 0: preprocess_bwd_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, ntiles, out); break;
-    case 1: preprocess_bwd_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, ntiles, out); break;
-    case 2: preprocess_bwd_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, ntiles, out); break;
-    default: preprocess_bwd_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, ntiles, out); break;
+    case 0: preprocess_bwd_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, out); break;
+    case 1: preprocess_bwd_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, out); break;
+    case 2: preprocess_bwd_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, out); break;
+    default: preprocess_bwd_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, grad_rec, out); break;
   }
   return launched();
 }
@@ -756,16 +750,16 @@ cudaError_t launch_preprocess_backward(const GaussPtrs& g, int64_t n, int sh_deg
 
 namespace ocgs {
 cudaError_t launch_preprocess_ewa(const GaussPtrs& g, int64_t n, int sh_degree, const DevCam* cams, int n_views,
-                                  int tile_w, int tile_h, RecPtrs rec, int32_t* ntiles, float4* bin,
+                                  int tile_w, int tile_h, RecPtrs rec, float4* bin,
                                   uint32_t* depth_key, int* status, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int bs = kPreThreads;
   const unsigned grid = (unsigned)((n + bs - 1) / bs);
   switch (sh_degree) {
-    case 0: preprocess_ewa_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    case 1: preprocess_ewa_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    case 2: preprocess_ewa_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
-    default: preprocess_ewa_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, ntiles, bin, depth_key, status); break;
+    case 0: preprocess_ewa_kernel<0><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    case 1: preprocess_ewa_kernel<1><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    case 2: preprocess_ewa_kernel<2><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
+    default: preprocess_ewa_kernel<3><<<grid, bs, 0, s>>>(g, n, cams, n_views, tile_w, tile_h, rec, bin, depth_key, status); break;
   }
   return launched();
 }

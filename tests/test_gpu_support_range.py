@@ -66,3 +66,31 @@ def test_results_do_not_depend_on_the_unit_of_length(opts):
             assert torch.equal(base[key], out[key]), (exp, key)
         for key, want in base_g.items():  # atomics: another order of the sums
             assert (grads[key] - want).abs().max() <= 1e-5 * want.abs().max(), (exp, key)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opts", [dict(), dict(pixels_per_thread=1), dict(persistent=True, pixels_per_thread=4)])
+def test_surfels_far_outside_the_image_have_no_gradient(opts):
+    """Finite centres whose projection overflows: they reach no tile, and their gradients are 0."""
+    from paper_2501_08174_gb300 import Rasterizer
+    rng = np.random.default_rng(3)
+    g = synthetic.object_scene(rng, 200, 1)
+    g = {key: np.array(g[key], np.float32) for key in KEYS}
+    g["xyz"][:, 2] += 3.0
+    far = [(1e36, 0.0, 0.5), (3e38, 0.0, 5.0), (0.0, -1e37, 0.5)]
+    g["xyz"][:3], g["quat"][:3], g["scale"][:3] = far, (1.0, 0.0, 0.0, 0.0), 0.05
+    cam = dict(viewmat=np.eye(4), fx=300.0, fy=300.0, cx=80.0, cy=60.0, width=160, height=120, near=0.2)
+    r = Rasterizer(0, **opts)
+    gd = to_device(g, r.device)
+    _, st = r.render(gd, [cam], depth2=True)
+    gen = torch.Generator().manual_seed(4)
+    P = 160 * 120
+    for planes in (("rgb", "alpha"), ("rgb", "alpha", "normal", "depth", "depth2")):
+        d = {p: torch.randn(P, 3, generator=gen) if p in ("rgb", "normal") else torch.randn(P, generator=gen)
+             for p in planes}
+        grads = r.render_backward(st, gd, {p: v.to(r.device) for p, v in d.items()})
+        for key in KEYS:
+            assert torch.isfinite(grads[key]).all(), key
+            assert (grads[key][:3] == 0).all() and float(grads[key].abs().max()) > 0, key
+    st.release()
+    r.close()
