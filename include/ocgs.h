@@ -124,7 +124,13 @@ typedef struct {
  * with a pixel still running at the end of that prefix is then binned with
  * the records behind it and continues from where its pixels stopped.  The
  * tile's list is the one-pass list in two segments, and the backward walks
- * both. */
+ * both.
+ *
+ * pixels_per_thread and batch are upper requests.  A render of few tiles would
+ * leave SMs without warps, so a launch takes 2 pixels per thread for 4 below
+ * 64 warps per SM, and 1 for 2 up to 16 warps per SM (the backward: up to 8,
+ * and never with a persistent queue); a batch that the shape taken is not
+ * built for becomes 32.  ocgs_get_options returns what was set. */
 typedef struct {
   int32_t tile_w;             /* 8, 16 or 32 */
   int32_t tile_h;             /* 8 or 16: 16x16, 16x8, 8x8 or 32x8 */
@@ -481,7 +487,7 @@ int64_t ocgs_kernel_launches(void);
 typedef struct {
   ocgs_options best;     /* chosen options (also set on the context) */
   double best_ms;        /* forward + backward time of the chosen options, ms */
-  int32_t n_tried;       /* candidates timed (0 when taken from the cache) */
+  int32_t n_tried;       /* candidates compared (0 when taken from the cache) */
   int32_t from_cache;    /* 1: read from the cache file */
 } ocgs_tune_result;
 
@@ -496,7 +502,9 @@ typedef struct {
  * persistent choice, front_fraction in {0, 0.05, 0.1, 0.2}; (3) 16 or 64
  * Gaussians per batch where the chosen shape offers them.  Each candidate runs
  * once untimed and twice timed (CUDA events on the context stream); one whose
- * pair count exceeds a render's capacity (OCGS_ERR_CAPACITY) is skipped.
+ * pair count exceeds a render's capacity (OCGS_ERR_CAPACITY) is skipped, and
+ * candidates that come to the same launches on this workload (see
+ * ocgs_options) are timed once, under the larger pixels_per_thread.
  * cache_path (host string or NULL) names a text file of earlier choices keyed
  * by GPU, SM count, SH degree, views and power-of-two buckets of Gaussians and
  * pixels; a hit skips the timing, a miss appends a line.  Synchronises;

@@ -196,7 +196,10 @@ class Rasterizer:
                     front_fraction: float = FRONT_FRACTION, batch: int = 32) -> None:
         """Launch options (see ocgs_options); none changes a result.  ``front_fraction``: share
         of the depth order binned in the first of two passes (persistent renders; 0 = one pass);
-        ``batch``: Gaussians a warp stages in shared memory at a time (16, 32 or 64)."""
+        ``batch``: Gaussians a warp stages in shared memory at a time (16, 32 or 64).
+        ``pixels_per_thread`` and ``batch`` are upper requests: a render of few tiles takes fewer
+        pixels per thread, so that every SM has warps, and then 32 per batch where the smaller
+        shape has no other."""
         o = _lib.Options(int(tile[0]), int(tile[1]), int(bool(persistent)), int(pixels_per_thread),
                          float(front_fraction), int(batch))
         self._call("ocgs_set_options", self._ctx, C.byref(o))
@@ -213,7 +216,8 @@ class Rasterizer:
         self._call("ocgs_set_coverage", self._ctx, int(bool(rect)))
 
     def options(self) -> dict:
-        """The context's launch options, as ``set_options`` takes them."""
+        """The context's launch options, as ``set_options`` took them (a launch of few tiles may
+        use fewer pixels per thread)."""
         return dict(tile=self.tile, persistent=self.persistent, pixels_per_thread=self.pixels_per_thread,
                     front_fraction=self.front_fraction, batch=self.batch)
 

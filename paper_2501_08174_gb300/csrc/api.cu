@@ -10,6 +10,7 @@
 #include "common.cuh"
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1385,7 +1386,29 @@ extern "C" ocgs_status ocgs_autotune(ocgs_ctx* ctx, const ocgs_gaussians* g, con
   };
   double best = 1e30;
   ocgs_options best_opts = saved;
+  // Candidates that come to the same launches (launch_shape: a render of few tiles takes fewer
+  // pixels per thread than asked for) are timed once, under the first name: picked among by
+  // noise, the name kept could be the slower one for a render of more tiles.
+  using Launches = std::array<float, 8>;
+  std::vector<Launches> timed;
+  auto launches = [&](const ocgs_options& o) {
+    const int64_t tiles = plan_cameras(cams, n_views, o.tile_w, o.tile_h, ctx->cover_rect).tiles;
+    auto shape = [&](bool backward) {
+      return launch_shape(o.tile_w, o.tile_h, o.pixels_per_thread, o.batch, tiles, ctx->sm_count, o.persistent != 0,
+                          backward);
+    };
+    const LaunchShape f = shape(false), b = shape(true);
+    return Launches{(float)o.tile_w, (float)o.tile_h, (float)o.persistent,
+                    o.persistent ? o.front_fraction : 0.f,  // the only renders that use it
+                    (float)f.ppt, (float)f.batch, (float)b.ppt, (float)b.batch};
+  };
   auto consider = [&](const ocgs_options& o) {
+    const Launches l = launches(o);
+    if (std::find(timed.begin(), timed.end(), l) != timed.end()) {
+      result->n_tried++;
+      return;
+    }
+    timed.push_back(l);
     const double ms = time_options(o);
     if (ms >= 0.0 && ms < best) {
       best = ms;
