@@ -22,7 +22,7 @@ namespace {
 using namespace raster;
 
 #ifdef OCGS_COUNT
-__device__ unsigned long long g_diag[8];
+__device__ unsigned long long g_diag[2];  // warp-entries, (pixel, entry) blends
 #endif
 
 // Resident warps per SM the compiler is asked to fit (caps registers per thread): 20 leaves
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
       __syncwarp();
       for (int j = cnt - 1; j >= 0; --j) {
 #ifdef OCGS_COUNT
-        if (lane == 0) OCGS_DIAG(2, 1);
+        if (lane == 0) OCGS_DIAG(0, 1);
 #endif
         // Every entry of the walk lies before warp_last, so some lane has jj < its last index, and
         // nearly every one that passed the staging's band test blends a pixel: all are evaluated as
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
           auto sum_add = [&](int q, float2 x) { acc[q] = p == 0 ? x : padd(acc[q], x); };
           const SplatEval2 e = splat_tail2<true>(g0, g2, hd[p], rb, live[2 * p], live[2 * p + 1]);
 #ifdef OCGS_COUNT
-          OCGS_DIAG(6, (e.ok[0] ? 1 : 0) + (e.ok[1] ? 1 : 0));  // (pixel, entry) blends
+          OCGS_DIAG(1, (e.ok[0] ? 1 : 0) + (e.ok[1] ? 1 : 0));
 #endif
           // undo the entry: T before it, its weight, and dL/dalpha
           const float2 om = pfma(e.alpha, bc2(-1.f), bc2(1.f));  // 1 - alpha
@@ -361,9 +361,6 @@ __global__ void __launch_bounds__(kBW * 32, (GEO ? OCGS_BWD_WARPS_GEO : OCGS_BWD
           sum_add(kGcx, gf2);
           sum_fma(kGcy, gf2, hd[p].dy);
         }
-#ifdef OCGS_COUNT
-        if (lane == 0) OCGS_DIAG(3, 1);
-#endif
         // the column offset of this thread's pixels
         const float2 dx = bc2(col.dx);
         acc[kGA00] = pmul(acc[kSumU], dx);
@@ -437,7 +434,7 @@ cudaError_t bwd_dispatch(const RasterBwdArgs& a, cudaStream_t s) {
 extern "C" int ocgs_diag_read_bwd(unsigned long long* out, int reset) {
   cudaMemcpyFromSymbol(out, g_diag, sizeof(g_diag));
   if (reset) {
-    unsigned long long z[8] = {0};
+    unsigned long long z[2] = {0};
     cudaMemcpyToSymbol(g_diag, z, sizeof(z));
   }
   return 0;

@@ -21,7 +21,7 @@ namespace {
 using namespace raster;
 
 #ifdef OCGS_COUNT
-__device__ unsigned long long g_diag[8];
+__device__ unsigned long long g_diag[2];  // warp-entries, (pixel, entry) blends
 #endif
 
 // Resident warps per SM the compiler is asked to fit (caps registers per
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, (!IMG ? OCGS_SWEEP_WARPS : Q
   // The exact band test in the staging: worth its registers where no images are held (sweep of
   // 300k surfels x 100 views 14.3 -> 13.1 ms; with images it spills, 2.72 -> 2.83 ms) and the
   // support is not the near-disc of a projected 3D Gaussian (1.85 -> 2.00 ms).
-    constexpr bool kBandTest = !IMG && !EWA;
+  constexpr bool kBandTest = !IMG && !EWA;
   __shared__ float4 s_g0[kBlockWarps][BATCH], s_g1[kBlockWarps][BATCH], s_g2[kBlockWarps][BATCH],
       s_a0[kBlockWarps][IMG ? BATCH : 1];
   // (n_y, n_z, blend bound, list position + 1); a pass without images keeps the bound in g0.w
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, (!IMG ? OCGS_SWEEP_WARPS : Q
           T[p] = Tn[p];
           if (SCORE) wmax = fmaxf(wmax, fmaxf(w[p].x, w[p].y));
 #ifdef OCGS_COUNT
-          OCGS_DIAG(2, (w[p].x > 0.f ? 1 : 0) + (w[p].y > 0.f ? 1 : 0));  // (pixel, entry) blends
+          OCGS_DIAG(1, (w[p].x > 0.f ? 1 : 0) + (w[p].y > 0.f ? 1 : 0));
 #endif
         }
         if (SCORE) {
@@ -347,7 +347,7 @@ __global__ void sum_u32_kernel(const uint32_t* __restrict__ v, int64_t n, unsign
 extern "C" int ocgs_diag_read(unsigned long long* out, int reset) {
   cudaMemcpyFromSymbol(out, g_diag, sizeof(g_diag));
   if (reset) {
-    unsigned long long z[8] = {0};
+    unsigned long long z[2] = {0};
     cudaMemcpyToSymbol(g_diag, z, sizeof(z));
   }
   return 0;
