@@ -251,9 +251,10 @@ def measured_traffic(kernel: str, workload_args: str):
 
 # ----------------------------------------------------------------------------- roofline model
 def algorithmic(stage: str, N: int, V: int, P: int, K: int, T: int, E: int, tile_passes: int, kept: int,
-                prune_calls: int = 1, M: int = 0) -> dict:
-    """Minimum HBM bytes (and FP32 flops) of each stage for one step (M: records binned in the
-    first of two passes, 0 for one pass)."""
+                prune_calls: int = 1, M: int = 0, PM: int = 0) -> dict:
+    """HBM bytes (and FP32 flops) that each stage's algorithm moves at least for one step (M: records
+    binned in the first of two passes, 0 for one pass; PM: mask pixels).  The depth sort is charged
+    for every record; those without a screen box leave it in the first pass."""
     VN = V * N
     if M:
         # front: counts and duplication (order and 48 B record each); behind the front: the
@@ -265,14 +266,21 @@ def algorithmic(stage: str, N: int, V: int, P: int, K: int, T: int, E: int, tile
         # counts and duplication (order and 48 B record each, 8 B out per pair), tile ranges
         # (4 B per pair, 8 B per tile)
         binning = VN * (52 + 52) + K * 12 + T * 8
-    ssim_px = 24 + 1 + 36 + 36 + 24 + 24  # images + mask, adjoint maps out and back, images again, d_rgb
+    # background loss: opacity and mask, the adjoint (read and written) outside the mask; masked L1:
+    # the mask, and both images and the adjoint inside it
+    loss = P * (4 + 1) + (P - PM) * 8 + P * 1 + PM * (12 + 12 + 24)
+    if prune_calls > 1:
+        # Eq. 3 in full: SSIM (the mask; inside it the images twice, the adjoint maps out and back and
+        # the adjoint), distortion (three planes and their adjoints), normal consistency (opacity; the
+        # covered pixels' stencils and maps are left out)
+        loss += P * 1 + PM * (24 + 36 + 36 + 24 + 24) + P * 36 + P * 4
     b = {
         "preprocess": N * 232 + VN * (72 + 48 + 4),       # record, binning record, depth key
         "depth_sort": VN * (4 + 12 + 3 * 16),             # histograms, first pass (index implied), three more
         "binning": binning,
         "tile_sort": K * (4 + tile_passes * 16),          # histograms, then key and value in and out
         "raster_fwd": VN * 72 + K * 4 + P * 40,
-        "loss": P * (4 + 1 + 8) + P * (12 + 12 + 1 + 24) + (ssim_px * P if prune_calls > 1 else 0),
+        "loss": loss,
         "raster_bwd": VN * (72 + 80) + K * 4 + P * 40,
         "preprocess_bwd": N * 232 * 3 + VN * 84,
         "prune": prune_calls * (N * 24 + kept * 232 * 2),
@@ -585,10 +593,11 @@ def run_ours(a, rank: int, world: int, local: int):
     fp32_peak = n_sm * 128 * 2 * peaks["sm_max_mhz"] * 1e6 / 1e12  # TFLOP/s: SMs x FP32 lanes x FMA x clock
     stages = {}
     step_bytes = 0
+    PM = int(np.count_nonzero(mask_np))
     for name, (tot_ms, cnt) in prof.items():
         if cnt == 0:
             continue  # a stage this workload does not run
-        alg = algorithmic(name, N, len(cams), P, K, T, E, tile_passes, kept, 3 if adam else 1, M)
+        alg = algorithmic(name, N, len(cams), P, K, T, E, tile_passes, kept, 3 if adam else 1, M, PM)
         step_bytes += alg["bytes"]
         per_ms = tot_ms / a.steps
         stages[name] = {"ms": per_ms, "launch_sets": cnt / a.steps,
@@ -597,7 +606,7 @@ def run_ours(a, rank: int, world: int, local: int):
     dom = max(stages, key=lambda k: stages[k]["ms"])
     dstage = stages[dom]
     per_launch_ms = prof[dom][0] / max(prof[dom][1], 1)
-    alg = algorithmic(dom, N, len(cams), P, K, T, E, tile_passes, kept, 3 if adam else 1, M)
+    alg = algorithmic(dom, N, len(cams), P, K, T, E, tile_passes, kept, 3 if adam else 1, M, PM)
     stage_kernel = {"raster_fwd": "raster_fwd_kernel", "raster_bwd": "raster_bwd_kernel",
                     "preprocess": "preprocess_kernel", "preprocess_bwd": "preprocess_bwd_kernel"}
     traffic = None

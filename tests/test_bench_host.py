@@ -46,3 +46,10 @@ def test_backward_byte_model_at_the_measured_workload():
     got = bench.algorithmic("raster_bwd", N, V, P, K, T=62_816, E=2_031_239_432, tile_passes=2, kept=0)
     assert got["bytes"] == N * V * (72 + 80) + 4 * K + 40 * P == 1_972_562_336
     assert got["flops"] == 2_031_239_432 * bench.FLOPS_BWD
+
+
+def test_loss_byte_model_charges_only_what_the_mask_lets_through():
+    kw = dict(N=10, V=1, P=1000, K=0, T=0, E=0, tile_passes=2, kept=0)
+    none, full = (bench.algorithmic("loss", **kw, PM=pm)["bytes"] for pm in (0, 1000))
+    assert none == 1000 * (5 + 8 + 1) and full == 1000 * (5 + 1 + 48)
+    assert bench.algorithmic("loss", **kw, PM=0, prune_calls=3)["bytes"] == none + 1000 * (1 + 36 + 4)
