@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kPruneThreads) prune_count_kernel(const float*
 // What bounds it: HBM (464 bytes per kept Gaussian of degree 3).  One thread per Gaussian
 // copying its 48 coefficients at a stride of 192 bytes took 292 us for 1M Gaussians of which
 // 69 % are kept; finding the positions by a look-back inside this kernel 143 us (its blocks
-// waited for one another more than they copied); this form 72 us with its count kernel.
+// waited for one another more than they copied); this form 62 us with its count kernel.
 template <int DEG>
 __global__ void __launch_bounds__(kPruneThreads) prune_copy_kernel(const float* __restrict__ score, uint32_t n,
                                                                    float tau, const GaussPtrs in, GaussOut out,

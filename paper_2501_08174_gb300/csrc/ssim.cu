@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kViewSumThreads) ssim_final_kernel(const doubl
 // partial[2 b]: sum of squared masked differences, partial[2 b + 1]: mask values
 // Bound by the FP64 rate (about two operations per cycle and SM) where the mask is: blocks of
 // 1024 pixels spread the masked ones over the SMs (blocks of 4096 took 36 us for one view of
-// 717k pixels, these 25), and the loads of a thread's four pixels are in flight together.  The
+// 717k pixels, these 23), and the loads of a thread's four pixels are in flight together.  The
 // pixels are counted as whole numbers: counted in FP64, the smaller blocks' sums took 488 us for
 // 15.4 M pixels against 454 with blocks of 4096; so they take 446.
 constexpr int kPsnrThreads = 256, kPsnrLoads = kPsnrBlockPixels / kPsnrThreads;
