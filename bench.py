@@ -220,7 +220,7 @@ def sources_digest() -> str:
     import hashlib
     pkg = os.path.join(ROOT, "paper_2501_08174_gb300")
     csrc = os.path.join(pkg, "csrc")
-    files = sorted(os.path.join(csrc, f) for f in os.listdir(csrc) if f.endswith((".cu", ".cuh")))
+    files = sorted(os.path.join(csrc, f) for f in os.listdir(csrc) if f.endswith((".cu", ".cuh", ".h")))
     files.append(os.path.join(pkg, "build.py"))
     h = hashlib.sha256()
     for path in files:
@@ -282,7 +282,7 @@ def algorithmic(stage: str, N: int, V: int, P: int, K: int, T: int, E: int, tile
         "raster_fwd": VN * 72 + K * 4 + P * 40,
         "loss": loss,
         "raster_bwd": VN * (72 + 80) + K * 4 + P * 40,
-        "preprocess_bwd": N * 232 * 3 + VN * 84,
+        "preprocess_bwd": N * 232 * 3 + VN * 80,
         "prune": prune_calls * (N * 24 + kept * 232 * 2),
         "adam": N * 232 * 7,  # parameters, gradients, m, v read; parameters, m, v written
     }[stage]

@@ -146,7 +146,7 @@ __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
 
 // gmap [P][6] (or NULL): d(weight term)/d(dx) and d/d(dy) of the pixel's central differences,
 // written for the pixels above a_min only (the gather reads no other).  A pixel per thread and
-// round at six blocks per SM: two per round at four blocks took 113 against 94 us for 10.8 M
+// round at six blocks per SM: two per round at four blocks took 113 against 94 us for 10.5 M
 // pixels of which a quarter are covered.
 __global__ void __launch_bounds__(kRegThreads, 6) normal_consistency_kernel(
     const float* __restrict__ alpha, const float* __restrict__ depth, const float* __restrict__ normal,
